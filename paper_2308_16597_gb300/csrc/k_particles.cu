@@ -67,20 +67,6 @@ bool link_zone_supported(int N, int storage)
     return link_tile_wx(N) <= 64 && link_smem_bytes(N, storage) <= (size_t)200 * 1024;
 }
 
-// Fixed slot (Sec. 3) of the link from zone node (a, b) along e_k, or -1 for
-// a corner line that cannot carry a link.  Axis directions: e1/e3 by row b,
-// e2/e4 by column a (N lines each); diagonals: e5/e7 by a - b + N - 2, e6/e8
-// by a + b - 1 (2N - 3 lines each).  Branch-free, so that the lanes of a warp
-// with different directions do not diverge.
-__device__ __forceinline__ int slot_of(int k, int a, int b, int N)
-{
-    const int M = 2 * N - 3;
-    const bool axis = k <= 4, odd = k & 1;
-    const int line = odd ? (axis ? b : a - b + N - 2) : (axis ? a : a + b - 1);
-    const int slot = axis ? (k - 1) * N + line : 4 * N + (k - 5) * M + line;
-    return (axis || (line >= 0 && line < M)) ? slot : -1;
-}
-
 // Counts (and overflow flag) of the screening grid of the next step, which
 // the next step's link kernel fills: block p of the np blocks of a
 // per-particle kernel clears its share.  The grid was last read by the

@@ -762,6 +762,20 @@ __host__ __device__ inline void slot_dir_line(int s, int N, int &k, int &line)
     }
 }
 
+// Fixed slot (Sec. 3) of the link from zone node (a, b) along e_k, or -1 for
+// a corner line that cannot carry a link.  Axis directions: e1/e3 by row b,
+// e2/e4 by column a (N lines each); diagonals: e5/e7 by a - b + N - 2, e6/e8
+// by a + b - 1 (2N - 3 lines each).  Branch-free, so that the lanes of a warp
+// with different directions do not diverge.
+__device__ __forceinline__ int slot_of(int k, int a, int b, int N)
+{
+    const int M = 2 * N - 3;
+    const bool axis = k <= 4, odd = k & 1;
+    const int line = odd ? (axis ? b : a - b + N - 2) : (axis ? a : a + b - 1);
+    const int slot = axis ? (k - 1) * N + line : 4 * N + (k - 5) * M + line;
+    return (axis || (line >= 0 && line < M)) ? slot : -1;
+}
+
 // ---------------------------------------------------------------------------
 // Batched instances.  Every step kernel is a device body that takes the
 // position of its block within one instance's launch (Blk): the
