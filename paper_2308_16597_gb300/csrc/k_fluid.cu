@@ -55,14 +55,6 @@ __device__ float pull_general(const Dev &D, const T *__restrict__ A, int x, int 
     return -v + 2.f * w5(d) * D.Twall[side];
 }
 
-// Values pulled into a node on the general path; for a newborn node the
-// refilling of Sec. 2.5 instead: e_c maximises n . e_c (FP64, ties to the
-// lowest index, n the outward normal at the new position), f is extrapolated from the nodes
-// x + m e_c (m = 1, 2, 3) that are fluid at both times (quadratic, linear,
-// copy, or f_eq(1, u_w)), its momentum is set to rho u_w, and
-// g = g_eq(T_w, u_w).
-// Returns 0 for a general pull, else 1 + the refill class (1 quadratic,
-// 2 linear, 3 copy, 4 equilibrium).
 // The pull of plane p at the side node (x, y), x = 0 or nx - 1, of a row
 // between the first and the last, for a plane whose source lies across the
 // side wall or the periodic seam (pull_general restricted to that case).
@@ -82,24 +74,25 @@ __device__ __forceinline__ float side_pull(const Dev &D, const T *__restrict__ A
     return -v + 2.f * w5(d) * D.Twall[d == 1 ? 0 : 1];
 }
 
+// The refilling of Sec. 2.5 at a newborn node that particle pid uncovered
+// this step: e_c maximises n . e_c (FP64, ties to the lowest index, n the
+// outward normal at the new position), f is extrapolated from the nodes
+// x + m e_c (m = 1, 2, 3) that are fluid at both times (quadratic, linear,
+// copy, or f_eq(1, u_w)), its momentum is set to rho u_w, and
+// g = g_eq(T_w, u_w).
+// Returns the refill class (1 quadratic, 2 linear, 3 copy, 4 equilibrium).
 template <typename T>
-__device__ __forceinline__ int slow_node(const Dev &D, const T *__restrict__ A,
-                                      const int *__restrict__ own_cur, int x, int y, uint8_t fl,
-                                      float *out)
+__device__ __forceinline__ int refill_node(const Dev &D, const T *__restrict__ A, int parity, int pid, int x, int y,
+                                           float *out)
 {
-    if (fl != kNewborn) {
-#pragma unroll
-        for (int p = 0; p < kPop; ++p) out[p] = pull_general(D, A, x, y, p);
-        return 0;
-    }
-    const int pid = own_cur[(long long)y * D.nx + x];
-    const double xc = D.cur.x[pid], yc = D.cur.y[pid];
+    const PartSoA &P = D.part[parity ^ 1]; // the state after the update
+    const double xc = P.x[pid], yc = P.y[pid];
     const double dx = __dsub_rn((double)x, xc), dy = __dsub_rn((double)y, yc);
     // outward normal: (dx, dy) for a disk, the gradient of the ellipse form
     // for an ellipse
     double nx = dx, ny = dy;
-    const double pr = D.cur.r[pid], pb = D.cur.b[pid];
-    if (is_ellipse(pr, pb)) ell_normal(ell_frame(xc, yc, D.cur.th[pid], pr, pb), dx, dy, nx, ny);
+    const double pr = P.r[pid], pb = P.b[pid];
+    if (is_ellipse(pr, pb)) ell_normal(ell_frame(xc, yc, P.th[pid], pr, pb), dx, dy, nx, ny);
     int c = 1;
     double best = __dadd_rn(__dmul_rn((double)ex(1), nx), __dmul_rn((double)ey(1), ny));
     for (int k = 2; k < kQ9; ++k) {
@@ -109,15 +102,16 @@ __device__ __forceinline__ int slow_node(const Dev &D, const T *__restrict__ A,
             c = k;
         }
     }
-    const float uwx = (float)(D.cur.ux[pid] - D.cur.om[pid] * dy);
-    const float uwy = (float)(D.cur.uy[pid] + D.cur.om[pid] * dx);
-    int nvalid = 0;
+    const float uwx = (float)(P.ux[pid] - P.om[pid] * dy);
+    const float uwy = (float)(P.uy[pid] + P.om[pid] * dx);
+    // the three stencil nodes, looked up at once: fluid at both times
+    bool calm[3];
+#pragma unroll
     for (int m = 1; m <= 3; ++m) {
-        int a = x + m * ex(c), b = y + m * ey(c);
-        if (a < 0 || a >= D.nx || b < 0 || b >= D.ny) break;
-        if (D.flags[(long long)b * D.pitch + a] != kFluid) break;
-        nvalid = m;
+        const int a = x + m * ex(c), b = y + m * ey(c);
+        calm[m - 1] = a >= 0 && a < D.nx && b >= 0 && b < D.ny && !solid_at(D, a, b, 0) && !solid_at(D, a, b, 1);
     }
+    const int nvalid = !calm[0] ? 0 : !calm[1] ? 1 : !calm[2] ? 2 : 3;
     float fh[kQ9];
     if (nvalid == 0) {
         const float uu = uwx * uwx + uwy * uwy;
@@ -148,7 +142,7 @@ __device__ __forceinline__ int slow_node(const Dev &D, const T *__restrict__ A,
     }
     const float djx = (rho * uwx - jx) * (1.f / 6.f), djy = (rho * uwy - jy) * (1.f / 6.f);
     for (int i = 0; i < kQ9; ++i) out[i] = fh[i] + ex(i) * djx + ey(i) * djy;
-    const float Tw = (float)D.cur.T[pid];
+    const float Tw = (float)P.T[pid];
     for (int i = 0; i < kQ5; ++i) out[kQ9 + i] = w5(i) * Tw * (1.f + 5.f * (ex(i) * uwx + ey(i) * uwy));
     return 4 - nvalid;
 }
@@ -454,14 +448,13 @@ __device__ __forceinline__ void prefetch_block(const Dev &D, const T *__restrict
 
 template <typename T, int V, bool kSharedFlags>
 __device__ __forceinline__ void sc_tail(const Dev &D, const T *__restrict__ Ain, T *__restrict__ Aout,
-                                        float (&c)[V][kPop], int x0, int y, const uint8_t *sflags);
+                                        float (&c)[V][kPop], int x0, int y, int parity, const uint2 *sbits);
 
 // pf_x < 0: no look-ahead prefetch here (the caller issues its own).
 template <typename T, int V, int mode = kSCAll>
 __device__ __forceinline__ void sc_body(const Dev &D, const T *__restrict__ Ain, T *__restrict__ Aout, int pf_x,
-                                        int pf_y, const Blk blk)
+                                        int pf_y, int parity, const Blk blk)
 {
-    using E = Elem<T>;
     using VW = typename Vec<T, V>::W;
     const int lane = threadIdx.x & 31;
     if (pf_x >= 0) prefetch_block<T, V, mode>(D, Ain, pf_x, pf_y);
@@ -485,8 +478,9 @@ __device__ __forceinline__ void sc_body(const Dev &D, const T *__restrict__ Ain,
     // values they bring feed only the planes of the side nodes x = 0 and
     // x = nx - 1 that pull across a wall or seam, which the general pull
     // replaces below, and the padding past nx, which is zeroed.
-    const bool interior = y >= 1 && y + 1 < D.ny;
-    if (interior) {
+    // (The fluid nodes of the first and last rows are k_boundary's: nothing
+    // is pulled for them.)
+    if (y >= 1 && y + 1 < D.ny) {
         const T *b0 = Ain + (long long)y * D.pitch + x0;
 #pragma unroll
         for (int p = 0; p < kPop; ++p) {
@@ -519,53 +513,23 @@ __device__ __forceinline__ void sc_body(const Dev &D, const T *__restrict__ Ain,
         }
     } else {
 #pragma unroll
-        for (int p = 0; p < kPop; ++p) {
-            const int d = pdir(p);
-            const int dx = ex(d), dy = ey(d);
-            int ys = y - dy;
-            bool rowok = ys >= 0 && ys < D.ny;
-            if (!rowok && D.per_y) {
-                ys = ys < 0 ? ys + D.ny : ys - D.ny;
-                rowok = true;
-            }
-            const T *src = Ain + (long long)p * D.ps + (long long)(rowok ? ys : 0) * D.pitch;
-            float v[V];
-            if (act && rowok) VecIo<T, V>::unpack(__ldg(reinterpret_cast<const VW *>(src + x0)), v);
-            else {
+        for (int p = 0; p < kPop; ++p)
 #pragma unroll
-                for (int k = 0; k < V; ++k) v[k] = 0.f;
-            }
-            if (dx == 0) {
-#pragma unroll
-                for (int k = 0; k < V; ++k) c[k][p] = v[k];
-            } else if (dx == 1) { // pull from x - 1
-                float l = __shfl_up_sync(kFull, v[V - 1], 1);
-                if (lane == 0) l = (act && rowok && x0 >= 1) ? Io<T>::ld(__ldg(src + x0 - 1)) : 0.f;
-                c[0][p] = l;
-#pragma unroll
-                for (int k = 1; k < V; ++k) c[k][p] = v[k - 1];
-            } else { // pull from x + 1
-                float r = __shfl_down_sync(kFull, v[0], 1);
-                if (lane == 31) r = (act && rowok && x0 + V < D.pitch) ? Io<T>::ld(__ldg(src + x0 + V)) : 0.f;
-#pragma unroll
-                for (int k = 0; k + 1 < V; ++k) c[k][p] = v[k + 1];
-                c[V - 1][p] = r;
-            }
-        }
+            for (int k = 0; k < V; ++k) c[k][p] = 0.f;
     }
     if (!act) return;
-    sc_tail<T, V, false>(D, Ain, Aout, c, x0, y, nullptr);
+    sc_tail<T, V, false>(D, Ain, Aout, c, x0, y, parity, nullptr);
 }
 
 // The part of a stream-collide update after the interior pulls, for the V
 // nodes x0 .. x0 + V - 1 of row y whose pulled values c holds: the side
 // nodes' wall or seam planes, the collision, the stores and the numeric
-// check.  The nodes' flags are read from sflags (shared memory) or, without
-// kSharedFlags, from the flag map where they are used (an address computed
-// earlier and held cost the one-block-per-tile kernels registers).
+// check.  The word pair of the nodes' bits is *sbits (shared memory) or,
+// without kSharedFlags, read from the node bits where it is used (an address
+// computed earlier and held cost the one-block-per-tile kernels registers).
 template <typename T, int V, bool kSharedFlags>
 __device__ __forceinline__ void sc_tail(const Dev &D, const T *__restrict__ Ain, T *__restrict__ Aout,
-                                        float (&c)[V][kPop], int x0, int y, const uint8_t *sflags)
+                                        float (&c)[V][kPop], int x0, int y, int parity, const uint2 *sbits)
 {
     using VW = typename Vec<T, V>::W;
     constexpr float kIo = Io<T>::kScaled ? kHalfScale : 1.f; // the side pulls' values in the kernel's scale
@@ -594,21 +558,22 @@ __device__ __forceinline__ void sc_tail(const Dev &D, const T *__restrict__ Ain,
             }
     }
     bool ok = true, gen[V], anygen = false;
+    // solid now; newborn: solid when the step began only
+    const uint2 bits = kSharedFlags
+                           ? *sbits
+                           : __ldg(reinterpret_cast<const uint2 *>(D.bits) + (long long)y * D.bpitch + (x0 >> 5));
+    const unsigned now = (parity ? bits.x : bits.y) >> (x0 & 31), before = (parity ? bits.y : bits.x) >> (x0 & 31);
+    const bool edge = y == 0 || y == D.ny - 1;
     if constexpr (V == 2) {
         // both nodes collided at once on paired FP32 instructions; solid
         // nodes (and the padding past nx) are zeroed after
         bool fluid[2];
-        // both nodes' flags in one 2-byte load (x0 is even)
-        const uint8_t *flp = kSharedFlags ? sflags : D.flags + (long long)y * D.pitch + x0;
-        const unsigned short fl2 = *reinterpret_cast<const unsigned short *>(flp);
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-            const int x = x0 + k;
-            const unsigned fl = (fl2 >> (8 * k)) & 0xffu;
-            fluid[k] = x < D.nx && fl != kSolid;
+            fluid[k] = x0 + k < D.nx && !((now >> k) & 1u);
             // newborn nodes and the first and last rows belong to k_boundary,
             // which writes them
-            gen[k] = fluid[k] && (fl == kNewborn || y == 0 || y == D.ny - 1);
+            gen[k] = fluid[k] && (((before >> k) & 1u) || edge);
             anygen |= gen[k];
         }
         float2 cc[kPop];
@@ -632,13 +597,11 @@ __device__ __forceinline__ void sc_tail(const Dev &D, const T *__restrict__ Ain,
     } else {
 #pragma unroll
         for (int k = 0; k < V; ++k) {
-            const int x = x0 + k;
-            const uint8_t fl = kSharedFlags ? sflags[k] : D.flags[(long long)y * D.pitch + x];
             gen[k] = false;
-            if (x < D.nx && fl != kSolid) {
+            if (x0 + k < D.nx && !((now >> k) & 1u)) {
                 // newborn nodes and the first and last rows belong to
                 // k_boundary, which writes them
-                gen[k] = fl == kNewborn || y == 0 || y == D.ny - 1;
+                gen[k] = ((before >> k) & 1u) || edge;
                 if (!gen[k]) ok &= collide(D, c[k]);
             } else {
 #pragma unroll
@@ -673,45 +636,47 @@ __device__ __forceinline__ void sc_tail(const Dev &D, const T *__restrict__ Ain,
 
 // General path, beside the stream-collide kernel (it reads only the previous
 // state and writes only nodes that kernel leaves alone): the fluid nodes of
-// the first and last rows (walls, periodic seams) and the newborn nodes
-// listed by k_flags, each pulled (or refilled, Sec. 2.5) by slow_node and
-// collided.  (The side columns' fluid nodes between those rows are the
-// stream-collide kernel's.)
+// the first and last rows (walls, periodic seams; kFrame) and the newborn
+// nodes (kRefill), which are the nodes on the particle update's list that no
+// particle holds now, taken up by the particle that owned them; each pulled
+// or refilled (Sec. 2.5) and collided.  (The side columns' fluid nodes between
+// those rows are the stream-collide kernel's.)
 // A fixed grid strides over the 2 nx nodes of the two rows and then the
-// list, whose length the device holds; a listed node on the frame (~n) is
-// taken from the list unless it lies in those rows.
-template <typename T>
+// list, whose length the device holds.
+enum { kFrame = 1, kRefill = 2 };
+template <typename T, int kWhat>
 __device__ __forceinline__ void boundary_body(const Dev &D, const T *__restrict__ Ain, T *__restrict__ Aout,
                                               const int *__restrict__ own_cur, int parity, const Blk blk)
 {
     using E = Elem<T>;
     const int nx = D.nx, ny = D.ny;
-    const int nframe = 2 * nx;
-    const int nlist = min((int)D.status->nb, D.newborn_cap);
+    const int nframe = (kWhat & kFrame) ? 2 * nx : 0;
+    const int nlist = (kWhat & kRefill) ? min((int)D.status->nb, D.left_cap) : 0;
     unsigned n4[4] = {0u, 0u, 0u, 0u};
     bool ok = true;
     for (int idx = blk.x * (int)blockDim.x + (int)threadIdx.x; idx < nframe + nlist; idx += blk.gx * (int)blockDim.x) {
         int x, y;
-        if (idx < nx) { x = idx; y = 0; }
-        else if (idx < nframe) { x = idx - nx; y = ny - 1; }
-        else {
-            const int v = D.newborn[idx - nframe], n = v < 0 ? ~v : v;
-            y = n / nx;
-            x = n - y * nx;
-            if (v < 0 && (y == 0 || y == ny - 1)) continue; // visited above
-        }
-        const long long o = (long long)y * D.pitch + x;
-        const uint8_t fl = D.flags[o];
-        if (fl == kSolid) continue;
         float c[kPop];
-        const int r = slow_node(D, Ain, own_cur, x, y, fl, c);
-        if (r) {
+        if (idx < nframe) {
+            x = idx < nx ? idx : idx - nx;
+            y = idx < nx ? 0 : ny - 1;
+            if (solid_at(D, x, y, parity ^ 1) || solid_at(D, x, y, parity)) continue; // solid, or newborn: listed
+#pragma unroll
+            for (int p = 0; p < kPop; ++p) c[p] = pull_general(D, Ain, x, y, p);
+        } else {
+            const int2 e = D.left[idx - nframe];
+            y = e.x / nx;
+            x = e.x - y * nx;
+            if (solid_at(D, x, y, parity ^ 1)) continue; // another particle's
+            if (D.crowd[parity][e.y] && own_cur[e.x] != e.y) continue; // its owner lists it too
+            const int r = refill_node(D, Ain, parity, e.y, x, y, c);
             n4[0] += 1u;
             n4[1] += r == 2;
             n4[2] += r == 3;
             n4[3] += r == 4;
         }
         ok &= collide(D, c);
+        const long long o = (long long)y * D.pitch + x;
 #pragma unroll
         for (int p = 0; p < kPop; ++p)
             if (in_bounds(D, (long long)p * D.ps + o, D.a_elems)) Aout[(long long)p * D.ps + o] = E::st(c[p]);
@@ -727,12 +692,13 @@ __device__ __forceinline__ void boundary_body(const Dev &D, const T *__restrict_
 // the ninth block's warps outweigh the spills).
 template <typename T, int V, int mode>
 __global__ void __launch_bounds__(kSCThreads, V == 1 ? 10 : 9)
-    k_stream_collide(const Dev D, const T *__restrict__ Ain, T *__restrict__ Aout, int ahead_y, int ahead_x)
+    k_stream_collide(const Dev D, const T *__restrict__ Ain, T *__restrict__ Aout, int ahead_y, int ahead_x,
+                     int parity)
 {
     const Blk blk = this_blk();
     int bx, by;
     ahead_block(blk, ahead_y, ahead_x, bx, by);
-    sc_body<T, V, mode>(D, Ain, Aout, bx, by, blk);
+    sc_body<T, V, mode>(D, Ain, Aout, bx, by, parity, blk);
 }
 
 
@@ -756,7 +722,7 @@ __global__ void __launch_bounds__(kSCThreads, V == 1 ? 10 : 9)
 //
 // Shared memory per stage: 14 plane segments of 128 V + 2 H elements
 // (H = 16 bytes of elements; node x_s + i at element H + i), then the
-// tile's 128 V flag bytes.  The reads past a row's ends (x = -H .. -1 for a
+// tile's node bits (8 bytes per 32 nodes).  The reads past a row's ends (x = -H .. -1 for a
 // plane pulling from x - 1, which has index p >= 1, so the previous plane or
 // row lies there; x = pitch .. pitch + H - 1 for one pulling from x + 1, the
 // next row, plane or the buffer's tail pad) feed only the side nodes' wall or
@@ -782,9 +748,10 @@ struct StGeo {
     static constexpr int W = kSCThreads * V;                     // nodes of a tile
     static constexpr int H = 16 / (int)sizeof(T);                // halo elements on a pulled side
     static constexpr int SEG_B = (W + 2 * H) * (int)sizeof(T);   // bytes of a plane segment
-    static constexpr int FLAGS_OFF = kPop * SEG_B;               // the tile's flags
+    static constexpr int BITS_OFF = kPop * SEG_B;                // the tile's node bits, both parities
+    static constexpr int BITS_B = W / 32 * 8;
     // with kInst (a batch): the tile's instance record (state, buffers)
-    static constexpr int INST_OFF = (FLAGS_OFF + W + 15) / 16 * 16;
+    static constexpr int INST_OFF = BITS_OFF + (BITS_B + 15) / 16 * 16;
     static constexpr int INST_B = kInst ? (int)sizeof(InstArgs) : 0;
     static constexpr int STAGE_B = (INST_OFF + INST_B + 127) / 128 * 128;
     static constexpr int SMEM_B = kStStages * STAGE_B + 128;     // + barriers and tile slots
@@ -865,9 +832,9 @@ struct StTail {
 static_assert(kStStages * 8 <= 32 && 32 + (kStStages + 2) * 16 + 8 <= 128, "staged stream-collide: tail layout");
 
 // The copy a thread issues for every tile, fixed for the launch: copy c
-// (planes 0..13, then the flags, then in a batch the tile's instance record)
+// (planes 0..13, then the node bits, then in a batch the tile's instance record)
 // belongs to lane c % 4 of warp c / 4, so no warp carries the copies alone.  Three registers: the copy (-1 none, kPop
-// the flags), its shared-memory destination in stage 0, and for a plane its
+// the node bits), its shared-memory destination in stage 0, and for a plane its
 // row shift e_y + 1 (bits 0-1) and whether it pulls from x - 1 (bit 2) or
 // x + 1 (bit 3), i.e. takes H elements more on that side.
 struct StLane {
@@ -882,7 +849,7 @@ __device__ __forceinline__ StLane st_lane(unsigned char *sm)
     const int lane = threadIdx.x & 31, c = (threadIdx.x >> 5) * 4 + lane;
     if (kInst && lane < 4 && c == kPop + 1) return StLane{c, smem_addr(sm + G::INST_OFF), 0}; // the record
     if (lane >= 4 || c > kPop) return StLane{-1, 0u, 0};
-    if (c == kPop) return StLane{c, smem_addr(sm + G::FLAGS_OFF), 0};
+    if (c == kPop) return StLane{c, smem_addr(sm + G::BITS_OFF), 0};
     const int d = pdir(c), dx = ex(d);
     return StLane{c, smem_addr(sm + c * G::SEG_B) + (unsigned)((dx == 1 ? 0 : G::H) * (int)sizeof(T)),
                   (ey(d) + 1) | (dx == 1 ? 4 : 0) | (dx == -1 ? 8 : 0)};
@@ -908,7 +875,7 @@ __device__ __forceinline__ void st_issue(const Dev &D, const T *__restrict__ Ain
         t.stile[s] = tile;
         if (y < 0) mbar_arrive(b);
         else
-            mbar_arrive_tx(b, (unsigned)(n * (kPop * (int)sizeof(T) + 1) + shifted_planes() * 16 + G::INST_B +
+            mbar_arrive_tx(b, (unsigned)(n * kPop * (int)sizeof(T) + G::BITS_B + shifted_planes() * 16 + G::INST_B +
                                          D.sc_extra_tx));
     }
     if (y < 0 || L.c < 0) return;
@@ -917,8 +884,8 @@ __device__ __forceinline__ void st_issue(const Dev &D, const T *__restrict__ Ain
         bulk_to_smem(dst, rec, (unsigned)G::INST_B, b);
         return;
     }
-    if (L.c == kPop) { // the tile's flags
-        bulk_to_smem(dst, D.flags + (long long)y * D.pitch + xs, (unsigned)n, b);
+    if (L.c == kPop) { // the tile's node bits (rows are padded to whole tiles' words)
+        bulk_to_smem(dst, D.bits + bit_word(D, xs, y, 0), (unsigned)G::BITS_B, b);
         return;
     }
     int ys = y - ((L.meta & 3) - 1);
@@ -1047,7 +1014,8 @@ __device__ __forceinline__ void staged_body(const P &pol)
                     ain = pol.ain(tile.x);
                     aout = pol.aout(tile.x);
                 }
-                sc_tail<T, V, true>(D, ain, aout, c, x0, y, sb + G::FLAGS_OFF + tid * V);
+                sc_tail<T, V, true>(D, ain, aout, c, x0, y, kInst ? pol.parity ^ rec->poff : pol.parity,
+                                    reinterpret_cast<const uint2 *>(sb + G::BITS_OFF) + (tid * V >> 5));
             }
         }
         if (tid == 0) t.snext[(k + 1) & 1] = claimed;
@@ -1083,7 +1051,7 @@ struct StSingle {
     const Dev &D;
     const T *Ain;
     T *Aout;
-    int ntx, nitems;
+    int ntx, nitems, parity;
     __device__ int4 decode(int it) const
     {
         if (it >= nitems) return make_int4(0, -1, 0, 0);
@@ -1150,9 +1118,10 @@ struct StBatch {
 
 template <typename T, int V>
 __global__ void __launch_bounds__(kSCThreads, LBM_ST_MINB)
-    k_stream_collide_staged(const Dev D, const T *__restrict__ Ain, T *__restrict__ Aout, int ntx, int nitems)
+    k_stream_collide_staged(const Dev D, const T *__restrict__ Ain, T *__restrict__ Aout, int ntx, int nitems,
+                            int parity)
 {
-    staged_body<T, V>(StSingle<T, V>{D, Ain, Aout, ntx, nitems});
+    staged_body<T, V>(StSingle<T, V>{D, Ain, Aout, ntx, nitems, parity});
 }
 
 template <typename T, int V>
@@ -1169,7 +1138,7 @@ __global__ void __launch_bounds__(128)
     k_boundary(const Dev D, const T *__restrict__ Ain, T *__restrict__ Aout, const int *__restrict__ own_cur,
                int parity)
 {
-    boundary_body<T>(D, Ain, Aout, own_cur, parity, this_blk());
+    boundary_body<T, kFrame | kRefill>(D, Ain, Aout, own_cur, parity, this_blk());
 }
 
 // Batched forms: one grid over all instances.  Stream-collide blocks are
@@ -1201,10 +1170,10 @@ __global__ void __launch_bounds__(kSCThreads, V == 1 ? 10 : 9) // as k_stream_co
     sc_tile(sc + i, (int)blockIdx.x, bx, by);
     const Blk blk{bx, by, 0, 0}; // the grid extents are not used by the body
     const int par = parity ^ a.poff;
-    sc_body<T, V>(a.D, static_cast<const T *>(a.A[par]), static_cast<T *>(a.A[par ^ 1]), -1, 0, blk);
+    sc_body<T, V>(a.D, static_cast<const T *>(a.A[par]), static_cast<T *>(a.A[par ^ 1]), -1, 0, par, blk);
 }
 
-template <typename T>
+template <typename T, int kWhat>
 __global__ void __launch_bounds__(128)
     k_boundary_batch(const InstArgs *__restrict__ I, const int *__restrict__ start, int n, int parity)
 {
@@ -1215,15 +1184,15 @@ __global__ void __launch_bounds__(128)
     const int s0 = __ldg(start + i);
     const Blk blk{(int)blockIdx.x - s0, 0, __ldg(start + i + 1) - s0, 1};
     const int par = parity ^ a.poff;
-    boundary_body<T>(sD, static_cast<const T *>(a.A[par]), static_cast<T *>(a.A[par ^ 1]), a.own[par], par,
-                     blk);
+    boundary_body<T, kWhat>(sD, static_cast<const T *>(a.A[par]), static_cast<T *>(a.A[par ^ 1]), a.own[par], par,
+                            blk);
 }
 
 // Collision without streaming, for the initial state and for distributions
 // supplied by the caller (mode 1 reads pre-collision values from Ain).
 template <typename T>
 __global__ void k_init_collide(const Dev D, const T *__restrict__ Ain, T *__restrict__ Aout, float T_init,
-                               int mode)
+                               int mode, int parity)
 {
     using E = Elem<T>;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1231,7 +1200,7 @@ __global__ void k_init_collide(const Dev D, const T *__restrict__ Ain, T *__rest
     if (x >= D.pitch || y >= D.ny) return;
     const long long n = (long long)y * D.pitch + x;
     float c[kPop];
-    const bool live = x < D.nx && D.flags[n] != kSolid;
+    const bool live = x < D.nx && !solid_at(D, x, y, parity);
     for (int p = 0; p < kPop; ++p) {
         if (mode == 1) c[p] = E::ld(Ain[(long long)p * D.ps + n]);
         else c[p] = p < kQ9 ? 0.f : w5(p - kQ9) * T_init;
@@ -1249,7 +1218,7 @@ __global__ void k_init_collide(const Dev D, const T *__restrict__ Ain, T *__rest
 // pre-collision (sum e f + F/2)/rho of Sec. 2.1.
 template <typename S>
 __global__ void k_fields(const Dev D, const S *__restrict__ A, int row0, float *rho_o, float *ux_o,
-                         float *uy_o, float *T_o)
+                         float *uy_o, float *T_o, int parity)
 {
     using E = Elem<S>;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1257,7 +1226,7 @@ __global__ void k_fields(const Dev D, const S *__restrict__ A, int row0, float *
     if (x >= D.nx || y >= D.ny) return;
     const long long n = (long long)y * D.pitch + x;
     const long long o = (long long)blockIdx.y * D.nx + x;
-    if (D.flags[n] == kSolid) {
+    if (solid_at(D, x, y, parity)) {
         const float nan = __int_as_float(0x7fc00000);
         rho_o[o] = nan; ux_o[o] = nan; uy_o[o] = nan; T_o[o] = nan;
         return;
@@ -1281,7 +1250,7 @@ __global__ void k_fields(const Dev D, const S *__restrict__ A, int row0, float *
 namespace {
 
 template <typename T, int V, int mode>
-cudaError_t stream_collide_m(const Dev &D, const void *Ain, void *Aout, cudaStream_t s)
+cudaError_t stream_collide_m(const Dev &D, const void *Ain, void *Aout, int parity, cudaStream_t s)
 {
     static int resident = 0;
     if (!resident) {
@@ -1298,7 +1267,7 @@ cudaError_t stream_collide_m(const Dev &D, const void *Ain, void *Aout, cudaStre
     dim3 block(bx, by);
     dim3 grid((tx + bx - 1) / bx, (D.ny + by - 1) / by);
     k_stream_collide<T, V, mode><<<grid, block, 0, s>>>(D, static_cast<const T *>(Ain), static_cast<T *>(Aout),
-                                                        resident / (int)grid.x, resident % (int)grid.x);
+                                                        resident / (int)grid.x, resident % (int)grid.x, parity);
     return cudaGetLastError();
 }
 
@@ -1319,7 +1288,7 @@ int staged_resident(K kernel, int smem)
 // claim tiles from the work counter, so blocks that start late, behind the
 // boundary kernel's, take fewer).
 template <typename T, int V>
-cudaError_t stream_collide_staged(const Dev &D, const void *Ain, void *Aout, cudaStream_t s)
+cudaError_t stream_collide_staged(const Dev &D, const void *Ain, void *Aout, int parity, cudaStream_t s)
 {
     using G = StGeo<T, V>;
     static int resident = 0;
@@ -1328,7 +1297,7 @@ cudaError_t stream_collide_staged(const Dev &D, const void *Ain, void *Aout, cud
     const int ntx = (D.pitch + G::W - 1) / G::W;
     const int nitems = ntx * D.ny;
     k_stream_collide_staged<T, V><<<min(resident, nitems), kSCThreads, G::SMEM_B, s>>>(
-        D, static_cast<const T *>(Ain), static_cast<T *>(Aout), ntx, nitems);
+        D, static_cast<const T *>(Ain), static_cast<T *>(Aout), ntx, nitems, parity);
     return cudaGetLastError();
 }
 
@@ -1346,14 +1315,15 @@ cudaError_t stream_collide_staged_batch(const InstArgs *I, const ScInst *sc, con
 }
 
 template <typename T, int V>
-cudaError_t stream_collide_t(const Dev &D, const void *Ain, void *Aout, int mode, cudaStream_t s)
+cudaError_t stream_collide_t(const Dev &D, const void *Ain, void *Aout, int mode, int parity, cudaStream_t s)
 {
     switch (mode) {
-    case kSCFar: return stream_collide_m<T, V, kSCFar>(D, Ain, Aout, s);
-    case kSCNear: return stream_collide_m<T, V, kSCNear>(D, Ain, Aout, s);
+    case kSCFar: return stream_collide_m<T, V, kSCFar>(D, Ain, Aout, parity, s);
+    case kSCNear: return stream_collide_m<T, V, kSCNear>(D, Ain, Aout, parity, s);
     default:
-        return D.sc_staged ? stream_collide_staged<T, V>(D, Ain, Aout, s)
-                           : stream_collide_m<T, V, kSCAll>(D, Ain, Aout, s);
+        if constexpr (V == 2) // FP32 is never staged (see fill_dev)
+            if (D.sc_staged) return stream_collide_staged<T, V>(D, Ain, Aout, parity, s);
+        return stream_collide_m<T, V, kSCAll>(D, Ain, Aout, parity, s);
     }
 }
 
@@ -1372,22 +1342,23 @@ cudaError_t boundary_t(const Dev &D, const void *Ain, void *Aout, const int *own
 }
 
 template <typename T>
-cudaError_t init_collide_t(const Dev &D, const void *Ain, void *Aout, float T_init, int mode, cudaStream_t s)
+cudaError_t init_collide_t(const Dev &D, const void *Ain, void *Aout, float T_init, int mode, int parity,
+                           cudaStream_t s)
 {
     dim3 block(128);
     dim3 grid((D.pitch + 127) / 128, D.ny);
     k_init_collide<T><<<grid, block, 0, s>>>(D, static_cast<const T *>(Ain), static_cast<T *>(Aout), T_init,
-                                             mode);
+                                             mode, parity);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t fields_t(const Dev &D, const void *A, int row0, int rows, float *rho, float *ux, float *uy,
-                     float *Tf, cudaStream_t s)
+                     float *Tf, int parity, cudaStream_t s)
 {
     dim3 block(128);
     dim3 grid((D.nx + 127) / 128, rows);
-    k_fields<T><<<grid, block, 0, s>>>(D, static_cast<const T *>(A), row0, rho, ux, uy, Tf);
+    k_fields<T><<<grid, block, 0, s>>>(D, static_cast<const T *>(A), row0, rho, ux, uy, Tf, parity);
     return cudaGetLastError();
 }
 
@@ -1399,12 +1370,12 @@ int near_tiles_per_row(int storage, int pitch)
     return (pitch + span - 1) / span;
 }
 
-cudaError_t launch_stream_collide(const Dev &D, const void *Ain, void *Aout, int mode, cudaStream_t s)
+cudaError_t launch_stream_collide(const Dev &D, const void *Ain, void *Aout, int mode, int parity, cudaStream_t s)
 {
     switch (D.storage) {
-    case LBM_STORE_FP32: return stream_collide_t<float, 1>(D, Ain, Aout, mode, s);
-    case LBM_STORE_BF16: return stream_collide_t<__nv_bfloat16, 2>(D, Ain, Aout, mode, s);
-    case LBM_STORE_FP16: return stream_collide_t<__half, 2>(D, Ain, Aout, mode, s);
+    case LBM_STORE_FP32: return stream_collide_t<float, 1>(D, Ain, Aout, mode, parity, s);
+    case LBM_STORE_BF16: return stream_collide_t<__nv_bfloat16, 2>(D, Ain, Aout, mode, parity, s);
+    case LBM_STORE_FP16: return stream_collide_t<__half, 2>(D, Ain, Aout, mode, parity, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -1449,14 +1420,22 @@ cudaError_t launch_stream_collide_batch(const InstArgs *I, const ScInst *sc, con
     return cudaGetLastError();
 }
 
+template <typename T>
+static void boundary_batch_t(const InstArgs *I, const int *start, int n, int total, int parity, bool refill,
+                             cudaStream_t s)
+{
+    if (refill) k_boundary_batch<T, kRefill><<<total, 128, 0, s>>>(I, start, n, parity);
+    else k_boundary_batch<T, kFrame><<<total, 128, 0, s>>>(I, start, n, parity);
+}
+
 cudaError_t launch_boundary_batch(const InstArgs *I, const int *start, int n, int total, int storage, int parity,
-                                  cudaStream_t s)
+                                  bool refill, cudaStream_t s)
 {
     if (total <= 0) return cudaSuccess;
     switch (storage) {
-    case LBM_STORE_FP32: k_boundary_batch<float><<<total, 128, 0, s>>>(I, start, n, parity); break;
-    case LBM_STORE_BF16: k_boundary_batch<__nv_bfloat16><<<total, 128, 0, s>>>(I, start, n, parity); break;
-    case LBM_STORE_FP16: k_boundary_batch<__half><<<total, 128, 0, s>>>(I, start, n, parity); break;
+    case LBM_STORE_FP32: boundary_batch_t<float>(I, start, n, total, parity, refill, s); break;
+    case LBM_STORE_BF16: boundary_batch_t<__nv_bfloat16>(I, start, n, total, parity, refill, s); break;
+    case LBM_STORE_FP16: boundary_batch_t<__half>(I, start, n, total, parity, refill, s); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -1493,24 +1472,24 @@ int stream_collide_batch_resident(int storage, dim3 block)
     return max(1, sms * per_sm);
 }
 
-cudaError_t launch_init_collide(const Dev &D, const void *Ain, void *Aout, float T_init, int mode,
+cudaError_t launch_init_collide(const Dev &D, const void *Ain, void *Aout, float T_init, int mode, int parity,
                                 cudaStream_t s)
 {
     switch (D.storage) {
-    case LBM_STORE_FP32: return init_collide_t<float>(D, Ain, Aout, T_init, mode, s);
-    case LBM_STORE_BF16: return init_collide_t<__nv_bfloat16>(D, Ain, Aout, T_init, mode, s);
-    case LBM_STORE_FP16: return init_collide_t<__half>(D, Ain, Aout, T_init, mode, s);
+    case LBM_STORE_FP32: return init_collide_t<float>(D, Ain, Aout, T_init, mode, parity, s);
+    case LBM_STORE_BF16: return init_collide_t<__nv_bfloat16>(D, Ain, Aout, T_init, mode, parity, s);
+    case LBM_STORE_FP16: return init_collide_t<__half>(D, Ain, Aout, T_init, mode, parity, s);
     default: return cudaErrorInvalidValue;
     }
 }
 
 cudaError_t launch_fields(const Dev &D, const void *A, int row0, int rows, float *rho, float *ux, float *uy,
-                          float *T, cudaStream_t s)
+                          float *T, int parity, cudaStream_t s)
 {
     switch (D.storage) {
-    case LBM_STORE_FP32: return fields_t<float>(D, A, row0, rows, rho, ux, uy, T, s);
-    case LBM_STORE_BF16: return fields_t<__nv_bfloat16>(D, A, row0, rows, rho, ux, uy, T, s);
-    case LBM_STORE_FP16: return fields_t<__half>(D, A, row0, rows, rho, ux, uy, T, s);
+    case LBM_STORE_FP32: return fields_t<float>(D, A, row0, rows, rho, ux, uy, T, parity, s);
+    case LBM_STORE_BF16: return fields_t<__nv_bfloat16>(D, A, row0, rows, rho, ux, uy, T, parity, s);
+    case LBM_STORE_FP16: return fields_t<__half>(D, A, row0, rows, rho, ux, uy, T, parity, s);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -8,14 +8,14 @@
 //   k_particles  pair screening through the cell grid, Newton-Euler update
 //                with gravity, buoyancy and spring repulsion (Sec. 2.2,
 //                Sec. 2.4) in FP64, and the raster of the new positions into
-//                the next owner map (cleared over the old zones by k_links);
-//   k_flags      node flags at the new positions and the newborn list;
+//                the next node bits (cleared over the old zones by k_links),
+//                with the list of the nodes the particles left;
 // plus the initialisation kernels (k_raster, k_geom_init), the
 // direct-addressing comparison (k_direct_prep, k_links_direct), the near-tile
 // bitmap of the opt-in split stream-collide (k_near_mask) and the batched
 // forms of the step kernels.
 #include <climits>
-#include <mutex>
+#include <type_traits>
 
 #include "lbm_internal.cuh"
 
@@ -23,7 +23,6 @@ namespace lbm {
 
 namespace {
 
-constexpr int kLinkThreads = 128;
 constexpr int kBoxThreads = 128;
 constexpr int kPartThreads = 256;
 constexpr double kPi = 3.14159265358979323846;
@@ -49,23 +48,22 @@ __device__ __forceinline__ T warp_sum(T v)
 // are 64-bit words).
 __host__ __device__ inline int link_tile_wy(int N) { return N + 4; }
 __host__ __device__ inline int link_tile_wx(int N) { return N + 4; }
-__host__ __device__ inline int link_occ_words(int N) { return (12 * N - 12 + 31) / 32; }
 
-// Shared memory: the fluid and owner row masks [wy] (u64 each), slot
-// occupancy words and their prefix [words], and per slot the link node and
-// the compacted slot list.
-size_t link_smem_bytes(int N, int storage)
+// Shared memory of a CTA: its record, the fluid and owner row masks [wy] (u64
+// each) and the list of links (at most one per slot).
+struct alignas(16) LinkTeam {
+    EllFrame ell;  // an ellipse's FP64 frame
+    int n;         // links found
+    unsigned over; // a line with two links
+};
+size_t link_smem_bytes(int N)
 {
-    (void)storage;
-    const size_t cap = (size_t)12 * N - 12;
-    return (size_t)2 * link_tile_wy(N) * sizeof(unsigned long long) +
-           (size_t)2 * link_occ_words(N) * sizeof(unsigned) + cap * 2 * sizeof(int);
+    const size_t b = sizeof(LinkTeam) + (size_t)2 * link_tile_wy(N) * sizeof(unsigned long long) +
+                     (size_t)(12 * N - 12) * sizeof(int);
+    return (b + 15) / 16 * 16;
 }
 
-bool link_zone_supported(int N, int storage)
-{
-    return link_tile_wx(N) <= 64 && link_smem_bytes(N, storage) <= (size_t)200 * 1024;
-}
+bool link_zone_supported(int N) { return link_tile_wx(N) <= 64; }
 
 // Counts (and overflow flag) of the screening grid of the next step, which
 // the next step's link kernel fills: block p of the np blocks of a
@@ -93,337 +91,362 @@ __device__ __forceinline__ void cell_insert(const Dev &D, int *grid, int b, floa
     } else grid[ncell] = 1;
 }
 
-// The last step's newborn nodes (fluid now, listed by the flags kernel of
-// that step) go back to plain fluid: the flags kernel of this step rewrites
-// only the nodes whose class changes at the particles' edges.  Entries of
-// block p of np blocks of nthreads threads.
-__device__ __forceinline__ void revert_newborn(const Dev &D, int p, int tid, int nthreads)
+// Zone of particle p one step back: its node bits, and for a crowded particle
+// its owner nodes, cleared in the maps the raster fills next (they hold the
+// positions of that time; every zone is cleared, so the words a zone shares
+// with another's need no care).  One warp per call, lanes on zone rows.
+__device__ __forceinline__ void clear_zone_bits(const Dev &D, int parity, int p, int lane)
 {
-    const int nb = min((int)D.status->nb, D.newborn_cap);
-    for (int e = p * nthreads + tid; e < nb; e += D.np * nthreads) {
-        const int v = D.newborn[e], n = v < 0 ? ~v : v;
-        const int y = n / D.nx, x = n - y * D.nx;
-        if (in_bounds(D, (long long)y * D.pitch + x, (long long)D.ny * D.pitch)) D.flags[(long long)y * D.pitch + x] = kFluid;
+    const GeomRec *G = D.geo[parity ^ 1] + p;
+    const int X0 = G->X0, Y0 = G->Y0, N = G->N;
+    const int w0 = max(X0, 0) >> 5, w1 = min(X0 + N - 1, D.nx - 1) >> 5;
+    for (int r = lane; r < N; r += 32) {
+        const int j = Y0 + r;
+        if (j < 0 || j >= D.ny) continue;
+        unsigned *row = D.bits + (long long)j * D.bpitch * 2 + (parity ^ 1);
+        for (int w = w0; w <= w1; ++w) row[2 * w] = 0u;
+    }
+}
+// (Whole block of nthreads threads.)
+__device__ __forceinline__ void clear_zone_owner(const Dev &D, int *__restrict__ own_nxt, int parity, int p, int tid,
+                                                 int nthreads)
+{
+    if (!D.crowd[parity ^ 1][p]) return;
+    const GeomRec *G = D.geo[parity ^ 1] + p;
+    const int X0 = G->X0, Y0 = G->Y0, N = G->N;
+    for (int r = tid >> 5; r < N; r += nthreads / 32) {
+        const int j = Y0 + r;
+        if (j < 0 || j >= D.ny) continue;
+        for (int c = tid & 31; c < N; c += 32) {
+            const int i = X0 + c;
+            if (i >= 0 && i < D.nx) own_nxt[(long long)j * D.nx + i] = -1;
+        }
     }
 }
 
-// One CTA per particle.  Phases:
+// Row masks of the link kernel's window, 64 columns from XA: the fluid nodes
+// of row j (none outside the domain), from the node bits; wide: more than 32
+// columns matter.
+__device__ __forceinline__ unsigned long long fluid_row(const Dev &D, int parity, int XA, int j, bool wide)
+{
+    if (j < 0 || j >= D.ny) return 0ull;
+    const unsigned *row = D.bits + (long long)j * D.bpitch * 2 + parity;
+    const int w0 = XA >> 5, sh = XA & 31; // XA may be negative: words before the row are not fluid
+    auto word = [&](int w) -> unsigned { return w >= 0 && w < D.bpitch ? ~row[2 * w] : 0u; };
+    const unsigned a = word(w0), b = word(w0 + 1), c = wide ? word(w0 + 2) : 0u;
+    unsigned long long m = ((unsigned long long)__funnelshift_r(b, c, sh) << 32) | __funnelshift_r(a, b, sh);
+    const int in = D.nx - XA; // columns inside the domain
+    if (in < 64) m &= in > 0 ? (1ull << in) - 1ull : 0ull;
+    return m;
+}
+
+// 32 bits of m from bit s on (zeros outside its 64 bits).
+__device__ __forceinline__ unsigned extract32(unsigned long long m, int s)
+{
+    if (s >= 0) return s < 64 ? (unsigned)(m >> s) : 0u;
+    return s > -32 ? (unsigned)m << -s : 0u;
+}
+
+// Transpose of the warp's 32 x 32 bits: lane l holds row l before, column l
+// after (bit r of it from row r).
+__device__ __forceinline__ unsigned transpose32(unsigned x, int lane)
+{
+    unsigned keep = 0x0000ffffu; // the bits of a lane without bit s that stay
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        const unsigned y = __shfl_xor_sync(0xffffffffu, x, s);
+        x = (lane & s) ? (x & ~keep) | ((y >> s) & keep) : (x & keep) | ((y << s) & ~keep);
+        keep ^= keep << (s >> 1);
+    }
+    return x;
+}
+
+// One CTA of kTeam warps per particle.  Phases:
 //  0. clear this CTA's share of the screening grid the next step's link
-//     kernel fills, and the particle's zone one step back in the owner map
-//     that the raster fills next; return the last step's newborn nodes to
-//     fluid;
-//  1. the warps read the owner map over the particle's window (zone plus
-//     the two-node margin of the bounce-back stencil) and record per row a
-//     fluid mask and an owned-by-this-particle mask (one ballot per 32
-//     nodes); thread 0 publishes the particle's screening record (and the
-//     FP64 frame of an ellipse); a warp prefetches into L2 the owner rows of
-//     the particle
+//     kernel fills, and the particle's zone one step back in the node bits
+//     (and owner map) that the raster fills next;
+//  1. row masks of the particle's window (zone plus the two-node margin of
+//     the bounce-back stencil), a lane per row: fluid nodes from the node
+//     bits, this particle's nodes from the row runs of its raster (a crowded
+//     particle's from the owner map, since it may share nodes with another);
+//     thread 0 publishes the particle's screening record (and the FP64 frame
+//     of an ellipse); a warp prefetches into L2 the bit rows of the particle
 //     `ahead` places later in launch order (one residency wave ahead).
 //     (Prefetching the populations of that particle's window as well, by
 //     tensor or row prefetches, or of this particle's links as they are
-//     found, measured slower: the kernel is bound by its latency chains and
-//     issue, not by DRAM, and the extra traffic and instructions cost more
-//     than the hits gained);
-//  2. thread (k, b) intersects the fluid mask of zone row b with the owner
-//     mask of row b + e_k,y shifted by e_k,x: each set bit is a link, which
-//     claims its fixed slot of the index array (direction k, line through
-//     the zone; Sec. 3) in an occupancy bitmap;
-//  3. the occupied slots are compacted in slot order (popcount prefix), so
-//     thread i takes the i-th link and the work is balanced;
-//  4. each link: wall fraction q, curved bounce-back of f and g (Sec. 2.3)
-//     from the populations read at x_f, x_f - e_k and x_f - 2 e_k,
-//     written into the solid node x_f + e_k (direction kbar) of A in HBM,
-//     where the next pull stream picks it up (one link per (solid node, kbar),
-//     and every read is of a fluid node, so the writes never race the reads),
-//     and the momentum-exchange bracket of Eq. force / Eq. torque, summed
-//     in exact fixed point per thread, per warp and over the warps (so the
-//     forces are bit-reproducible);
-//  5. the particle enters the screening grid of this step's update.
-template <typename T>
+//     found, measured slower);
+//  2. links.  Along any line of the zone (Sec. 3: the rows, the columns and
+//     the two families of diagonals) the particle's nodes are one run, and
+//     the only nodes that can be linked to it there are the two next to the
+//     run's ends, one per direction: a warp per family brings the row masks
+//     to a lane per line (shears and 32 x 32 bit transposes), takes the
+//     run's ends, looks the two nodes up in the fluid masks and appends the
+//     links to a list; a line without a link empties its slot of the index
+//     array;
+//  3. each link: its slot of the index array, wall fraction q, curved
+//     bounce-back of f and g (Sec. 2.3) from the populations read at x_f,
+//     x_f - e_k and x_f - 2 e_k, written into the solid node x_f + e_k
+//     (direction kbar) of A in HBM, where the next pull stream picks it up
+//     (one link per (solid node, kbar), and every read is of a fluid node, so
+//     the writes never race the reads), and the momentum-exchange bracket of
+//     Eq. force / Eq. torque, summed in exact fixed point per thread, per
+//     warp and over the warps (so the forces are bit-reproducible, whatever
+//     the list's order);
+//  4. the particle enters the screening grid of this step's update.
+template <typename T, int kTeam>
 __device__ __forceinline__ void links_body(const Dev &D, T *A, const int *__restrict__ own,
                                            int *__restrict__ own_nxt, int parity, const int p, const int pa)
 {
+    extern __shared__ __align__(16) unsigned char sm[];
     using E = Elem<T>;
-    extern __shared__ __align__(16) unsigned char lsm[];
-    __shared__ int s_nvalid;
-    __shared__ unsigned s_over;
-    __shared__ EllFrame s_ell;
+    constexpr unsigned F = 0xffffffffu;
+    constexpr int kThreads = 32 * kTeam;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const GeomRec G = D.geo_cur[p];
-    const int N = G.N, cap = 12 * N - 12;
-    const int X0 = G.X0, Y0 = G.Y0;
+    const GeomRec *Gp = D.geo[parity] + p;
+    const int X0 = Gp->X0, Y0 = Gp->Y0, N = Gp->N;
     const int base = D.slot_base[p];
+    const int crowded = D.crowd[parity][p];
 
-    const int Nm = D.zone_max;
-    const int wy = link_tile_wy(Nm), wx = link_tile_wx(Nm);
-    const int XA = X0 - 2, YA = Y0 - 2, off = 2;
-    unsigned long long *Fm = reinterpret_cast<unsigned long long *>(lsm); // [wy]
-    unsigned long long *Om = Fm + wy;                                       // [wy]
-    const int nw = link_occ_words(Nm), capm = 12 * Nm - 12;
-    unsigned *occ = reinterpret_cast<unsigned *>(Om + wy); // [nw]
-    unsigned *pre = occ + nw;                               // [nw]
-    int *info = reinterpret_cast<int *>(pre + nw);          // [cap] k | a << 4 | b << 12 of the slot's link
-    int *list = info + capm;                                // [cap] valid slots in order
+    const int wy = link_tile_wy(N), wx = link_tile_wx(N);
+    const int XA = X0 - 2, YA = Y0 - 2;
+    LinkTeam &S = *reinterpret_cast<LinkTeam *>(sm);
+    unsigned long long *Fm = reinterpret_cast<unsigned long long *>(sm + sizeof(LinkTeam)); // [wy]
+    unsigned long long *Om = Fm + link_tile_wy(D.zone_max);                                  // [wy]
+    int *list = reinterpret_cast<int *>(Om + link_tile_wy(D.zone_max)); // k | a << 4 | b << 10 | slot << 16
 
-    // ---- 0. the screening grid the particle update fills next: this CTA's
-    // slice of its counts; the owner map the raster fills next (positions
-    // n + 1) still holds positions n - 1: clear this particle's zone of that
-    // time
-    clear_cells_slice(D, parity, p, tid, kLinkThreads);
-    revert_newborn(D, p, tid, kLinkThreads);
-    {
-        const GeomRec Gp = D.geo_prev[p];
-        for (int r = warp; r < Gp.N; r += kLinkThreads / 32) {
-            const int j = Gp.Y0 + r;
-            if (j < 0 || j >= D.ny) continue;
-            for (int c = lane; c < Gp.N; c += 32) {
-                const int i = Gp.X0 + c;
-                if (i >= 0 && i < D.nx) own_nxt[(long long)j * D.nx + i] = -1;
-            }
-        }
-    }
-
-    // ---- 1. owner masks (all warps) and the look-ahead prefetch
+    // ---- 0., 1.
+    clear_cells_slice(D, parity, p, tid, kThreads);
+    if (p == 0 && tid == 0) D.status->nb = 0u; // the step's list of nodes left
     if (tid == 0) {
-        s_over = 0u;
-        const DiskDF d0 = geom_df(G);
-        D.pos4[p] = make_float4(d0.xh, d0.yh, d0.xl, d0.yl);
-        D.prc[p] = make_float2(G.r, G.C);
-        if (G.r < 0.f) s_ell = ell_frame(D.cur.x[p], D.cur.y[p], D.cur.th[p], D.cur.r[p], D.cur.b[p]);
+        S.n = 0;
+        S.over = 0u;
     }
-    {
-        // owner rows in chunks of four per warp, all four loads issued before
-        // the first ballot, so a chunk costs one memory latency
-        constexpr int kW = kLinkThreads / 32;
-        for (int r0 = 0; r0 < wy; r0 += 4 * kW) {
-            int vlo[4], vhi[4];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const int r = r0 + warp + t * kW, j = YA + r, i = XA + lane;
-                vlo[t] = (r < wy && inside(D, i, j)) ? own[(long long)j * D.nx + i] : -2;
-                vhi[t] = (wx > 32 && r < wy && inside(D, i + 32, j)) ? own[(long long)j * D.nx + i + 32] : -2;
-            }
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                if (r0 + t * kW >= wy) break; // no warp has a row left
-                const int r = r0 + warp + t * kW;
-                const unsigned lo_f = __ballot_sync(0xffffffffu, vlo[t] == -1);
-                const unsigned lo_o = __ballot_sync(0xffffffffu, vlo[t] == p);
-                unsigned hi_f = 0u, hi_o = 0u;
-                if (wx > 32) {
-                    hi_f = __ballot_sync(0xffffffffu, vhi[t] == -1);
-                    hi_o = __ballot_sync(0xffffffffu, vhi[t] == p);
+    if (warp == 0)
+        for (int r = lane; r < wy; r += 32) Fm[r] = fluid_row(D, parity, XA, YA + r, wx > 32);
+    if (!crowded) {
+        if (warp == 1)
+            for (int r = lane; r < wy; r += 32) {
+                unsigned long long m = 0ull;
+                if (r >= 2 && r < N + 2) {
+                    const int2 run = D.runs[parity][(long long)p * D.zone_max + r - 2];
+                    if (run.x <= run.y) m = ((2ull << (run.y - XA)) - 1ull) & (~0ull << (run.x - XA));
                 }
-                if (lane == 0 && r < wy) {
-                    Fm[r] = ((unsigned long long)hi_f << 32) | lo_f;
-                    Om[r] = ((unsigned long long)hi_o << 32) | lo_o;
-                }
+                Om[r] = m;
             }
+    } else {
+        for (int r = warp; r < wy; r += kTeam) {
+            const int j = YA + r, i = XA + lane;
+            const int lo = inside(D, i, j) ? own[(long long)j * D.nx + i] : -1;
+            const int hi = wx > 32 && inside(D, i + 32, j) ? own[(long long)j * D.nx + i + 32] : -1;
+            const unsigned ol = __ballot_sync(F, lo == p), oh = __ballot_sync(F, hi == p);
+            if (lane == 0) Om[r] = ((unsigned long long)oh << 32) | ol;
         }
     }
-    // L2 prefetch of the owner rows of particle pa, the one a residency wave
+    if (warp == 2) clear_zone_bits(D, parity, p, lane);
+    clear_zone_owner(D, own_nxt, parity, p, tid, kThreads);
+    if (tid == kThreads - 1) {
+        D.pos4[p] = make_float4(Gp->xh, Gp->yh, Gp->xl, Gp->yl);
+        D.prc[p] = make_float2(Gp->r, Gp->C);
+        if (Gp->r < 0.f) {
+            const PartSoA &P = D.part[parity];
+            S.ell = ell_frame(P.x[p], P.y[p], P.th[p], P.r[p], P.b[p]);
+        }
+    }
+    // L2 prefetch of the bit rows of particle pa, the one a residency wave
     // later in launch order (none: pa < 0)
-    if (warp == 1 && pa >= 0) {
-        const GeomRec Ga = D.geo_cur[pa];
-        const int xa = Ga.X0 - 2, ya = Ga.Y0 - 2;
-        for (int r = lane; r < 2 * wy; r += 32) {
-            const int j = ya + (r >> 1), i = min(max(xa + (r & 1) * (wx - 1), 0), D.nx - 1);
+    if (warp == 3 && pa >= 0) {
+        const GeomRec *Ga = D.geo[parity] + pa;
+        const int xa = Ga->X0 - 2, ya = Ga->Y0 - 2;
+        for (int r = lane; r < link_tile_wy(D.zone_max); r += 32) {
+            const int j = ya + r;
             if (j >= 0 && j < D.ny)
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(own + (long long)j * D.nx + i) : "memory");
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(D.bits + bit_word(D, max(xa, 0), j, 0)) : "memory");
         }
     }
-    for (int w = tid; w < nw; w += kLinkThreads) occ[w] = 0u;
     __syncthreads();
 
-    // ---- 2. link detection: item (k, b), one mask intersection per row;
-    // items run direction-major.  A warp's links are spread evenly over its
-    // lanes (a prefix sum of the items' bit counts; lane j takes the j-th
-    // link of the warp), since a few rows (the flat top and bottom of a disk
-    // for e2 / e4) hold many links and most hold one
+    // ---- 2. links: the rows, the columns, the diagonals of constant a - b,
+    // those of constant a + b; lane l of a round takes line i
     {
-        const unsigned F = 0xffffffffu;
-        const unsigned long long Z = ((1ull << N) - 1ull) << off;
-        for (int e0 = warp * 32; e0 < 8 * N; e0 += kLinkThreads) {
-            const int e = e0 + lane;
+        const int f = warp & 3, M = 2 * N - 3, lines = f < 2 ? N : M;
+        const int kf = f < 2 ? f + 1 : f + 3;                   // direction into the run's start: 1, 2, 5, 6
+        const int sf = f == 0 ? 0 : f == 1 ? N : f == 2 ? 4 * N : 4 * N + M; // its slots; those of the end follow
+        const int sb = sf + (f < 2 ? 2 * N : 2 * M);
+        for (int i0 = 32 * (warp >> 2); i0 < lines; i0 += 8 * kTeam) {
+            const int i = i0 + lane;
+            // the particle's nodes on line i: bit t, the row b of the node
+            // (its column a on a row)
             unsigned long long m = 0ull;
-            int k = 1, b = 0;
-            if (e < 8 * N) {
-                k = 1 + e / N;
-                b = e - (k - 1) * N;
-                const int kx = ex(k), ky = ey(k);
-                const unsigned long long o = Om[b + 2 + ky];
-                m = Fm[b + 2] & (kx > 0 ? o >> 1 : kx < 0 ? o << 1 : o) & Z;
-            }
-            const int cnt = __popcll(m);
-            int inc = cnt;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(F, inc, o);
-                if (lane >= o) inc += t;
-            }
-            const int total = __shfl_sync(F, inc, 31), excl = inc - cnt;
-            for (int j0 = 0; j0 < total; j0 += 32) {
-                const int j = j0 + lane;
-                // the item holding link j: the last lane whose first link is
-                // at or before j
-                int l = 0;
-#pragma unroll
-                for (int step = 16; step > 0; step >>= 1) {
-                    const int ec = __shfl_sync(F, excl, l + step);
-                    if (ec <= j) l += step;
+            if (f == 0) {
+                if (i < N) m = Om[i + 2] >> 2;
+            } else {
+                for (int h = 0; h < N; h += 32) {
+                    const int b = h + lane;
+                    const unsigned long long R = b < N ? Om[b + 2] >> 2 : 0ull;
+                    const unsigned x = extract32(R, f == 1 ? i0 : f == 2 ? i0 + b - (N - 2) : i0 + 1 - b);
+                    m |= (unsigned long long)transpose32(x, lane) << h;
                 }
-                unsigned long long ml = __shfl_sync(F, m, l);
-                const int kl = __shfl_sync(F, k, l), bl = __shfl_sync(F, b, l), el = __shfl_sync(F, excl, l);
-                if (j >= total) continue;
-                for (int t = j - el; t > 0; --t) ml &= ml - 1ull; // drop the lower links of the item
-                const int a = (__ffsll((long long)ml) - 1) - off;
-                const int sl = slot_of(kl, a, bl, N);
-                if (sl < 0) {
-                    s_over = 1u;
-                    continue;
+            }
+            // zone column a of line i at t (the row of f > 0)
+            auto col = [&](int t) { return f == 0 ? t : f == 1 ? i : f == 2 ? t + i - (N - 2) : i + 1 - t; };
+            auto fluid = [&](int t) -> bool {
+                const int a = col(t), b = f == 0 ? i : t;
+                return a >= 0 && a < N && b >= 0 && b < N && ((Fm[b + 2] >> (a + 2)) & 1ull);
+            };
+            bool lo = false, hi = false;
+            int t0 = 0, t1 = 0;
+            if (i < lines && m) {
+                t0 = __ffsll((long long)m) - 2;  // before the run's start
+                t1 = 64 - __clzll((long long)m); // after its end
+                lo = fluid(t0);
+                hi = fluid(t1);
+                // two runs (only in an owner map that no raster made): a link
+                // inside would be the line's second
+                unsigned long long st = m & ~(m << 1), en = m & ~(m >> 1);
+                st &= st - 1ull;
+                en &= ~(1ull << (t1 - 1));
+                while (st) {
+                    if (fluid(__ffsll((long long)st) - 2) || fluid(__ffsll((long long)en))) S.over = 1u;
+                    st &= st - 1ull;
+                    en &= en - 1ull;
                 }
-                const unsigned bit = 1u << (sl & 31);
-                if (atomicOr(&occ[sl >> 5], bit) & bit) s_over = 1u;
-                else info[sl] = kl | (a << 4) | (bl << 12);
+            }
+            const unsigned wl = __ballot_sync(F, lo), wh = __ballot_sync(F, hi);
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&S.n, __popc(wl) + __popc(wh));
+            at = __shfl_sync(F, at, 0);
+            const unsigned below = (1u << lane) - 1u;
+            if (i < lines) {
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const bool on = e ? hi : lo;
+                    const int t = e ? t1 : t0, sl = (e ? sb : sf) + i, k = kf + 2 * e;
+                    if (on) {
+                        const int pos = at + (e ? __popc(wl) + __popc(wh & below) : __popc(wl & below));
+                        list[pos] = k | (col(t) << 4) | ((f == 0 ? i : t) << 10) | (sl << 16);
+                    } else if (in_bounds(D, (long long)base + sl, D.nslots)) {
+                        D.slot_node[base + sl] = -1;
+                        D.slot_q[base + sl] = 0.f;
+                    }
+                }
             }
         }
     }
     __syncthreads();
+    const int nvalid = S.n;
 
-    // ---- 3. compaction of the occupied slots in slot order
-    const int nwp = (cap + 31) >> 5;
-    if (warp == 0) {
-        const unsigned c = lane < nwp ? (unsigned)__popc(occ[lane]) : 0u;
-        unsigned inc = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned t = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += t;
-        }
-        if (lane < nwp) pre[lane] = inc - c;
-        if (lane == 31) s_nvalid = (int)inc;
-    }
-    __syncthreads();
-    const int nvalid = s_nvalid;
-    for (int sl = tid; sl < cap; sl += kLinkThreads) {
-        const unsigned w = occ[sl >> 5], bit = 1u << (sl & 31);
-        if (w & bit) list[pre[sl >> 5] + __popc(w & (bit - 1u))] = sl;
-        else if (in_bounds(D, (long long)base + sl, D.nslots)) {
-            D.slot_node[base + sl] = -1;
-            D.slot_q[base + sl] = 0.f;
-        }
-    }
-    __syncthreads();
-
-    // ---- 4. bounce-back and momentum exchange, thread i on the i-th link
+    // ---- 3. bounce-back and momentum exchange, thread i on the links i,
+    // i + kThreads, ...
+    const GeomRec G = *Gp;
     const DiskDF dk = geom_df(G);
     const bool ell = G.r < 0.f; // an ellipse: q in FP64
-    const float Ux = G.ux, Uy = G.uy, Om_ = G.om, wT = G.wT;
-    // populations of fluid nodes: no CTA writes them during this kernel
-    const T *Ar = A;
-    auto tv = [&](int plane, int i, int j) -> float {
-        const long long e = (long long)plane * D.ps + (long long)j * D.pitch + i;
-        return in_bounds(D, e, D.a_elems) ? E::ld(__ldg(Ar + e)) : 0.f;
-    };
     auto fluid = [&](int i, int j) -> bool { return (Fm[j - YA] >> (i - XA)) & 1ull; };
-    // one round per kLinkThreads links: every warp sums its round at once
-    // (exact integer sums), lane 0 adds it to the warp's total; no
-    // accumulator stays live across rounds
-    __shared__ LinkSums s_ws[kLinkThreads / 32];
-    __shared__ int s_wc[kLinkThreads / 32][3];
-    const int rounds = (nvalid + kLinkThreads - 1) / kLinkThreads;
-    for (int it = 0; it < rounds; ++it) {
-        const int li = it * kLinkThreads + tid;
-        LinkAcc acc;
-        if (li < nvalid) {
-            const int sl = list[li];
-            const int inf = info[sl], k = inf & 15;
-            const int kx = ex(k), ky = ey(k);
-            const int fi = X0 + ((inf >> 4) & 255), fj = Y0 + (inf >> 12);
-            float dxf, dyf;
-            const float q = ell ? link_q_ellipse(fi, fj, k, s_ell, dxf, dyf) : link_q_df(fi, fj, k, dk, dxf, dyf);
-            if (in_bounds(D, (long long)base + sl, D.nslots)) {
-                D.slot_node[base + sl] = fj * D.nx + fi;
-                D.slot_q[base + sl] = q;
-            }
-
-            // curved bounce-back in deviation form: every rule is an affine
-            // combination of populations of equal weight, so it holds for
-            // f~ = f - w unchanged
-            const int kb = opp(k);
-            const int i1 = fi - kx, j1 = fj - ky, i2 = fi - 2 * kx, j2 = fj - 2 * ky;
-            const bool have1 = fluid(i1, j1);
-            const bool have2 = fluid(i2, j2);
-            const int ii1 = have1 ? i1 : fi, jj1 = have1 ? j1 : fj;
-            const int ii2 = have2 ? i2 : fi, jj2 = have2 ? j2 : fj;
-            const float fk0 = tv(k, fi, fj), fk1 = tv(k, ii1, jj1), fk2 = tv(k, ii2, jj2);
-            const float fb0 = tv(kb, fi, fj), fb1 = tv(kb, ii1, jj1);
-            const float rx = dxf + q * kx, ry = dyf + q * ky;
-            const float uwx = Ux - Om_ * ry, uwy = Uy + Om_ * rx;
-            const float wall = 6.f * w9(k) * -(kx * uwx + ky * uwy); // 2 w rho0 e_kbar.u_w / c_s^2
-            int lvl;
-            const float fnew = bouzidi32(q, fk0, fk1, fk2, fb0, fb1, have1, have2, wall, lvl);
-            const long long ns = (long long)(fj + ky) * D.pitch + (fi + kx);
-            if (in_bounds(D, kb * D.ps + ns, D.a_elems)) A[kb * D.ps + ns] = E::st(fnew);
-            if (k <= 4) {
-                const float gnew = thermal32(q, tv(kQ9 + k, fi, fj), tv(kQ9 + k, ii1, jj1),
-                                             tv(kQ9 + kb, fi, fj), have1, wT);
-                if (in_bounds(D, (kQ9 + kb) * D.ps + ns, D.a_elems)) A[(kQ9 + kb) * D.ps + ns] = E::st(gnew);
-            }
-            // momentum exchange: with f = w + f~ the bracket of Eq. force is
-            // 2 w_k e_k + [f~_k^+ (e_k - u_w) - f~_kbar (e_kbar - u_w)]; the
-            // constant part and its torque 2 w_k ((i - x_c) e_k,y - (j - y_c) e_k,x)
-            // (q drops out) are kept as exact integer sums, assembled in FP64 by
-            // the particle update
-            const float bx = fk0 * (kx - uwx) - fnew * (-kx - uwx);
-            const float by = fk0 * (ky - uwy) - fnew * (-ky - uwy);
-            acc.add(bx, by, rx * by - ry * bx, k, lvl, k <= 4 && !have1, fi * ky - fj * kx);
+    long long vx = 0, vy = 0, vt = 0;
+    // the constant part's directions, x + 65536 y (axis, diagonal), and its
+    // torque moments; counts of the fallbacks, a field of 10 bits each (a
+    // particle has at most 12 x 60 - 12 links)
+    int axd = 0, dgd = 0, axt = 0, dgt = 0;
+    unsigned falls = 0u;
+    for (int li = tid; li < nvalid; li += kThreads) {
+        const int inf = list[li], k = inf & 15, sl = inf >> 16;
+        const int kx = ex(k), ky = ey(k), kb = opp(k);
+        const int fi = X0 + ((inf >> 4) & 63), fj = Y0 + ((inf >> 10) & 63);
+        const bool have1 = fluid(fi - kx, fj - ky);
+        const bool have2 = fluid(fi - 2 * kx, fj - 2 * ky);
+        // populations of fluid nodes: no team writes them during this kernel
+        const long long n0 = (long long)fj * D.pitch + fi, dn = (long long)ky * D.pitch + kx;
+        const long long n1 = have1 ? n0 - dn : n0, n2 = have2 ? n0 - 2 * dn : n0;
+        auto tv = [&](long long e) -> float { return in_bounds(D, e, D.a_elems) ? E::ld(__ldg(A + e)) : 0.f; };
+        const long long pk = k * D.ps, pb = kb * D.ps;
+        const float fk0 = tv(pk + n0), fk1 = tv(pk + n1), fk2 = tv(pk + n2);
+        const float fb0 = tv(pb + n0), fb1 = tv(pb + n1);
+        const long long gk = pk + kQ9 * D.ps, gb = pb + kQ9 * D.ps;
+        float gk0 = 0.f, gk1 = 0.f, gb0 = 0.f;
+        if (k <= 4) {
+            gk0 = tv(gk + n0);
+            gk1 = tv(gk + n1);
+            gb0 = tv(gb + n0);
         }
-        LinkSums Sw;
-        int c3w[3];
-        acc.finish(Sw, c3w);
-        if (lane == 0) {
-            if (it == 0) {
-                s_ws[warp] = Sw;
-                s_wc[warp][0] = c3w[0]; s_wc[warp][1] = c3w[1]; s_wc[warp][2] = c3w[2];
-            } else {
-                add_sums(s_ws[warp], Sw);
-                s_wc[warp][0] += c3w[0]; s_wc[warp][1] += c3w[1]; s_wc[warp][2] += c3w[2];
-            }
+        float dxf, dyf;
+        const float q = ell ? link_q_ellipse(fi, fj, k, S.ell, dxf, dyf) : link_q_df(fi, fj, k, dk, dxf, dyf);
+        if (in_bounds(D, (long long)base + sl, D.nslots)) {
+            D.slot_node[base + sl] = fj * D.nx + fi;
+            D.slot_q[base + sl] = q;
+        }
+        // curved bounce-back in deviation form: every rule is an affine
+        // combination of populations of equal weight, so it holds for
+        // f~ = f - w unchanged
+        const float rx = dxf + q * kx, ry = dyf + q * ky;
+        const float uwx = G.ux - G.om * ry, uwy = G.uy + G.om * rx;
+        const float wall = 6.f * w9(k) * -(kx * uwx + ky * uwy); // 2 w rho0 e_kbar.u_w / c_s^2
+        int lvl;
+        const float fnew = bouzidi32(q, fk0, fk1, fk2, fb0, fb1, have1, have2, wall, lvl);
+        const long long ns = n0 + dn;
+        if (in_bounds(D, pb + ns, D.a_elems)) A[pb + ns] = E::st(fnew);
+        if (k <= 4 && in_bounds(D, gb + ns, D.a_elems))
+            A[gb + ns] = E::st(thermal32(q, gk0, gk1, gb0, have1, G.wT));
+        // momentum exchange: with f = w + f~ the bracket of Eq. force is
+        // 2 w_k e_k + [f~_k^+ (e_k - u_w) - f~_kbar (e_kbar - u_w)]; the
+        // constant part and its torque 2 w_k ((i - x_c) e_k,y - (j - y_c) e_k,x)
+        // (q drops out) are kept as exact integer sums, assembled in FP64 by
+        // the particle update
+        const float bx = fk0 * (kx - uwx) - fnew * (-kx - uwx);
+        const float by = fk0 * (ky - uwy) - fnew * (-ky - uwy);
+        vx += fix_force(bx);
+        vy += fix_force(by);
+        vt += fix_torque(rx * by - ry * bx);
+        const int tz = fi * ky - fj * kx, d = kx + 65536 * ky;
+        falls += (lvl == 1 ? 1u : lvl == 2 ? 1u << 10 : 0u) + (k <= 4 && !have1 ? 1u << 20 : 0u);
+        if (k <= 4) {
+            axd += d;
+            axt += tz;
+        } else {
+            dgd += d;
+            dgt += tz;
         }
     }
-    if (rounds == 0 && lane == 0) { // no link
-        LinkSums Sz;
-        Sz.fx = Sz.fy = Sz.tz = 0;
-        Sz.ax_x = Sz.ax_y = Sz.ax_t = Sz.dg_x = Sz.dg_y = Sz.dg_t = 0;
-        s_ws[warp] = Sz;
-        s_wc[warp][0] = s_wc[warp][1] = s_wc[warp][2] = 0;
+    LinkSums R;
+    R.fx = warp_sum64(vx);
+    R.fy = warp_sum64(vy);
+    R.tz = warp_sum64(vt);
+    axd = __reduce_add_sync(F, axd);
+    dgd = __reduce_add_sync(F, dgd);
+    R.ax_t = __reduce_add_sync(F, axt);
+    R.dg_t = __reduce_add_sync(F, dgt);
+    falls = __reduce_add_sync(F, falls);
+    R.ax_x = (short)(axd & 0xffff);
+    R.ax_y = (axd - R.ax_x) >> 16;
+    R.dg_x = (short)(dgd & 0xffff);
+    R.dg_y = (dgd - R.dg_x) >> 16;
+    R.pad[0] = R.pad[1] = R.pad[2] = R.pad[3] = 0;
+    int c3[3] = {(int)(falls & 1023u), (int)((falls >> 10) & 1023u), (int)(falls >> 20)};
+    // the particle's sums over the warps (exact integer sums, so the grouping
+    // does not matter)
+    __shared__ LinkSums s_ws[kTeam];
+    __shared__ int s_wc[kTeam][3];
+    if (lane == 0) {
+        s_ws[warp] = R;
+        s_wc[warp][0] = c3[0]; s_wc[warp][1] = c3[1]; s_wc[warp][2] = c3[2];
     }
-    // ---- 5. the particle's sums over the warps (exact integer sums, so the
-    // grouping does not matter)
     __syncthreads();
     if (tid == 0) {
-        LinkSums S = s_ws[0];
-        int c3[3] = {s_wc[0][0], s_wc[0][1], s_wc[0][2]};
 #pragma unroll
-        for (int w = 1; w < kLinkThreads / 32; ++w) {
-            add_sums(S, s_ws[w]);
+        for (int w = 1; w < kTeam; ++w) {
+            add_sums(R, s_ws[w]);
             c3[0] += s_wc[w][0]; c3[1] += s_wc[w][1]; c3[2] += s_wc[w][2];
         }
-        {
-            D.lsum[p] = S;
-            unsigned long long *C = D.status->cnt[parity];
-            if (c3[0]) atomicAdd(&C[kCntBzLinear], (unsigned long long)c3[0]);
-            if (c3[1]) atomicAdd(&C[kCntBzSimple], (unsigned long long)c3[1]);
-            if (c3[2]) atomicAdd(&C[kCntThermHalf], (unsigned long long)c3[2]);
-            if (nvalid) atomicAdd(&C[kCntLinks], (unsigned long long)nvalid);
-            if (s_over) atomicOr(&D.status->err, kErrOverflow);
-        }
+        D.lsum[p] = R;
+        unsigned long long *C = D.status->cnt[parity];
+        if (c3[0]) atomicAdd(&C[kCntBzLinear], (unsigned long long)c3[0]);
+        if (c3[1]) atomicAdd(&C[kCntBzSimple], (unsigned long long)c3[1]);
+        if (c3[2]) atomicAdd(&C[kCntThermHalf], (unsigned long long)c3[2]);
+        if (nvalid) atomicAdd(&C[kCntLinks], (unsigned long long)nvalid);
+        if (S.over) atomicOr(&D.status->err, kErrOverflow);
     }
-    // the particle's position into the screening grid this step's update
-    // reads (its counts cleared by the previous step's link kernel): the
-    // atomic's round trip ends the CTA instead of lengthening the update
-    if (tid == 32) cell_insert(D, D.cells[parity], p, G.xh, G.yh);
+    // ---- 4. the particle's position into the screening grid this step's
+    // update reads (its counts cleared by the previous step's link kernel):
+    // the atomic's round trip ends the CTA instead of lengthening the update
+    if (tid == kThreads - 1) cell_insert(D, D.cells[parity], p, G.xh, G.yh);
 }
 
 // Spring repulsion magnitude of Sec. 2.4 for a gap (distance to the wall
@@ -460,25 +483,26 @@ constexpr int kPartPerBlock = kPartThreads / 32;
 
 // Support distance of particle p along the unit vector (nx, ny): its radius
 // for a disk.
-__device__ __forceinline__ double support_of(const Dev &D, int p, double nx, double ny)
+__device__ __forceinline__ double support_of(const PartSoA &P, int p, double nx, double ny)
 {
-    const double r = D.cur.r[p], b = D.cur.b[p];
+    const double r = P.r[p], b = P.b[p];
     if (!is_ellipse(r, b)) return r;
-    return ell_support(ell_frame(0.0, 0.0, D.cur.th[p], r, b), nx, ny);
+    return ell_support(ell_frame(0.0, 0.0, P.th[p], r, b), nx, ny);
 }
 
 // Pair repulsion on particle a from particle b when either is an ellipse, in
 // FP64: the gap along the line of centres is the centre distance minus both
 // support distances along it.
-__device__ __noinline__ void pair_force_ellipse(const Dev &D, int a, int b, long long &sx, long long &sy)
+__device__ __noinline__ void pair_force_ellipse(const Dev &D, int parity, int a, int b, long long &sx, long long &sy)
 {
-    const double dx = D.cur.x[a] - D.cur.x[b], dy = D.cur.y[a] - D.cur.y[b];
+    const PartSoA &P = D.part[parity];
+    const double dx = P.x[a] - P.x[b], dy = P.y[a] - P.y[b];
     const double dist = sqrt(dx * dx + dy * dy);
-    const double gap = dist - support_of(D, a, -dx / dist, -dy / dist) - support_of(D, b, dx / dist, dy / dist);
+    const double gap = dist - support_of(P, a, -dx / dist, -dy / dist) - support_of(P, b, dx / dist, dy / dist);
     if (gap > D.s_rep) return;
     auto scale = [&](int p) {
-        const double r = D.cur.r[p], pb = D.cur.b[p];
-        return kPi * r * (is_ellipse(r, pb) ? pb : r) * (D.cur.rho[p] - D.rho_f) * D.g;
+        const double r = P.r[p], pb = P.b[p];
+        return kPi * r * (is_ellipse(r, pb) ? pb : r) * (P.rho[p] - D.rho_f) * D.g;
     };
     const double mag = repulsion(gap, D.s_rep, D.eps_w, 0.5 * (scale(a) + scale(b)));
     sx += fix_of(mag * dx / dist);
@@ -505,13 +529,19 @@ __device__ __noinline__ void pair_force(float4 pa, float2 ca, float4 pb, float2 
 
 // Screening of particle a (position pa, (r, C) ca) against candidate b:
 // circumscribed circles within reach (r < 0 marks an ellipse), then the
-// pair force.
-__device__ __forceinline__ void screen_pair(const Dev &D, int a, float4 pa, float2 ca, int b, float4 pb, float2 cb,
-                                            float s_rep, float inv_eps, long long &sx, long long &sy)
+// pair force.  crowd: set when the two may share nodes after their moves,
+// each less than one node along either axis: centres within 2 sqrt(2) of the
+// sum of the radii, taken as 3 plus the FP32 rounding of the centres.
+__device__ __forceinline__ void screen_pair(const Dev &D, int parity, int a, float4 pa, float2 ca, int b, float4 pb,
+                                            float2 cb, float s_rep, float inv_eps, long long &sx, long long &sy,
+                                            bool &crowd)
 {
-    const float dxf = pa.x - pb.x, dyf = pa.y - pb.y, lim = fabsf(ca.x) + fabsf(cb.x) + s_rep + 1.f;
-    if (dxf * dxf + dyf * dyf > lim * lim || b == a) return;
-    if (ca.x < 0.f || cb.x < 0.f) pair_force_ellipse(D, a, b, sx, sy);
+    const float dxf = pa.x - pb.x, dyf = pa.y - pb.y, rr = fabsf(ca.x) + fabsf(cb.x);
+    const float lim = rr + s_rep + 1.f, touch = rr + 3.f + 2.4e-7f * (float)(D.nx + D.ny), d2 = dxf * dxf + dyf * dyf;
+    if (b == a) return;
+    crowd |= !(d2 > touch * touch);
+    if (d2 > lim * lim) return;
+    if (ca.x < 0.f || cb.x < 0.f) pair_force_ellipse(D, parity, a, b, sx, sy);
     else pair_force(pa, ca, pb, cb, s_rep, inv_eps, sx, sy);
 }
 
@@ -606,24 +636,58 @@ __device__ __forceinline__ void disk_run(const Dev &D, const Box &B, const GeomR
     hi_out = min(hi, D.nx - 1);
 }
 
-// Raster of one particle by one warp: lane per zone row for the runs, then
-// coalesced writes.  runs (may be null): the particle's row runs (lo, hi),
-// empty when lo > hi, kept for the next step's flags.
-__device__ __forceinline__ void raster_one(const Dev &D, int *own, const GeomRec &G, double x, double y, double r,
-                                           double th, double pb, int p, int2 *runs)
+// Nodes of run [lo, hi] of a row outside run [xlo, xhi] (one or two
+// intervals; all of it when [xlo, xhi] is empty), in order.
+template <typename F>
+__device__ __forceinline__ void run_minus(int lo, int hi, int xlo, int xhi, F &&f)
+{
+    if (xlo > xhi) {
+        for (int i = lo; i <= hi; ++i) f(i);
+        return;
+    }
+    for (int i = lo; i <= min(hi, xlo - 1); ++i) f(i);
+    for (int i = max(lo, xhi + 1); i <= hi; ++i) f(i);
+}
+
+// Raster of one particle by one warp, a lane per zone row: the row's run
+// (lo, hi) of inside nodes, empty when lo > hi, kept by parity; its node bits
+// (bits; at most three words a row, by atomic or); for a crowded particle
+// its nodes in the owner map (own not null).  old (may be null): its runs
+// one step back, from zone row Y0_old (a particle moves less than a node, so
+// its old nodes lie in the rows of its new zone): the nodes it left are
+// listed for the refilling.
+__device__ __forceinline__ void raster_one(const Dev &D, int par, int *own, const GeomRec &G, double x, double y,
+                                           double r, double th, double pb, int p, bool bits, const int2 *old,
+                                           int Y0_old)
 {
     const int lane = threadIdx.x & 31;
     const Box B = box_of(G);
+    int2 *runs = D.runs[par] + (long long)p * D.zone_max;
     for (int b0 = 0; b0 < B.N; b0 += 32) {
         const int j = B.Y0 + b0 + lane;
         int lo = 1, hi = 0;
         if (b0 + lane < B.N) {
             if (G.r < 0.f) ellipse_run(D, B, G, x, y, th, r, pb, j, lo, hi);
             else disk_run(D, B, G, x, y, r, j, lo, hi);
-            if (runs && in_bounds(D, (long long)p * D.zone_max + b0 + lane, (long long)D.np * D.zone_max))
+            if (in_bounds(D, (long long)p * D.zone_max + b0 + lane, (long long)D.np * D.zone_max))
                 runs[b0 + lane] = make_int2(lo, hi);
+            if (bits && lo <= hi) {
+                unsigned *row = D.bits + (long long)j * D.bpitch * 2 + par;
+                for (int w = lo >> 5; w <= hi >> 5; ++w) {
+                    const int c0 = max(lo - 32 * w, 0), c1 = min(hi - 32 * w, 31);
+                    atomicOr(row + 2 * w, (~0u << c0) & (~0u >> (31 - c1)));
+                }
+            }
+            if (old && j >= Y0_old && j < Y0_old + B.N && j >= 0 && j < D.ny) {
+                const int2 o = old[j - Y0_old];
+                run_minus(o.x, o.y, lo, hi, [&](int i) {
+                    const unsigned at = atomicAdd(&D.status->nb, 1u);
+                    if (at < (unsigned)D.left_cap) D.left[at] = make_int2(j * D.nx + i, p);
+                    else atomicOr(&D.status->err, kErrOverflow);
+                });
+            }
         }
-        write_runs(D, own, B, b0, lo, hi, p);
+        if (own) write_runs(D, own, B, b0, lo, hi, p);
     }
 }
 
@@ -668,7 +732,7 @@ __device__ __forceinline__ void particle_tail(const Dev &D, int b, int parity, l
 {
     double x = st[0], y = st[1], ux = st[2], uy = st[3];
     double th = st[4], om = st[5];
-    const double r = st[6], rho = st[7], pb = st[9];
+    const double r = st[6], pb = st[9];
     // an ellipse: wall gaps to its support distances along the wall normals
     const bool ell = is_ellipse(r, pb);
     double Fx, Fy, Tz;
@@ -734,11 +798,11 @@ __device__ __forceinline__ void particle_tail(const Dev &D, int b, int parity, l
         x = xo;
         y = yo;
     }
-    const double T = st[8];
-    D.nxt.x[b] = x; D.nxt.y[b] = y; D.nxt.ux[b] = ux; D.nxt.uy[b] = uy; D.nxt.th[b] = th;
-    D.nxt.om[b] = om; D.nxt.r[b] = r; D.nxt.rho[b] = rho; D.nxt.T[b] = T; D.nxt.b[b] = pb;
+    // (both parities hold r, rho, T and b)
+    const PartSoA &nxt = D.part[parity ^ 1];
+    nxt.x[b] = x; nxt.y[b] = y; nxt.ux[b] = ux; nxt.uy[b] = uy; nxt.th[b] = th; nxt.om[b] = om;
     const GeomRec Gn = move_geom(Gc, x, y, r, pb, th, ux, uy, om);
-    D.geo_nxt[b] = Gn;
+    D.geo[parity ^ 1][b] = Gn;
     out.G = Gn;
     out.x = x; out.y = y; out.r = r; out.th = th; out.b = pb;
 }
@@ -752,8 +816,8 @@ __device__ __forceinline__ void particles_body(const Dev &D, int parity, int *ow
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int a = blk * kPartPerBlock + warp;
     if (blk == 0 && threadIdx.x < kNumCounters) D.status->cnt[parity ^ 1][threadIdx.x] = 0ull;
-    if (blk == 0 && threadIdx.x == 0) D.status->nb = 0u;
     const bool me = a < D.np;
+    bool crowd = D.direct; // direct addressing reads the owner map of every particle
     // the last warp stages the tail's inputs (the block's particle states and
     // link sums) while every warp screens, so that the FP64 tail starts
     // without a global round trip
@@ -764,12 +828,12 @@ __device__ __forceinline__ void particles_body(const Dev &D, int parity, int *ow
     if (warp == kPartPerBlock - 1) {
         for (int t = lane; t < kPartPerBlock * kPartFields; t += 32) {
             const int q = t / kPartFields, f = t - q * kPartFields, bq = blk * kPartPerBlock + q;
-            if (bq < D.np) s_cur[q][f] = D.cur.x[(long long)f * D.np + bq];
+            if (bq < D.np) s_cur[q][f] = D.part[parity].x[(long long)f * D.np + bq];
         }
         static_assert(sizeof(GeomRec) == 64, "a geometry record is 16 words");
         for (int t = lane; t < kPartPerBlock * 16; t += 32) {
             const int q = t >> 4, w = t & 15, bq = blk * kPartPerBlock + q;
-            if (bq < D.np) reinterpret_cast<int *>(&s_geo[q])[w] = reinterpret_cast<const int *>(&D.geo_cur[bq])[w];
+            if (bq < D.np) reinterpret_cast<int *>(&s_geo[q])[w] = reinterpret_cast<const int *>(&D.geo[parity][bq])[w];
         }
         if (lane < kPartPerBlock && blk * kPartPerBlock + lane < D.np) s_pk[lane] = D.pconst[blk * kPartPerBlock + lane];
         if (!D.direct)
@@ -816,7 +880,7 @@ __device__ __forceinline__ void particles_body(const Dev &D, int parity, int *ow
                 const int c = __shfl_sync(0xffffffffu, cell, l);
                 if (t >= e && t < e + n) b = __ldg(grid + ncell + 1 + c * kCellCap + (t - e));
             }
-            if (b >= 0) screen_pair(D, a, pa, ca, b, D.pos4[b], D.prc[b], s_rep, inv_eps, sx, sy);
+            if (b >= 0) screen_pair(D, parity, a, pa, ca, b, D.pos4[b], D.prc[b], s_rep, inv_eps, sx, sy, crowd);
         }
     } else {
         // a cell overflowed: every pair, in shared-memory tiles
@@ -830,7 +894,8 @@ __device__ __forceinline__ void particles_body(const Dev &D, int parity, int *ow
             }
             __syncthreads();
             if (!me) continue;
-            for (int u = lane; u < nb; u += 32) screen_pair(D, a, pa, ca, t0 + u, sp[u], sc[u], s_rep, inv_eps, sx, sy);
+            for (int u = lane; u < nb; u += 32)
+                screen_pair(D, parity, a, pa, ca, t0 + u, sp[u], sc[u], s_rep, inv_eps, sx, sy, crowd);
         }
     }
 #pragma unroll
@@ -847,15 +912,17 @@ __device__ __forceinline__ void particles_body(const Dev &D, int parity, int *ow
     if (warp == 0 && lane < kPartPerBlock && b < D.np)
         particle_tail(D, b, parity, sred[0][lane], sred[1][lane], sras[lane], s_cur[lane], s_ls[lane],
                       s_geo[lane], s_pk[lane]);
-    // then the owner map at the new positions: warp w rasters the block's
+    // then the raster at the new positions: warp w rasters the block's
     // particle w (its own new state only, so no other block is waited for)
     __syncthreads();
     if (a < D.np) {
         const RasterIn &R = sras[warp];
-        raster_one(D, own_nxt, R.G, R.x, R.y, R.r, R.th, R.b, a, D.runs[parity ^ 1] + (long long)a * D.zone_max);
+        crowd = __any_sync(0xffffffffu, crowd);
+        if (lane == 0) D.crowd[parity ^ 1][a] = crowd;
+        raster_one(D, parity ^ 1, crowd ? own_nxt : nullptr, R.G, R.x, R.y, R.r, R.th, R.b, a, true,
+                   D.runs[parity] + (long long)a * D.zone_max, s_geo[warp].Y0);
     }
 }
-
 
 
 // Owner map: node (i,j) belongs to disk p iff (i - x)^2 + (j - y)^2 <= r^2
@@ -867,137 +934,25 @@ __device__ __forceinline__ void particles_body(const Dev &D, int parity, int *ow
 // of its ends and settled with the exact predicate at the ends only; the
 // runs are then written row by row with coalesced atomicMax requests.
 
-__device__ __forceinline__ void raster_body(const Dev &D, int *own, const GeomRec *__restrict__ geo,
-                                            const PartSoA &pos, int2 *runs, const int blk)
+__device__ __forceinline__ void raster_body(const Dev &D, int *own, bool bits, int par, const int blk)
 {
     const int p = blk * (kBoxThreads / 32) + (threadIdx.x >> 5);
     if (p >= D.np) return;
-    raster_one(D, own, geo[p], pos.x[p], pos.y[p], pos.r[p], pos.th[p], pos.b[p], p,
-               runs ? runs + (long long)p * D.zone_max : nullptr);
-}
-
-// Class of a node from the two owner maps: solid at the new time, newborn
-// (solid before, fluid now) or fluid.
-__device__ __forceinline__ uint8_t node_class(int oc, int on) { return on >= 0 ? kSolid : oc >= 0 ? kNewborn : kFluid; }
-
-// A newborn node into this step's list (j * nx + i off the cavity frame,
-// ~(j * nx + i) on it, where the general path takes it anyway).
-__device__ __forceinline__ void list_newborn(const Dev &D, int i, int j)
-{
-    const unsigned at = atomicAdd(&D.status->nb, 1u);
-    const int n = j * D.nx + i;
-    const bool frame = i == 0 || i == D.nx - 1 || j == 0 || j == D.ny - 1;
-    if (at < (unsigned)D.newborn_cap) D.newborn[at] = frame ? ~n : n;
-    else atomicOr(&D.status->err, kErrOverflow);
-}
-
-// Nodes of run [lo, hi] of row j outside run [xlo, xhi] (one or two
-// intervals; all of it when [xlo, xhi] is empty), in order.
-template <typename F>
-__device__ __forceinline__ void run_minus(int lo, int hi, int xlo, int xhi, F &&f)
-{
-    if (xlo > xhi) {
-        for (int i = lo; i <= hi; ++i) f(i);
-        return;
-    }
-    for (int i = lo; i <= min(hi, xlo - 1); ++i) f(i);
-    for (int i = max(lo, xhi + 1); i <= hi; ++i) f(i);
-}
-
-// Node flags of a step.  Before it, every node holds its class for the
-// previous step (the link kernel has returned that step's newborn nodes to
-// fluid); a node's class can only change where it enters or leaves a
-// particle, so the team of particle p visits, row by row, the nodes of its
-// disk at the new position outside its disk at the current one (solid now:
-// every disk holding a node writes the same class) and the nodes of its
-// current disk outside the new one (solid if another particle now holds
-// them, else newborn, listed once, by the particle that owned the node),
-// from the row runs the rasters kept.  A team of TEAM warps per particle
-// (one warp when the particles alone fill the GPU, else 2 or 4), lane l on
-// rows l, l + 32 TEAM, ...  Team warp 0 also moves the particle's new state
-// into the current slot and keeps the old position for the next clear.
-// Initialisation (rotate == 0): every node of the zone rectangle from the
-// owner map (own_cur == own_nxt), nothing listed.
-template <int TEAM>
-__device__ __forceinline__ void flags_body(const Dev &D, const int *__restrict__ own_cur,
-                                           const int *__restrict__ own_nxt, int rotate, int parity, const int p)
-{
-    const int lane = threadIdx.x & 31, tw = (threadIdx.x >> 5) % TEAM;
-    // a team past the last particle still reaches the block barrier below
-    const bool act = p < D.np; // uniform across the team
-    Box Bb{0, 0, 0}, Bc{0, 0, 0};
-    if (act) {
-        Bb = box_of(D.geo_cur[p]);
-        Bc = box_of(D.geo_nxt[p]);
-    }
-    if (rotate) {
-        // the new state moves into the current slot (and the current position
-        // into the previous one) while the other threads work on the flags;
-        // every thread of the team has read the boxes before
-        if (TEAM == 1) __syncwarp();
-        else __syncthreads();
-        if (act && tw == 0) switch (lane) {
-        case 0: D.px[p] = D.cur.x[p]; D.cur.x[p] = D.nxt.x[p]; break;
-        case 1: D.py[p] = D.cur.y[p]; D.cur.y[p] = D.nxt.y[p]; break;
-        case 2: D.cur.ux[p] = D.nxt.ux[p]; break;
-        case 3: D.cur.uy[p] = D.nxt.uy[p]; break;
-        case 4: D.cur.th[p] = D.nxt.th[p]; break;
-        case 5: D.cur.om[p] = D.nxt.om[p]; break;
-        case 6: D.geo_prev[p] = D.geo_cur[p]; D.geo_cur[p] = D.geo_nxt[p]; break;
-        default: break;
-        }
-    }
-    if (!act) return;
-    const long long nflags = (long long)D.ny * D.pitch;
-    if (!rotate) {
-        // every node of the zone (one position: own_cur == own_nxt)
-        for (int r = tw; r < Bb.N; r += TEAM) {
-            const int j = Bb.Y0 + r;
-            if (j < 0 || j >= D.ny) continue;
-            for (int c = lane; c < Bb.N; c += 32) {
-                const int i = Bb.X0 + c;
-                if (i < 0 || i >= D.nx) continue;
-                const int n = j * D.nx + i;
-                const long long o = (long long)j * D.pitch + i;
-                if (in_bounds(D, o, nflags)) D.flags[o] = node_class(own_cur[n], own_nxt[n]);
-            }
-        }
-        return;
-    }
-    const int2 *Ro = D.runs[parity] + (long long)p * D.zone_max;     // current position
-    const int2 *Rn = D.runs[parity ^ 1] + (long long)p * D.zone_max; // new position
-    const int ylo = min(Bb.Y0, Bc.Y0), yhi = max(Bb.Y0 + Bb.N, Bc.Y0 + Bc.N);
-    for (int j = ylo + tw * 32 + lane; j < yhi; j += TEAM * 32) {
-        if (j < 0 || j >= D.ny) continue;
-        int2 o = make_int2(1, 0), w = make_int2(1, 0);
-        if (j - Bb.Y0 >= 0 && j - Bb.Y0 < Bb.N) o = Ro[j - Bb.Y0];
-        if (j - Bc.Y0 >= 0 && j - Bc.Y0 < Bc.N) w = Rn[j - Bc.Y0];
-        const long long row = (long long)j * D.pitch;
-        // entering the particle: solid at the new time
-        run_minus(w.x, w.y, o.x, o.y, [&](int i) {
-            if (in_bounds(D, row + i, nflags)) D.flags[row + i] = kSolid;
-        });
-        // leaving it: newborn unless another particle holds the node now
-        run_minus(o.x, o.y, w.x, w.y, [&](int i) {
-            const int n = j * D.nx + i;
-            const int oc = own_cur[n];
-            const uint8_t f = node_class(oc, own_nxt[n]);
-            if (in_bounds(D, row + i, nflags)) D.flags[row + i] = f;
-            if (f == kNewborn && oc == p) list_newborn(D, i, j);
-        });
-    }
+    const PartSoA &P = D.part[par];
+    if (own && (threadIdx.x & 31) == 0) D.crowd[par][p] = 1;
+    raster_one(D, par, own, D.geo[par][p], P.x[p], P.y[p], P.r[p], P.th[p], P.b[p], p, bits, nullptr, 0);
 }
 
 // Near-tile bitmap: every warp tile (one row, 32 V nodes) that meets a
 // particle's zone at the current position widened by kNearMargin nodes.  One
 // thread per particle and zone row; the bitmap is cleared beforehand.
-__global__ void __launch_bounds__(128) k_near_mask(const Dev D, int span)
+__global__ void __launch_bounds__(128) k_near_mask(const Dev D, int span, int parity)
 {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     const int Nm = D.zone_max + 2 * kNearMargin;
     const int p = g / Nm, r = g - p * Nm;
     if (p >= D.np) return;
-    const GeomRec G = D.geo_cur[p];
+    const GeomRec G = D.geo[parity][p];
     const int j = G.Y0 - kNearMargin + r;
     if (r >= G.N + 2 * kNearMargin || j < 0 || j >= D.ny) return;
     const int x0 = max(G.X0 - kNearMargin, 0), x1 = min(G.X0 + G.N - 1 + kNearMargin, D.pitch - 1);
@@ -1008,25 +963,17 @@ __global__ void __launch_bounds__(128) k_near_mask(const Dev D, int span)
 }
 
 // ---- direct addressing (comparison with the index array)
-// Per particle: clear its zone one step back in the next owner map, return
-// the last step's newborn nodes to fluid, publish its centre for the pair
-// screening, zero its sums.
+// Per particle: clear its zone one step back in the next node bits and owner
+// map, publish its centre for the pair screening, zero its sums.
 __global__ void __launch_bounds__(kBoxThreads) k_direct_prep(const Dev D, int *__restrict__ own_nxt, int parity)
 {
-    const int p = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int p = blockIdx.x;
     clear_cells_slice(D, parity, p, threadIdx.x, kBoxThreads);
-    revert_newborn(D, p, threadIdx.x, kBoxThreads);
-    const GeomRec Gp = D.geo_prev[p];
-    for (int r = warp; r < Gp.N; r += kBoxThreads / 32) {
-        const int j = Gp.Y0 + r;
-        if (j < 0 || j >= D.ny) continue;
-        for (int c = lane; c < Gp.N; c += 32) {
-            const int i = Gp.X0 + c;
-            if (i >= 0 && i < D.nx) own_nxt[(long long)j * D.nx + i] = -1;
-        }
-    }
+    if (p == 0 && threadIdx.x == 0) D.status->nb = 0u;
+    if (threadIdx.x < 32) clear_zone_bits(D, parity, p, threadIdx.x);
+    clear_zone_owner(D, own_nxt, parity, p, threadIdx.x, kBoxThreads);
     if (threadIdx.x == 0) {
-        const GeomRec G = D.geo_cur[p];
+        const GeomRec G = D.geo[parity][p];
         const DiskDF d0 = geom_df(G);
         D.pos4[p] = make_float4(d0.xh, d0.yh, d0.xl, d0.yl);
         D.prc[p] = make_float2(G.r, G.C);
@@ -1062,11 +1009,10 @@ __global__ void __launch_bounds__(128)
             if (si < 0 || si >= D.nx || sj < 0 || sj >= D.ny) continue;
             const int p = own[(long long)sj * D.nx + si];
             if (p < 0) continue;
-            const GeomRec G = D.geo_cur[p];
+            const GeomRec G = D.geo[parity][p];
+            const PartSoA &P = D.part[parity];
             float dxf, dyf;
-            const float q = G.r < 0.f ? link_q_ellipse(i, j, k,
-                                                       ell_frame(D.cur.x[p], D.cur.y[p], D.cur.th[p], D.cur.r[p],
-                                                                 D.cur.b[p]),
+            const float q = G.r < 0.f ? link_q_ellipse(i, j, k, ell_frame(P.x[p], P.y[p], P.th[p], P.r[p], P.b[p]),
                                                        dxf, dyf)
                                       : link_q_df(i, j, k, geom_df(G), dxf, dyf);
             const int kb = opp(k);
@@ -1118,43 +1064,76 @@ __global__ void __launch_bounds__(128)
 }
 
 // ---- single-instance kernels
-// 16 CTAs per SM (the 2,048-thread limit; 32 registers): the kernel is
-// latency-bound, and 16 particles in flight per SM instead of the 9 that 56
-// registers allow beat the few spilled registers (80 against 91 us per step
-// on the 4000^2 / 4800-disk benchmark).
-constexpr int kLinkCtasPerSm = 16;
-template <typename T>
-__global__ void __launch_bounds__(kLinkThreads, kLinkCtasPerSm)
+// Warps per particle, one CTA each: eight while that is a single wave (three
+// CTAs of 80 registers per SM), else four (eight CTAs of 64 registers).  Link
+// kernel, us, eight / four (CUDA events): 8 disks 9.9 / 11.9, 300 disks
+// 12.1 / 14.2, 129 ellipses 21.3 / 23.0, 4800 disks 84.7 / 72.1.  (One warp per
+// particle, four particles per CTA: 75.4 with 4800 disks; 12 CTAs per SM:
+// 82.3.)  With many particles it is bound by its scattered accesses: the
+// loads and stores of the links alone, from a kernel that does nothing else,
+// take 61 us for 4800 disks in 4000^2 from HBM, in any layout of the planes.
+constexpr int link_ctas(int team) { return team == 4 ? 8 : 3; }
+template <typename T, int kTeam>
+__global__ void __launch_bounds__(32 * kTeam, link_ctas(kTeam))
     k_links(const Dev D, T *A, const int *__restrict__ own,
             int *__restrict__ own_nxt, int parity, int ahead)
 {
     // CTAs in the link order (descending y, the rows stream-collide wrote
     // last first)
     const int b = (int)blockIdx.x;
-    links_body<T>(D, A, own, own_nxt, parity, __ldg(D.lorder + b), b + ahead < D.np ? __ldg(D.lorder + b + ahead) : -1);
+    links_body<T, kTeam>(D, A, own, own_nxt, parity, __ldg(D.lorder + b),
+                         b + ahead < D.np ? __ldg(D.lorder + b + ahead) : -1);
 }
 __global__ void __launch_bounds__(kPartThreads, 4) k_particles(const Dev D, int parity, int *own_nxt)
 {
     particles_body(D, parity, own_nxt, (int)blockIdx.x);
 }
 __global__ void __launch_bounds__(kBoxThreads)
-    k_raster(const Dev D, int *own, const GeomRec *__restrict__ geo, const PartSoA pos, int2 *runs)
+    k_raster(const Dev D, int *own, bool bits, int parity)
 {
-    raster_body(D, own, geo, pos, runs, (int)blockIdx.x);
+    raster_body(D, own, bits, parity, (int)blockIdx.x);
 }
-template <int TEAM>
-__global__ void __launch_bounds__(kBoxThreads, 9)
-    k_flags(const Dev D, const int *__restrict__ own_cur, const int *__restrict__ own_nxt, int rotate, int parity)
+// The whole owner map (-1 before) from the row runs of a parity.
+__global__ void __launch_bounds__(kBoxThreads) k_owner(const Dev D, int *own, int parity)
 {
-    flags_body<TEAM>(D, own_cur, own_nxt, rotate, parity,
-                     (int)blockIdx.x * (kBoxThreads / 32 / TEAM) + (int)(threadIdx.x >> 5) / TEAM);
+    const int p = (int)blockIdx.x * (kBoxThreads / 32) + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (p >= D.np) return;
+    const Box B = box_of(D.geo[parity][p]);
+    for (int b0 = 0; b0 < B.N; b0 += 32) {
+        int2 run = make_int2(1, 0);
+        if (b0 + lane < B.N) run = D.runs[parity][(long long)p * D.zone_max + b0 + lane];
+        write_runs(D, own, B, b0, run.x, run.y, p);
+    }
+}
+// A state image's flag map from the node bits before a step of `parity`, a
+// thread per node, and back, a thread per word.
+__global__ void k_flags_out(const Dev D, uint8_t *flags, int parity)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+    if (i >= D.pitch) return;
+    flags[(long long)j * D.pitch + i] = solid_at(D, i, j, parity)       ? kSolid
+                                        : solid_at(D, i, j, parity ^ 1) ? kNewborn
+                                                                        : kFluid;
+}
+__global__ void k_flags_in(const Dev D, const uint8_t *flags, int parity)
+{
+    const int w = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+    if (w >= D.bpitch) return;
+    unsigned now = 0u, before = 0u;
+    for (int b = 0; b < 32 && 32 * w + b < D.nx; ++b) {
+        const uint8_t f = flags[(long long)j * D.pitch + 32 * w + b];
+        now |= (f == kSolid ? 1u : 0u) << b;
+        before |= (f == kNewborn ? 1u : 0u) << b;
+    }
+    D.bits[bit_word(D, 32 * w, j, parity)] = now;
+    D.bits[bit_word(D, 32 * w, j, parity ^ 1)] = before;
 }
 
 // ---- batched kernels: one grid over all instances (InstArgs table, block
 // offsets `start`).  The link kernel's look-ahead owner-row prefetch stays
 // within the instance.
-template <typename T>
-__global__ void __launch_bounds__(kLinkThreads, kLinkCtasPerSm)
+template <typename T, int kTeam>
+__global__ void __launch_bounds__(32 * kTeam, link_ctas(kTeam))
     k_links_batch(const InstArgs *__restrict__ I, const int *__restrict__ start, int n, int parity, int ahead)
 {
     __shared__ Dev sD;
@@ -1163,7 +1142,8 @@ __global__ void __launch_bounds__(kLinkThreads, kLinkCtasPerSm)
     copy_dev(sD, a.D);
     const int par = parity ^ a.poff;
     const int b = (int)blockIdx.x - __ldg(start + i);
-    links_body<T>(sD, static_cast<T *>(a.A[par]), a.own[par], a.own[par ^ 1], par, b, b + ahead < sD.np ? b + ahead : -1);
+    links_body<T, kTeam>(sD, static_cast<T *>(a.A[par]), a.own[par], a.own[par ^ 1], par, b,
+                         b + ahead < sD.np ? b + ahead : -1);
 }
 __global__ void __launch_bounds__(kPartThreads, 4)
     k_particles_batch(const InstArgs *__restrict__ I, const int *__restrict__ start, int n, int parity)
@@ -1174,42 +1154,18 @@ __global__ void __launch_bounds__(kPartThreads, 4)
     const int par = parity ^ I[i].poff;
     particles_body(sD, par, I[i].own[par ^ 1], (int)blockIdx.x - __ldg(start + i));
 }
-__global__ void __launch_bounds__(kBoxThreads)
-    k_raster_batch(const InstArgs *__restrict__ I, const int *__restrict__ start, int n, int parity)
-{
-    __shared__ Dev sD;
-    const int i = batch_find(start, n, (int)blockIdx.x);
-    const InstArgs &a = I[i];
-    copy_dev(sD, a.D);
-    raster_body(sD, a.own[parity ^ a.poff ^ 1], sD.geo_nxt, sD.nxt, sD.runs[parity ^ a.poff ^ 1],
-                (int)blockIdx.x - __ldg(start + i));
-}
-__global__ void __launch_bounds__(kBoxThreads)
-    k_flags_batch(const InstArgs *__restrict__ I, const int *__restrict__ start, int n, int parity)
-{
-    __shared__ Dev sD;
-    const int i = batch_find(start, n, (int)blockIdx.x);
-    const InstArgs &a = I[i];
-    copy_dev(sD, a.D);
-    const int par = parity ^ a.poff;
-    flags_body<1>(sD, a.own[par], a.own[par ^ 1], 1, par,
-                  ((int)blockIdx.x - __ldg(start + i)) * (kBoxThreads / 32) + (int)(threadIdx.x >> 5));
-}
-
-// Geometry records of the current state and of the previous positions.
+// Geometry records of both parities' states.
 __global__ void k_geom_init(const Dev D)
 {
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= D.np) return;
-    const GeomRec G = make_geom(D.cur.x[a], D.cur.y[a], D.cur.r[a], D.cur.b[a], D.cur.th[a], D.cur.ux[a],
-                                D.cur.uy[a], D.cur.om[a], D.cur.T[a], D.cur.rho[a], D.rho_f, D.g);
-    D.geo_cur[a] = G;
-    D.geo_nxt[a] = G;
-    D.pconst[a] = part_consts(D.cur.r[a], D.cur.b[a], D.cur.rho[a], D.rho_f, D.g);
-    // (the orientation one step back is not kept: the current one, which
-    // only shapes the raster of that owner map inside the same zone)
-    D.geo_prev[a] = make_geom(D.px[a], D.py[a], D.cur.r[a], D.cur.b[a], D.cur.th[a], 0.0, 0.0, 0.0, D.cur.T[a],
-                              D.cur.rho[a], D.rho_f, D.g);
+    for (int q = 0; q < 2; ++q) {
+        const PartSoA &P = D.part[q];
+        D.geo[q][a] = make_geom(P.x[a], P.y[a], P.r[a], P.b[a], P.th[a], P.ux[a], P.uy[a], P.om[a], P.T[a], P.rho[a],
+                                D.rho_f, D.g);
+    }
+    const PartSoA &P = D.part[0];
+    D.pconst[a] = part_consts(P.r[a], P.b[a], P.rho[a], D.rho_f, D.g);
 }
 
 // Link order: the particles by descending y in kOrderBands bands of rows,
@@ -1221,12 +1177,12 @@ __global__ void k_geom_init(const Dev D)
 // against 0.3750 ms).  Only the order of the CTAs changes, not what any of
 // them computes.
 constexpr int kOrderBands = 1024;
-__global__ void __launch_bounds__(kOrderBands) k_link_order(const Dev D)
+__global__ void __launch_bounds__(kOrderBands) k_link_order(const Dev D, int parity)
 {
     __shared__ int cnt[kOrderBands], at[kOrderBands];
     const int t = threadIdx.x;
     auto band = [&](int p) {
-        const double y = D.cur.y[p];
+        const double y = D.part[parity].y[p];
         const int b = (int)((double)kOrderBands * (((double)D.ny - 1.0) - y) / (double)D.ny);
         return min(max(b, 0), kOrderBands - 1);
     };
@@ -1250,32 +1206,55 @@ __global__ void __launch_bounds__(kOrderBands) k_link_order(const Dev D)
     }
 }
 
-__global__ void k_pack_particles(const Dev D, lbm_particle *out)
+__global__ void k_pack_particles(const Dev D, lbm_particle *out, int parity)
 {
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= D.np) return;
+    const PartSoA &C = D.part[parity];
     lbm_particle P;
-    P.x = D.cur.x[a]; P.y = D.cur.y[a]; P.ux = D.cur.ux[a]; P.uy = D.cur.uy[a];
-    P.theta = D.cur.th[a]; P.omega = D.cur.om[a]; P.r = D.cur.r[a]; P.rho = D.cur.rho[a];
-    P.T = D.cur.T[a]; P.b = D.cur.b[a];
+    P.x = C.x[a]; P.y = C.y[a]; P.ux = C.ux[a]; P.uy = C.uy[a];
+    P.theta = C.th[a]; P.omega = C.om[a]; P.r = C.r[a]; P.rho = C.rho[a];
+    P.T = C.T[a]; P.b = C.b[a];
     out[a] = P;
 }
 
 namespace {
 
-template <typename T>
-void *link_kernel()
+// f(storage tag, team tag) for a storage and a team size.
+template <typename F>
+auto link_dispatch(int storage, int team, F &&f)
 {
-    return reinterpret_cast<void *>(&k_links<T>);
+    auto by_team = [&](auto t) {
+        return team == 4 ? f(t, std::integral_constant<int, 4>{}) : f(t, std::integral_constant<int, 8>{});
+    };
+    return storage == LBM_STORE_BF16   ? by_team(__nv_bfloat16{})
+           : storage == LBM_STORE_FP16 ? by_team(__half{})
+                                       : by_team(float{});
 }
 
-void *link_kernel_for(int storage)
+// Warps per particle for np particles (see link_ctas).
+int link_team(int np, int sms) { return np <= link_ctas(8) * sms ? 8 : 4; }
+int sm_count()
 {
-    switch (storage) {
-    case LBM_STORE_BF16: return link_kernel<__nv_bfloat16>();
-    case LBM_STORE_FP16: return link_kernel<__half>();
-    default: return link_kernel<float>();
-    }
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    return sms;
+}
+
+// Shared-memory limit of a link kernel for zones of side N, and the CTAs of it
+// that the GPU holds at once (the distance of its prefetch).
+template <typename K>
+cudaError_t prepare_link_kernel(K fn, int team, int N, int sms, int *ahead)
+{
+    const int smem = (int)link_smem_bytes(N);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    int per_sm = 0;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * team, smem)) != cudaSuccess) return e;
+    *ahead = max(1, sms * per_sm);
+    return cudaSuccess;
 }
 
 } // namespace
@@ -1283,80 +1262,52 @@ void *link_kernel_for(int storage)
 cudaError_t prepare_links(Dev &D)
 {
     D.link_ahead = 1;
-    D.flag_team = 1;
+    D.link_team = 4;
     if (D.np == 0) return cudaSuccess;
-    const size_t smem = link_smem_bytes(D.zone_max, D.storage);
-    const void *fn = link_kernel_for(D.storage);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0, sms = 0, dev = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kLinkThreads, smem)) != cudaSuccess)
-        return e;
-    D.link_ahead = max(1, sms * per_sm); // particles (CTAs) resident at once
-    // flags: one warp per particle when there are enough particles to fill
-    // the GPU (about 36 warps per SM), else teams of 2 or 4 warps
-    const int warps = sms * 36;
-    D.flag_team = D.np * 2 > warps ? 1 : D.np * 4 > warps ? 2 : 4;
-    return cudaSuccess;
+    const int sms = sm_count();
+    if (!sms) return cudaErrorUnknown;
+    D.link_team = link_team(D.np, sms);
+    return link_dispatch(D.storage, D.link_team, [&](auto t, auto team) {
+        return prepare_link_kernel(k_links<decltype(t), decltype(team)::value>, decltype(team)::value, D.zone_max, sms,
+                                   &D.link_ahead);
+    });
 }
 
 cudaError_t launch_links(const Dev &D, void *A, const int *own_cur, int *own_nxt, int parity,
                          cudaStream_t s)
 {
     if (D.np == 0) return cudaSuccess;
-    const size_t smem = link_smem_bytes(D.zone_max, D.storage);
-    const int grid = D.np;
-    switch (D.storage) {
-    case LBM_STORE_FP32:
-        k_links<float><<<grid, kLinkThreads, smem, s>>>(D, static_cast<float *>(A), own_cur, own_nxt, parity,
-                                                        D.link_ahead);
-        break;
-    case LBM_STORE_BF16:
-        k_links<__nv_bfloat16><<<grid, kLinkThreads, smem, s>>>(D, static_cast<__nv_bfloat16 *>(A), own_cur,
-                                                                own_nxt, parity, D.link_ahead);
-        break;
-    case LBM_STORE_FP16:
-        k_links<__half><<<grid, kLinkThreads, smem, s>>>(D, static_cast<__half *>(A), own_cur, own_nxt, parity,
-                                                         D.link_ahead);
-        break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    return link_dispatch(D.storage, D.link_team, [&](auto t, auto team) {
+        using T = decltype(t);
+        constexpr int W = decltype(team)::value;
+        k_links<T, W><<<D.np, 32 * W, link_smem_bytes(D.zone_max), s>>>(D, static_cast<T *>(A), own_cur, own_nxt,
+                                                                        parity, D.link_ahead);
+        return cudaGetLastError();
+    });
 }
 
 // ---- batched launches (one grid over all instances)
-cudaError_t prepare_links_batch(int zone_max, int storage, size_t *smem, int *ahead)
+cudaError_t prepare_links_batch(int zone_max, int np, int storage, LinkPlan *plan)
 {
-    *smem = link_smem_bytes(zone_max, storage);
-    const void *fn = storage == LBM_STORE_BF16   ? reinterpret_cast<const void *>(&k_links_batch<__nv_bfloat16>)
-                     : storage == LBM_STORE_FP16 ? reinterpret_cast<const void *>(&k_links_batch<__half>)
-                                                 : reinterpret_cast<const void *>(&k_links_batch<float>);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0, sms = 0, dev = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kLinkThreads, *smem)) != cudaSuccess)
-        return e;
-    *ahead = max(1, sms * per_sm);
-    return cudaSuccess;
+    const int sms = sm_count();
+    if (!sms) return cudaErrorUnknown;
+    plan->team = link_team(np, sms);
+    plan->smem = link_smem_bytes(zone_max);
+    return link_dispatch(storage, plan->team, [&](auto t, auto team) {
+        return prepare_link_kernel(k_links_batch<decltype(t), decltype(team)::value>, decltype(team)::value, zone_max,
+                                   sms, &plan->ahead);
+    });
 }
 
 cudaError_t launch_links_batch(const InstArgs *I, const int *start, int n, int total, int storage, int parity,
-                               int ahead, size_t smem, cudaStream_t s)
+                               const LinkPlan &plan, cudaStream_t s)
 {
     if (total <= 0) return cudaSuccess;
-    switch (storage) {
-    case LBM_STORE_FP32: k_links_batch<float><<<total, kLinkThreads, smem, s>>>(I, start, n, parity, ahead); break;
-    case LBM_STORE_BF16:
-        k_links_batch<__nv_bfloat16><<<total, kLinkThreads, smem, s>>>(I, start, n, parity, ahead);
-        break;
-    case LBM_STORE_FP16: k_links_batch<__half><<<total, kLinkThreads, smem, s>>>(I, start, n, parity, ahead); break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    return link_dispatch(storage, plan.team, [&](auto t, auto team) {
+        constexpr int W = decltype(team)::value;
+        k_links_batch<decltype(t), W><<<total, 32 * W, plan.smem, s>>>(I, start, n, parity, plan.ahead);
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_particles_batch(const InstArgs *I, const int *start, int n, int total, int parity,
@@ -1367,41 +1318,26 @@ cudaError_t launch_particles_batch(const InstArgs *I, const int *start, int n, i
     return cudaGetLastError();
 }
 
-cudaError_t launch_raster_batch(const InstArgs *I, const int *start, int n, int total, int parity, cudaStream_t s)
-{
-    if (total <= 0) return cudaSuccess;
-    k_raster_batch<<<total, kBoxThreads, 0, s>>>(I, start, n, parity);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_flags_batch(const InstArgs *I, const int *start, int n, int total, int parity, cudaStream_t s)
-{
-    if (total <= 0) return cudaSuccess;
-    k_flags_batch<<<total, kBoxThreads, 0, s>>>(I, start, n, parity);
-    return cudaGetLastError();
-}
-
 // Blocks of each batched step kernel for one instance.
 void batch_blocks(const Dev &D, dim3 sc_block, int out[kBatchPhases])
 {
     const int V = D.storage == LBM_STORE_FP32 ? 1 : 2;
     out[kBLinks] = D.np;
-    out[kBParticles] = D.np > 0 ? (D.np + kPartPerBlock - 1) / kPartPerBlock : 1;
-    out[kBRaster] = (D.np + kBoxThreads / 32 - 1) / (kBoxThreads / 32);
-    out[kBFlags] = (D.np + kBoxThreads / 32 - 1) / (kBoxThreads / 32);
+    out[kBParticles] = (D.np + kPartPerBlock - 1) / kPartPerBlock;
+    out[kBRefill] = (D.np + kBoxThreads - 1) / kBoxThreads;
     out[kBStream] = ((D.pitch / V + (int)sc_block.x - 1) / (int)sc_block.x) *
                     ((D.ny + (int)sc_block.y - 1) / (int)sc_block.y);
     out[kBBoundary] = kBoundaryBlocksPerInstance;
 }
 
-cudaError_t launch_near_mask(const Dev &D, cudaStream_t s)
+cudaError_t launch_near_mask(const Dev &D, int parity, cudaStream_t s)
 {
     const size_t words = ((size_t)D.ny * D.near_tpr + 31) / 32;
     cudaError_t e = cudaMemsetAsync(D.near, 0, words * sizeof(unsigned), s);
     if (e != cudaSuccess || D.np == 0) return e;
     const int span = 32 * (D.storage == LBM_STORE_FP32 ? 1 : 2);
     const long long threads = (long long)D.np * (D.zone_max + 2 * kNearMargin);
-    k_near_mask<<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(D, span);
+    k_near_mask<<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(D, span, parity);
     return cudaGetLastError();
 }
 
@@ -1426,16 +1362,16 @@ cudaError_t launch_links_direct(const Dev &D, void *A, const int *own_cur, int *
 
 cudaError_t launch_particles(const Dev &D, int parity, int *own_nxt, cudaStream_t s)
 {
-    const int blocks = D.np > 0 ? (D.np + kPartPerBlock - 1) / kPartPerBlock : 1;
-    k_particles<<<blocks, kPartThreads, 0, s>>>(D, parity, own_nxt);
+    if (D.np == 0) return cudaSuccess;
+    k_particles<<<(D.np + kPartPerBlock - 1) / kPartPerBlock, kPartThreads, 0, s>>>(D, parity, own_nxt);
     return cudaGetLastError();
 }
 
-cudaError_t launch_raster(const Dev &D, int *own, const GeomRec *geo, const PartSoA &pos, int2 *runs, cudaStream_t s)
+cudaError_t launch_raster(const Dev &D, int *own, bool bits, int parity, cudaStream_t s)
 {
     if (D.np == 0) return cudaSuccess;
     const int per = kBoxThreads / 32;
-    k_raster<<<(D.np + per - 1) / per, kBoxThreads, 0, s>>>(D, own, geo, pos, runs);
+    k_raster<<<(D.np + per - 1) / per, kBoxThreads, 0, s>>>(D, own, bits, parity);
     return cudaGetLastError();
 }
 
@@ -1446,10 +1382,10 @@ cudaError_t launch_geom_init(const Dev &D, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_link_order(const Dev &D, cudaStream_t s)
+cudaError_t launch_link_order(const Dev &D, int parity, cudaStream_t s)
 {
     if (D.np == 0) return cudaSuccess;
-    k_link_order<<<1, kOrderBands, 0, s>>>(D);
+    k_link_order<<<1, kOrderBands, 0, s>>>(D, parity);
     return cudaGetLastError();
 }
 
@@ -1463,40 +1399,30 @@ cudaError_t launch_cells_init(const Dev &D, cudaStream_t s)
     return cudaSuccess;
 }
 
-cudaError_t launch_flags(const Dev &D, const int *own_cur, const int *own_nxt, int rotate, int parity,
-                         cudaStream_t s)
+cudaError_t launch_owner(const Dev &D, int *own, int parity, cudaStream_t s)
 {
     if (D.np == 0) return cudaSuccess;
-    const int per = kBoxThreads / 32 / max(D.flag_team, 1); // particles per block
-    const int grid = (D.np + per - 1) / per;
-    switch (D.flag_team) {
-    case 4: k_flags<4><<<grid, kBoxThreads, 0, s>>>(D, own_cur, own_nxt, rotate, parity); break;
-    case 2: k_flags<2><<<grid, kBoxThreads, 0, s>>>(D, own_cur, own_nxt, rotate, parity); break;
-    default: k_flags<1><<<grid, kBoxThreads, 0, s>>>(D, own_cur, own_nxt, rotate, parity); break;
-    }
+    const int per = kBoxThreads / 32;
+    k_owner<<<(D.np + per - 1) / per, kBoxThreads, 0, s>>>(D, own, parity);
     return cudaGetLastError();
 }
 
-// Newborn nodes of a restored state: every node whose flag says newborn
-// goes into the list (emptied first by the caller), which the next step's
-// link kernel returns to fluid.
-__global__ void k_collect_newborn(const Dev D)
+cudaError_t launch_flags_out(const Dev &D, uint8_t *flags, int parity, cudaStream_t s)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-    if (i >= D.nx) return;
-    if (D.flags[(long long)j * D.pitch + i] == kNewborn) list_newborn(D, i, j);
-}
-
-cudaError_t launch_collect_newborn(const Dev &D, cudaStream_t s)
-{
-    k_collect_newborn<<<dim3((D.nx + 127) / 128, D.ny), 128, 0, s>>>(D);
+    k_flags_out<<<dim3((D.pitch + 127) / 128, D.ny), 128, 0, s>>>(D, flags, parity);
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_particles(const Dev &D, lbm_particle *out, cudaStream_t s)
+cudaError_t launch_flags_in(const Dev &D, const uint8_t *flags, int parity, cudaStream_t s)
+{
+    k_flags_in<<<dim3((D.bpitch + 31) / 32, D.ny), 32, 0, s>>>(D, flags, parity);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pack_particles(const Dev &D, lbm_particle *out, int parity, cudaStream_t s)
 {
     if (D.np == 0) return cudaSuccess;
-    k_pack_particles<<<(D.np + 127) / 128, 128, 0, s>>>(D, out);
+    k_pack_particles<<<(D.np + 127) / 128, 128, 0, s>>>(D, out, parity);
     return cudaGetLastError();
 }
 

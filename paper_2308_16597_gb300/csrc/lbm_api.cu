@@ -56,7 +56,7 @@ int validate(const lbm_domain *d, const lbm_particle *p, int32_t n, const lbm_pa
         // angle reduction by pi/2
         if (is_ellipse(P.r, P.b) && (P.b < 1.0 || P.b > P.r || std::fabs(P.theta) > 1.6e6)) return LBM_EINVAL;
         // the link kernel holds a particle's zone in shared memory
-        if (!link_zone_supported(zone_size(P.r), prm->storage)) return LBM_EINVAL;
+        if (!link_zone_supported(zone_size(P.r))) return LBM_EINVAL;
         // a disk stays inside the cavity; next to a periodic seam it keeps two
         // nodes of clearance so that no link or stencil wraps around
         const double mx = px ? 2.0 : -0.5, my = py ? 2.0 : -0.5;
@@ -103,39 +103,41 @@ void layout(const lbm_domain *d, const lbm_particle *p, int32_t n, int storage, 
     // reads up to 33 elements past the last row of the last plane
     for (int b = 0; b < 2; ++b) L.A[b] = take((size_t)kPop * L.ps * storage_bytes(storage) + kDistTailPad);
     for (int b = 0; b < 2; ++b) L.own[b] = take(nn * sizeof(int));
-    L.flags = take((size_t)L.pitch * d->ny);
+    // node bits: a row of either parity padded to whole 16-byte units
+    L.bpitch = (int)round_up((size_t)L.pitch / 32, 8);
+    L.bits = take((size_t)bits_words(L.bpitch, d->ny) * sizeof(unsigned));
     L.slot_node = take(L.nslots * sizeof(int));
     L.slot_q = take(L.nslots * sizeof(float));
     L.slot_base = take((size_t)(n + 1) * sizeof(int));
-    L.cur = take((size_t)kPartFields * n * sizeof(double));
-    L.nxt = take((size_t)kPartFields * n * sizeof(double));
-    L.prev = take((size_t)2 * n * sizeof(double));
+    for (int b = 0; b < 2; ++b) L.part[b] = take((size_t)kPartFields * n * sizeof(double));
+    for (int b = 0; b < 2; ++b) L.crowd[b] = take((size_t)n * sizeof(int));
     L.force = take((size_t)3 * n * sizeof(double));
     L.pos4 = take((size_t)n * sizeof(float4));
     L.prc = take((size_t)n * sizeof(float2));
     L.lsum = take((size_t)n * sizeof(LinkSums));
-    for (int b = 0; b < 3; ++b) L.geo[b] = take((size_t)n * sizeof(GeomRec));
+    for (int b = 0; b < 2; ++b) L.geo[b] = take((size_t)n * sizeof(GeomRec));
     L.pconst = take((size_t)n * sizeof(double4));
     L.lorder = take((size_t)n * sizeof(int));
     L.status = take(sizeof(Status));
     L.pack = take((size_t)n * sizeof(lbm_particle));
     L.stage_rows = (int)std::max<size_t>(1, std::min<size_t>(d->ny, kStageBytes / (16 * (size_t)d->nx)));
     L.stage = take((size_t)4 * L.stage_rows * d->nx * sizeof(float));
-    // newborn nodes of one step: a disk moving less than one node per step
-    // uncovers fewer than 2N nodes; room for 4N per particle
+    // nodes left in one step: a disk moving less than one node per step
+    // leaves fewer than 2N nodes; room for 4N per particle
     int zmax = 0;
     for (int a = 0; a < n; ++a) zmax = std::max(zmax, zone_size(p[a].r));
-    L.newborn_cap = std::max(1024, 4 * n * zmax);
-    L.newborn = take((size_t)L.newborn_cap * sizeof(int));
+    L.left_cap = std::max(1024, 4 * n * zmax);
+    L.left = take((size_t)L.left_cap * sizeof(int2));
     // each zone row's run of inside nodes, at the current and the next positions
     for (int b = 0; b < 2; ++b) L.runs[b] = take((size_t)n * std::max(zmax, 1) * sizeof(int2));
     L.near = take(((size_t)d->ny * near_tiles_per_row(storage, L.pitch) + 31) / 32 * sizeof(unsigned));
     L.dsum = take((size_t)n * sizeof(DirectSums));
     // cell grid of the pair screening: side 2 r_max + s + 2 (every pair in
-    // reach lies in neighbouring cells), grown to hold at most 4 Mi cells
+    // reach, or near enough to share nodes one step on, lies in neighbouring
+    // cells), grown to hold at most 4 Mi cells
     double rmax = 1.0;
     for (int a = 0; a < n; ++a) rmax = std::max(rmax, p[a].r);
-    double side = 2.0 * rmax + std::max(s_rep, 0.0) + 2.0;
+    double side = 2.0 * rmax + std::max(s_rep, 2.0) + 2.0;
     side = std::max(side, std::sqrt((double)d->nx * d->ny / (double)(1 << 22)));
     L.cell_side = side;
     L.cell_gx = n > 0 ? std::max(1, (int)std::ceil(d->nx / side)) : 1;
@@ -217,10 +219,9 @@ int timed(lbm_handle *h, int kind, cudaStream_t st, F &&launch)
 }
 
 // One time step, in the order
-//   gather + bounce-back + force (particle state at n, owner map at n; also
-//   clears the other owner map over the zones at n - 1)
+//   gather + bounce-back + force (particle state and node bits at n; also
+//   clears the other node bits over the zones at n - 1)
 //   -> particle update (n -> n+1) with the raster of the new positions
-//   -> flags at n+1
 //   -> fused stream + collide of A_n into A_{n+1}, beside the general path
 //      (frame and newborn nodes, refill).
 int enqueue_step(lbm_handle *h, int par, cudaStream_t st)
@@ -235,15 +236,15 @@ int enqueue_step(lbm_handle *h, int par, cudaStream_t st)
         // the lattice away from every particle needs nothing of this step's
         // particle work: stream-collide those tiles beside it
         if (serial) {
-            if ((rc = timed(h, kKNearMask, st, [&] { return launch_near_mask(D, st); }))) return rc;
-            if ((rc = timed(h, kKStreamCollide, st, [&] { return launch_stream_collide(D, Ain, Aout, kSCFar, st); })))
+            if ((rc = timed(h, kKNearMask, st, [&] { return launch_near_mask(D, par, st); }))) return rc;
+            if ((rc = timed(h, kKStreamCollide, st, [&] { return launch_stream_collide(D, Ain, Aout, kSCFar, par, st); })))
                 return rc;
         } else {
             CK(h, cudaEventRecord(h->fork0, st));
             CK(h, cudaStreamWaitEvent(h->far, h->fork0, 0));
-            if ((rc = timed(h, kKNearMask, h->far, [&] { return launch_near_mask(D, h->far); }))) return rc;
+            if ((rc = timed(h, kKNearMask, h->far, [&] { return launch_near_mask(D, par, h->far); }))) return rc;
             if ((rc = timed(h, kKStreamCollide, h->far,
-                            [&] { return launch_stream_collide(D, Ain, Aout, kSCFar, h->far); })))
+                            [&] { return launch_stream_collide(D, Ain, Aout, kSCFar, par, h->far); })))
                 return rc;
             CK(h, cudaEventRecord(h->join0, h->far));
         }
@@ -256,15 +257,12 @@ int enqueue_step(lbm_handle *h, int par, cudaStream_t st)
             return rc;
     }
     // particle update and raster of the new positions (one kernel)
-    if ((rc = timed(h, kKParticles, st, [&] { return launch_particles(D, par, on, st); }))) return rc;
-    if (h->np > 0) {
-        if ((rc = timed(h, kKFlags, st, [&] { return launch_flags(D, oc, on, 1, par, st); }))) return rc;
-    }
+    if (h->np > 0 && (rc = timed(h, kKParticles, st, [&] { return launch_particles(D, par, on, st); }))) return rc;
     if (overlap && !serial) CK(h, cudaStreamWaitEvent(st, h->join0, 0));
     const int kind = overlap ? kKStreamCollideNear : kKStreamCollide;
     const int mode = overlap ? kSCNear : kSCAll;
     if (serial) {
-        if ((rc = timed(h, kind, st, [&] { return launch_stream_collide(D, Ain, Aout, mode, st); }))) return rc;
+        if ((rc = timed(h, kind, st, [&] { return launch_stream_collide(D, Ain, Aout, mode, par, st); }))) return rc;
         return timed(h, kKBoundary, st, [&] { return launch_boundary(D, Ain, Aout, oc, par, st); });
     }
     // k_boundary and k_stream_collide write disjoint nodes of Aout and read
@@ -274,15 +272,15 @@ int enqueue_step(lbm_handle *h, int par, cudaStream_t st)
     if ((rc = timed(h, kKBoundary, h->side, [&] { return launch_boundary(D, Ain, Aout, oc, par, h->side); })))
         return rc;
     CK(h, cudaEventRecord(h->join, h->side));
-    if ((rc = timed(h, kind, st, [&] { return launch_stream_collide(D, Ain, Aout, mode, st); }))) return rc;
+    if ((rc = timed(h, kind, st, [&] { return launch_stream_collide(D, Ain, Aout, mode, par, st); }))) return rc;
     CK(h, cudaStreamWaitEvent(st, h->join, 0));
     return LBM_OK;
 }
 
 int kernels_per_step(const lbm_handle *h)
 {
-    if (h->np == 0) return 3;
-    return ((h->prm.flags & LBM_FLAG_OVERLAP) ? 7 : 5) + ((h->prm.flags & LBM_FLAG_DIRECT_LINKS) ? 1 : 0);
+    if (h->np == 0) return 2;
+    return ((h->prm.flags & LBM_FLAG_OVERLAP) ? 6 : 4) + ((h->prm.flags & LBM_FLAG_DIRECT_LINKS) ? 1 : 0);
 }
 
 // Graph of `steps` consecutive steps from parity par (an even count ends on
@@ -385,9 +383,10 @@ void fill_dev(lbm_handle *h)
     D.eps_w = P.eps_w;
     D.s_rep = P.s_rep;
     D.fixed = (P.flags & LBM_FLAG_FIXED_PARTICLES) ? 1 : 0;
-    D.flags = reinterpret_cast<uint8_t *>(ws + L.flags);
-    D.newborn = reinterpret_cast<int *>(ws + L.newborn);
-    D.newborn_cap = L.newborn_cap;
+    D.bits = reinterpret_cast<unsigned *>(ws + L.bits);
+    D.bpitch = L.bpitch;
+    D.left = reinterpret_cast<int2 *>(ws + L.left);
+    D.left_cap = L.left_cap;
     for (int b = 0; b < 2; ++b) D.runs[b] = reinterpret_cast<int2 *>(ws + L.runs[b]);
     D.near = reinterpret_cast<unsigned *>(ws + L.near);
     D.dsum = reinterpret_cast<DirectSums *>(ws + L.dsum);
@@ -401,19 +400,15 @@ void fill_dev(lbm_handle *h)
     D.slot_node = reinterpret_cast<int *>(ws + L.slot_node);
     D.slot_q = reinterpret_cast<float *>(ws + L.slot_q);
     D.slot_base = reinterpret_cast<int *>(ws + L.slot_base);
-    D.cur = soa_at(ws, L.cur, h->np);
-    D.nxt = soa_at(ws, L.nxt, h->np);
-    D.px = reinterpret_cast<double *>(ws + L.prev);
-    D.py = D.px + h->np;
+    for (int b = 0; b < 2; ++b) D.part[b] = soa_at(ws, L.part[b], h->np);
+    for (int b = 0; b < 2; ++b) D.crowd[b] = reinterpret_cast<int *>(ws + L.crowd[b]);
     D.force = reinterpret_cast<double *>(ws + L.force);
     D.pos4 = reinterpret_cast<float4 *>(ws + L.pos4);
     D.nslots = (long long)L.nslots;
     D.a_elems = (long long)kPop * L.ps + (long long)(kDistTailPad / storage_bytes(D.storage));
     D.prc = reinterpret_cast<float2 *>(ws + L.prc);
     D.lsum = reinterpret_cast<LinkSums *>(ws + L.lsum);
-    D.geo_prev = reinterpret_cast<GeomRec *>(ws + L.geo[0]);
-    D.geo_cur = reinterpret_cast<GeomRec *>(ws + L.geo[1]);
-    D.geo_nxt = reinterpret_cast<GeomRec *>(ws + L.geo[2]);
+    for (int b = 0; b < 2; ++b) D.geo[b] = reinterpret_cast<GeomRec *>(ws + L.geo[b]);
     D.pconst = reinterpret_cast<double4 *>(ws + L.pconst);
     D.lorder = reinterpret_cast<int *>(ws + L.lorder);
     D.status = reinterpret_cast<Status *>(ws + L.status);
@@ -440,34 +435,57 @@ int upload_particles(lbm_handle *h, const lbm_particle *p)
         for (int f = 0; f < kPartFields; ++f) soa[(size_t)f * n + a] = v[f];
     }
     const size_t bytes = soa.size() * sizeof(double);
-    CK(h, cudaMemcpyAsync(h->D.cur.x, soa.data(), bytes, cudaMemcpyHostToDevice, h->stream));
-    CK(h, cudaMemcpyAsync(h->D.nxt.x, h->D.cur.x, bytes, cudaMemcpyDeviceToDevice, h->stream));
-    CK(h, cudaMemcpyAsync(h->D.px, h->D.cur.x, 2 * n * sizeof(double), cudaMemcpyDeviceToDevice,
-                          h->stream));
+    for (int b = 0; b < 2; ++b)
+        CK(h, cudaMemcpyAsync(h->D.part[b].x, soa.data(), bytes, cudaMemcpyHostToDevice, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
     return LBM_OK;
 }
 
-int rebuild_maps(lbm_handle *h)
+// What the kernels keep of the positions beside the particle state: geometry
+// records, screening grids, link order, row runs and the owner map (whole:
+// every particle counts as crowded until it has moved); bits: the node bits
+// too.  The maps of the other parity, which the next step clears over the
+// zones one step back, hold nothing.
+int rebuild_maps(lbm_handle *h, bool bits)
 {
     const size_t nn = (size_t)h->d.nx * h->d.ny;
-    CK(h, cudaMemsetAsync(h->own[0], 0xff, nn * sizeof(int), h->stream));
-    CK(h, cudaMemsetAsync(h->own[1], 0xff, nn * sizeof(int), h->stream));
-    CK(h, cudaMemsetAsync(h->D.flags, 0, (size_t)h->L.pitch * h->d.ny, h->stream));
-    int *oc = h->own[h->parity];
+    for (int b = 0; b < 2; ++b) CK(h, cudaMemsetAsync(h->own[b], 0xff, nn * sizeof(int), h->stream));
+    if (bits) CK(h, cudaMemsetAsync(h->D.bits, 0, (size_t)bits_words(h->L.bpitch, h->d.ny) * sizeof(unsigned), h->stream));
+    if (h->np == 0) return LBM_OK;
+    CK(h, cudaMemsetAsync(h->D.crowd[h->parity ^ 1], 0, h->np * sizeof(int), h->stream));
     CK(h, launch_geom_init(h->D, h->stream));
     CK(h, launch_cells_init(h->D, h->stream));
-    CK(h, launch_link_order(h->D, h->stream));
+    CK(h, launch_link_order(h->D, h->parity, h->stream));
     h->since_order = 0;
-    CK(h, launch_raster(h->D, oc, h->D.geo_cur, h->D.cur, h->D.runs[h->parity], h->stream));
-    CK(h, launch_flags(h->D, oc, oc, 0, h->parity, h->stream));
-    // no newborn node yet
-    CK(h, cudaMemsetAsync(&h->D.status->nb, 0, sizeof(unsigned), h->stream));
-    // the owner map one step back, which the first clear expects in the other buffer
-    PartSoA prev = h->D.cur;
-    prev.x = h->D.px;
-    prev.y = h->D.py;
-    CK(h, launch_raster(h->D, h->own[h->parity ^ 1], h->D.geo_prev, prev, nullptr, h->stream));
+    CK(h, launch_raster(h->D, h->own[h->parity], bits, h->parity, h->stream));
+    return LBM_OK;
+}
+
+// The owner map of the current positions and, after it, a state image's flag
+// map, made in the distribution buffer that the next step overwrites;
+// release_maps zeroes what they took of it (its gaps between the planes hold
+// zeros).
+struct Maps {
+    int *own;
+    uint8_t *flags;
+    size_t bytes;
+};
+int make_maps(lbm_handle *h, Maps &m)
+{
+    const size_t own_b = round_up((size_t)h->d.nx * h->d.ny * sizeof(int), kAlign);
+    const size_t flag_b = (size_t)h->L.pitch * h->d.ny;
+    char *base = static_cast<char *>(h->A[h->parity ^ 1]);
+    m.own = reinterpret_cast<int *>(base);
+    m.flags = reinterpret_cast<uint8_t *>(base + own_b);
+    m.bytes = own_b + flag_b;
+    CK(h, cudaMemsetAsync(m.own, 0xff, own_b, h->stream));
+    CK(h, launch_owner(h->D, m.own, h->parity, h->stream));
+    CK(h, launch_flags_out(h->D, m.flags, h->parity, h->stream));
+    return LBM_OK;
+}
+int release_maps(lbm_handle *h, const Maps &m)
+{
+    CK(h, cudaMemsetAsync(m.own, 0, m.bytes, h->stream));
     return LBM_OK;
 }
 
@@ -553,14 +571,14 @@ int lbm_init(lbm_handle **out, const lbm_domain *d, const lbm_particle *p, int32
             return fail(LBM_ECUDA);
         if ((rc = upload_particles(h, p))) return fail(rc);
     }
-    if ((rc = rebuild_maps(h))) return fail(rc);
+    if ((rc = rebuild_maps(h, true))) return fail(rc);
     // both buffers zeroed whole (the gaps between planes, where the plane
     // stride exceeds ny x pitch, and the tail pad included), so that state
     // images hold no leftover bytes of the workspace
     const size_t abytes = (size_t)kPop * h->L.ps * storage_bytes(h->D.storage) + kDistTailPad;
     for (int b = 0; b < 2; ++b)
         if (cudaMemsetAsync(h->A[b], 0, abytes, h->stream) != cudaSuccess) return fail(LBM_ECUDA);
-    if (launch_init_collide(h->D, h->A[1], h->A[0], (float)prm->T_init, 0, h->stream) != cudaSuccess)
+    if (launch_init_collide(h->D, h->A[1], h->A[0], (float)prm->T_init, 0, h->parity, h->stream) != cudaSuccess)
         return fail(LBM_ECUDA);
     if ((rc = sync_status(h))) return fail(rc);
     *out = h;
@@ -576,7 +594,7 @@ int lbm_step(lbm_handle *h, int32_t nsteps)
     for (int32_t k = 0; k < nsteps;) {
         // the link order follows the particles every kOrderSteps steps
         if (h->since_order >= kOrderSteps) {
-            CK(h, launch_link_order(h->D, h->stream));
+            CK(h, launch_link_order(h->D, h->parity, h->stream));
             ++h->launches;
             h->since_order = 0;
         }
@@ -614,7 +632,7 @@ int lbm_get_fields(lbm_handle *h, float *rho, float *ux, float *uy, float *T, in
     const void *A = h->A[h->parity];
     const int nx = h->d.nx, ny = h->d.ny;
     if (on_device) {
-        CK(h, launch_fields(h->D, A, 0, ny, rho, ux, uy, T, h->stream));
+        CK(h, launch_fields(h->D, A, 0, ny, rho, ux, uy, T, h->parity, h->stream));
         return h->sticky;
     }
     int rc = sync_status(h);
@@ -625,7 +643,7 @@ int lbm_get_fields(lbm_handle *h, float *rho, float *ux, float *uy, float *T, in
     for (int r0 = 0; r0 < ny; r0 += R) {
         const int rows = std::min(R, ny - r0);
         const size_t cnt = (size_t)rows * nx;
-        CK(h, launch_fields(h->D, A, r0, rows, st, st + cnt, st + 2 * cnt, st + 3 * cnt, h->stream));
+        CK(h, launch_fields(h->D, A, r0, rows, st, st + cnt, st + 2 * cnt, st + 3 * cnt, h->parity, h->stream));
         for (int f = 0; f < 4; ++f)
             CK(h, cudaMemcpyAsync(outs[f] + (size_t)r0 * nx, st + f * cnt, cnt * sizeof(float),
                                   cudaMemcpyDeviceToHost, h->stream));
@@ -639,7 +657,7 @@ int lbm_get_particles(lbm_handle *h, lbm_particle *out, int32_t n)
     if (!h || n != h->np || (n > 0 && !out)) return LBM_EINVAL;
     if (n > 0) {
         lbm_particle *pk = reinterpret_cast<lbm_particle *>(h->ws + h->L.pack);
-        CK(h, launch_pack_particles(h->D, pk, h->stream));
+        CK(h, launch_pack_particles(h->D, pk, h->parity, h->stream));
         CK(h, cudaMemcpyAsync(out, pk, (size_t)n * sizeof(lbm_particle), cudaMemcpyDeviceToHost,
                               h->stream));
     }
@@ -652,7 +670,7 @@ int lbm_get_particles_async(lbm_handle *h, lbm_particle *out, int32_t n)
     if (h->sticky) return h->sticky;
     if (n > 0) {
         lbm_particle *pk = reinterpret_cast<lbm_particle *>(h->ws + h->L.pack);
-        CK(h, launch_pack_particles(h->D, pk, h->stream));
+        CK(h, launch_pack_particles(h->D, pk, h->parity, h->stream));
         CK(h, cudaMemcpyAsync(out, pk, (size_t)n * sizeof(lbm_particle), cudaMemcpyDeviceToHost,
                               h->stream));
     }
@@ -699,8 +717,11 @@ int lbm_destroy(lbm_handle *h)
 int lbm_get_owner(lbm_handle *h, int32_t *out)
 {
     if (!h || !out) return LBM_EINVAL;
-    CK(h, cudaMemcpyAsync(out, h->own[h->parity], (size_t)h->d.nx * h->d.ny * sizeof(int),
-                          cudaMemcpyDeviceToHost, h->stream));
+    Maps m;
+    int rc = make_maps(h, m);
+    if (rc) return rc;
+    CK(h, cudaMemcpyAsync(out, m.own, (size_t)h->d.nx * h->d.ny * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    if ((rc = release_maps(h, m))) return rc;
     return sync_status(h);
 }
 
@@ -743,12 +764,15 @@ int lbm_get_state(lbm_handle *h, void *buf, size_t bytes)
     if (!h || !buf || bytes < state_parts(h, sz)) return LBM_EINVAL;
     int rc = sync_status(h);
     if (rc) return rc;
-    const void *src[5] = {h->A[h->parity], h->own[h->parity], h->D.flags, h->D.cur.x, h->D.px};
+    Maps m;
+    if ((rc = make_maps(h, m))) return rc;
+    const void *src[5] = {h->A[h->parity], m.own, m.flags, h->D.part[h->parity].x, h->D.part[h->parity ^ 1].x};
     char *o = static_cast<char *>(buf);
     for (int i = 0; i < 5; ++i) {
         if (sz[i]) CK(h, cudaMemcpyAsync(o, src[i], sz[i], cudaMemcpyDeviceToHost, h->stream));
         o += sz[i];
     }
+    if ((rc = release_maps(h, m))) return rc;
     return sync_status(h);
 }
 
@@ -757,31 +781,26 @@ int lbm_set_state(lbm_handle *h, const void *buf, size_t bytes)
     size_t sz[5];
     if (!h || !buf || bytes < state_parts(h, sz)) return LBM_EINVAL;
     CK(h, cudaStreamSynchronize(h->stream));
-    void *dst[5] = {h->A[h->parity], h->own[h->parity], h->D.flags, h->D.cur.x, h->D.px};
-    const char *in = static_cast<const char *>(buf);
+    const int par = h->parity;
+    // the positions one step back go where that state lies, with the other
+    // fields of the current one (an orientation only shapes a zone that is
+    // cleared whole); the flag map through the other distribution buffer
+    uint8_t *flags = static_cast<uint8_t *>(h->A[par ^ 1]);
+    void *dst[5] = {h->A[par], nullptr, flags, h->D.part[par].x, nullptr};
+    const char *in = static_cast<const char *>(buf), *part[5];
     for (int i = 0; i < 5; ++i) {
-        if (sz[i]) CK(h, cudaMemcpyAsync(dst[i], in, sz[i], cudaMemcpyHostToDevice, h->stream));
+        if (sz[i] && dst[i]) CK(h, cudaMemcpyAsync(dst[i], in, sz[i], cudaMemcpyHostToDevice, h->stream));
+        part[i] = in;
         in += sz[i];
     }
+    CK(h, launch_flags_in(h->D, flags, par, h->stream));
+    CK(h, cudaMemsetAsync(flags, 0, sz[2], h->stream));
     if (h->np > 0) {
-        CK(h, cudaMemcpyAsync(h->D.nxt.x, h->D.cur.x, sz[3], cudaMemcpyDeviceToDevice, h->stream));
-        // owner map one step back, expected by the next clear
-        const size_t nn = (size_t)h->d.nx * h->d.ny;
-        CK(h, cudaMemsetAsync(h->own[h->parity ^ 1], 0xff, nn * sizeof(int), h->stream));
-        PartSoA prev = h->D.cur;
-        prev.x = h->D.px;
-        prev.y = h->D.py;
-        CK(h, launch_geom_init(h->D, h->stream));
-        CK(h, launch_cells_init(h->D, h->stream));
-        CK(h, launch_link_order(h->D, h->stream));
-        h->since_order = 0;
-        CK(h, launch_raster(h->D, h->own[h->parity ^ 1], h->D.geo_prev, prev, nullptr, h->stream));
-        // the row runs of the restored positions (their raster rewrites the
-        // restored owner map with the values it holds), and the newborn
-        // list of the restored flags, which the next step returns to fluid
-        CK(h, launch_raster(h->D, h->own[h->parity], h->D.geo_cur, h->D.cur, h->D.runs[h->parity], h->stream));
-        CK(h, cudaMemsetAsync(&h->D.status->nb, 0, sizeof(unsigned), h->stream));
-        CK(h, launch_collect_newborn(h->D, h->stream));
+        CK(h, cudaMemcpyAsync(h->D.part[par ^ 1].x, h->D.part[par].x, sz[3], cudaMemcpyDeviceToDevice, h->stream));
+        CK(h, cudaMemcpyAsync(h->D.part[par ^ 1].x, part[4], sz[4], cudaMemcpyHostToDevice, h->stream));
+        int rc = rebuild_maps(h, false);
+        if (rc) return rc;
+        CK(h, cudaMemcpyAsync(h->own[par], part[1], sz[1], cudaMemcpyHostToDevice, h->stream));
     }
     return sync_status(h);
 }
@@ -812,7 +831,7 @@ int lbm_set_distributions(lbm_handle *h, const double *f, const double *g)
             }
     void *scratch = h->A[h->parity ^ 1];
     CK(h, cudaMemcpyAsync(scratch, img.data(), img.size(), cudaMemcpyHostToDevice, h->stream));
-    CK(h, launch_init_collide(h->D, scratch, h->A[h->parity], 0.f, 1, h->stream));
+    CK(h, launch_init_collide(h->D, scratch, h->A[h->parity], 0.f, 1, h->parity, h->stream));
     return sync_status(h);
 }
 

@@ -56,8 +56,8 @@ struct lbm_batch {
     unsigned *d_counter = nullptr; // [2] the staged kernel's work counter and done count
     int sc_shift = 0;
     int total[kBatchPhases] = {};
-    int tile = 0, sc_resident = 1, links_ahead = 1;
-    size_t links_smem = 0;
+    int tile = 0, sc_resident = 1;
+    LinkPlan links;
     cudaGraphExec_t gexec[4][2] = {}; // 2^l steps (l = 0..3) from each parity
     long long launches = 0;
     int sticky = LBM_OK;
@@ -140,18 +140,18 @@ cudaError_t launch_sc(const lbm_batch *b, int par, cudaStream_t st)
 }
 
 // One step of every instance, in the order of lbm_step: links -> particles
-// (and raster) -> flags -> stream-collide beside the general path.
+// (and raster) -> stream-collide beside the general path (the first and last
+// rows, and the refilling).
 int enqueue_batch_step(lbm_batch *b, int par, cudaStream_t st)
 {
     const InstArgs *I = b->d_inst;
     const int n = b->n;
-    BCK(b, launch_links_batch(I, starts(b, kBLinks), n, b->total[kBLinks], b->storage, par, b->links_ahead,
-                              b->links_smem, st));
+    BCK(b, launch_links_batch(I, starts(b, kBLinks), n, b->total[kBLinks], b->storage, par, b->links, st));
     BCK(b, launch_particles_batch(I, starts(b, kBParticles), n, b->total[kBParticles], par, st));
-    BCK(b, launch_flags_batch(I, starts(b, kBFlags), n, b->total[kBFlags], par, st));
     BCK(b, cudaEventRecord(b->fork, st));
     BCK(b, cudaStreamWaitEvent(b->side, b->fork, 0));
-    BCK(b, launch_boundary_batch(I, starts(b, kBBoundary), n, b->total[kBBoundary], b->storage, par, b->side));
+    BCK(b, launch_boundary_batch(I, starts(b, kBBoundary), n, b->total[kBBoundary], b->storage, par, false, b->side));
+    BCK(b, launch_boundary_batch(I, starts(b, kBRefill), n, b->total[kBRefill], b->storage, par, true, b->side));
     BCK(b, cudaEventRecord(b->join, b->side));
     BCK(b, launch_sc(b, par, st));
     BCK(b, cudaStreamWaitEvent(st, b->join, 0));
@@ -250,13 +250,13 @@ int lbm_batch_create(lbm_batch **out, lbm_handle *const *hs, int32_t n, void *d_
         lbm_handle *h = hs[i];
         // every handle's own work must be complete before the batch runs
         if (cudaStreamSynchronize(h->stream) != cudaSuccess) return fail(LBM_ECUDA);
+        inst[i] = InstArgs{};
         inst[i].D = h->D;
         inst[i].A[0] = h->A[0];
         inst[i].A[1] = h->A[1];
         inst[i].own[0] = h->own[0];
         inst[i].own[1] = h->own[1];
         inst[i].poff = h->parity;
-        inst[i].pad = 0;
         b->poff[i] = h->parity;
         b->zone_max = std::max(b->zone_max, h->D.zone_max);
     }
@@ -269,8 +269,9 @@ int lbm_batch_create(lbm_batch **out, lbm_handle *const *hs, int32_t n, void *d_
             cudaSuccess ||
         cudaMemsetAsync(b->d_counter, 0, 2 * sizeof(unsigned), b->stream) != cudaSuccess)
         return fail(LBM_ECUDA);
-    if (prepare_links_batch(std::max(b->zone_max, 4), b->storage, &b->links_smem, &b->links_ahead) !=
-        cudaSuccess)
+    int np = 0;
+    for (int i = 0; i < n; ++i) np += hs[i]->np;
+    if (prepare_links_batch(std::max(b->zone_max, 4), np, b->storage, &b->links) != cudaSuccess)
         return fail(LBM_ECUDA);
     if ((rc = upload_starts(b))) return fail(rc);
     *out = b;
@@ -326,7 +327,7 @@ int lbm_batch_step(lbm_batch *b, int32_t nsteps)
     for (int i = 0; i < b->n; ++i)
         if (b->hs[i]->parity != (b->parity ^ b->poff[i])) return LBM_EINVAL; // a handle was stepped on its own
     int per_step = 0;
-    for (int ph = 0; ph < kBatchPhases; ++ph) per_step += ph != kBRaster && b->total[ph] > 0;
+    for (int ph = 0; ph < kBatchPhases; ++ph) per_step += b->total[ph] > 0;
     for (int32_t k = 0; k < nsteps;) {
         // the largest graph (8, 4, 2 or 1 steps) that fits what is left
         int l = 3;

@@ -73,7 +73,7 @@ enum { kScC1 = 0, kScC2, kScB4, kScB7, kScC7, kScC8, kScG2, kScThree, kScBfx, kN
 // Bytes per stored population.
 __host__ __device__ constexpr int storage_bytes(int storage) { return storage == LBM_STORE_FP32 ? 4 : 2; }
 
-// Per-node state bytes of the flag map.
+// Node classes of a state image's flag map (see solid_at).
 constexpr uint8_t kFluid = 0;   // fluid at the previous and the current time
 constexpr uint8_t kSolid = 1;   // inside a particle at the current time
 constexpr uint8_t kNewborn = 2; // uncovered by a particle during the last step
@@ -93,7 +93,7 @@ struct Status {
     unsigned int err;
     unsigned int pad;
     unsigned long long cnt[2][kNumCounters]; // double-buffered by step parity
-    unsigned int nb;     // newborn nodes listed this step (reset by the particle update)
+    unsigned int nb;     // nodes the particles left this step (reset by the link kernel)
     unsigned int nb_pad;
     // the staged stream-collide's work counter (next row tile to claim) and
     // the count of its blocks done; the last block done resets both to 0
@@ -127,11 +127,15 @@ struct Dev {
     int fixed;
     int zone_max;      // largest zone side N over the particles (sizes the link kernel's tile)
     int link_ahead;    // link-kernel CTAs resident on the GPU (distance of its L2 prefetch)
-    int flag_team;     // warps per particle in the flags kernel (1, 2 or 4)
-    // device buffers
-    uint8_t *flags;    // [ny][pitch]
-    int *newborn;      // [newborn_cap]: this step's newborn nodes, j * nx + i off the cavity frame, ~(j * nx + i) on it
-    int newborn_cap;
+    int link_team;     // its warps per particle
+    // device buffers.  What a step reads and writes of the particles and of
+    // the nodes they hold lies in pairs by step parity: with par that of the
+    // step, [par] is the state it starts from and [par ^ 1] that one step
+    // back, which the step replaces by the state it ends with.
+    unsigned *bits;    // [ny][bpitch][2]: bit x % 32 of word x / 32 of either parity: node (x, y) lies in a particle
+    int bpitch;        // words per row and parity (a multiple of 8: a row tile's words are whole 16-byte units)
+    int2 *left;        // [left_cap]: the nodes particles left this step: (j * nx + i, particle)
+    int left_cap;
     int2 *runs[2];     // [np][zone_max] by step parity: each zone row's run (lo, hi) of nodes inside the particle
     unsigned *near;    // bit per warp tile (row, 32 V nodes) within reach of a particle this step
     int near_tpr;      // warp tiles per row of that bitmap
@@ -140,8 +144,12 @@ struct Dev {
     int *slot_node;    // [nslots]
     float *slot_q;     // [nslots]
     int *slot_base;    // [np + 1]
-    PartSoA cur, nxt;  // state at n (and n+1 after the raster rotation) / new state
-    double *px, *py;   // positions one step back (boxes to clear)
+    PartSoA part[2];   // particle states by parity
+    // [np] by parity: whether the particle may share nodes with another
+    // (centres within reach of the radii when it moved there).  The owner
+    // maps hold the nodes of these particles only; those of any other are
+    // its row runs.
+    int *crowd[2];
     double *force;     // [3 np]: hydrodynamic Fx, Fy, Tz of the last step
     float4 *pos4;      // [np]: centre as double-float (xh, yh, xl, yl) at the start of the step
     float2 *prc;       // [np]: (GeomRec r, C) in FP32 for the pair screening (r < 0: an ellipse)
@@ -150,7 +158,7 @@ struct Dev {
     int direct;            // links found by the node-parallel scan instead of the index array
     int sc_staged;         // whole-lattice stream-collide through the staged kernel (else one block per tile)
     int sc_extra_tx;       // bytes the staged kernel announces beyond its copies (tests of its bounded waits)
-    struct GeomRec *geo_prev, *geo_cur, *geo_nxt; // [np] each: FP32/int geometry of the three positions
+    struct GeomRec *geo[2]; // [np] by parity: FP32/int geometry of the positions
     double4 *pconst;   // [np]: constants of the update (1/M, 1/I, weight W, repulsion scale C)
     int *lorder;       // [np]: the link kernel's CTA order (particles by descending y)
     // pair screening: a grid of square cells of side 1 / cell_inv >= 2 r_max
@@ -195,6 +203,23 @@ __device__ __forceinline__ int cell_of(const Dev &D, float xh, float yh)
 __device__ __forceinline__ long long fix_of(float v) { return __float2ll_rn(v * 0x1p40f); }
 __device__ __forceinline__ long long fix_of(double v) { return __double2ll_rn(v * 0x1p40); }
 __device__ __forceinline__ double fix_value(long long v) { return (double)v * 0x1p-40; }
+
+// The word of the node bits that holds node (x, y) at a parity, and whether a
+// particle holds the node.  (Two bits per node took the place of a flag byte
+// and, but for crowded particles, of the owner map in the step's kernels:
+// at 4000^2 / 4800 disks the kernels that write and read them, see k_links.)
+// A node is solid where the bit of the current time is set, newborn where
+// only that of the time before is, else fluid.
+__device__ __forceinline__ long long bit_word(const Dev &D, int x, int y, int par)
+{
+    return ((long long)y * D.bpitch + (x >> 5)) * 2 + par;
+}
+__device__ __forceinline__ bool solid_at(const Dev &D, int x, int y, int par)
+{
+    return (D.bits[bit_word(D, x, y, par)] >> (x & 31)) & 1u;
+}
+// Words of the node bits.
+__host__ __device__ inline long long bits_words(int bpitch, int ny) { return (long long)ny * bpitch * 2; }
 
 // ---------------------------------------------------------------------------
 // Exact FP64 geometry shared by raster, gather and refill.  Every operation is
@@ -407,7 +432,10 @@ __device__ __forceinline__ void disk_gap2_df(int i, int j, const DiskDF &D, floa
     two_prod(dyh, dyh, p2, e2);
     two_sum(p1, p2, s, es);
     two_sum(s, -D.r2h, t, et);
-    low = ((e1 + e2) + (es + et)) - D.r2l + 2.f * (dxh * dxl + dyh * dyl) + (dxl * dxl + dyl * dyl);
+    // (the sums of two products fused one way, written out: every kernel that
+    // inlines this rounds alike)
+    const float cross = fmaf(dyh, dyl, __fmul_rn(dxh, dxl)), low2 = fmaf(dyl, dyl, __fmul_rn(dxl, dxl));
+    low = ((e1 + e2) + (es + et)) - D.r2l + 2.f * cross + low2;
 }
 // The same, rounded to FP32.
 __device__ __forceinline__ float disk_gap2(int i, int j, const DiskDF &D, float &dxh, float &dxl,
@@ -585,6 +613,19 @@ struct DirectSums {
 // the variable part of Eq. force / Eq. torque of a link; k its direction;
 // lvl its Bouzidi fallback level; half whether its thermal rule fell back to
 // half-way; tz the torque moment i e_k,y - j e_k,x of its constant part.
+
+// Sum over the warp, modulo 2^64, on every lane: three limbs of 22, 22 and 20
+// bits, each summed by one warp reduction (sums below 2^27), instead of five
+// rounds of two shuffles and a 64-bit addition.
+__device__ __forceinline__ long long warp_sum64(long long v)
+{
+    const unsigned F = 0xffffffffu;
+    const unsigned l0 = __reduce_add_sync(F, (unsigned)v & 0x3fffffu);
+    const unsigned l1 = __reduce_add_sync(F, (unsigned)(v >> 22) & 0x3fffffu);
+    const int l2 = __reduce_add_sync(F, (int)(v >> 44));
+    return (long long)((unsigned long long)l0 + ((unsigned long long)l1 << 22) + ((unsigned long long)(long long)l2 << 44));
+}
+
 struct LinkAcc {
     long long fx = 0, fy = 0, tq = 0;
     int axx = 0, axy = 0, axt = 0, dgx = 0, dgy = 0, dgt = 0, cl = 0, cs = 0, ct = 0;
@@ -605,13 +646,7 @@ struct LinkAcc {
     __device__ __forceinline__ void finish(LinkSums &S, int *cnt3)
     {
         const unsigned F = 0xffffffffu;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            fx += __shfl_xor_sync(F, fx, o);
-            fy += __shfl_xor_sync(F, fy, o);
-            tq += __shfl_xor_sync(F, tq, o);
-        }
-        S.fx = fx; S.fy = fy; S.tz = tq;
+        S.fx = warp_sum64(fx); S.fy = warp_sum64(fy); S.tz = warp_sum64(tq);
         S.ax_x = (int)__reduce_add_sync(F, (unsigned)axx);
         S.ax_y = (int)__reduce_add_sync(F, (unsigned)axy);
         S.ax_t = (int)__reduce_add_sync(F, (unsigned)axt);
@@ -812,13 +847,15 @@ __device__ __forceinline__ void copy_dev(Dev &dst, const Dev &src)
         reinterpret_cast<int *>(&dst)[w] = __ldg(reinterpret_cast<const int *>(&src) + w);
     __syncthreads();
 }
-// Per-instance arguments of the batched kernels (device table).
+// Per-instance arguments of the batched kernels (device table; padded to
+// whole 16-byte units, since a bulk copy takes it).
+constexpr int kInstPad = (16 - (sizeof(Dev) + 4 * sizeof(void *) + sizeof(int)) % 16) % 16 / 4 + 4;
 struct InstArgs {
     Dev D;
     void *A[2];   // distribution buffers by step parity
     int *own[2];  // owner maps by step parity
     int poff;     // the instance's step parity = the batch's parity ^ poff
-    int pad;
+    int pad[kInstPad];
 };
 
 // Stream-collide blocks of one instance in a batched launch: its first
@@ -864,12 +901,12 @@ enum SCMode { kSCAll = 0, kSCFar = 1, kSCNear = 2 };
 constexpr int kNearMargin = 2;
 
 // Planes are passed untyped: their element type is D.storage.
-cudaError_t launch_stream_collide(const Dev &D, const void *Ain, void *Aout, int mode, cudaStream_t s);
+cudaError_t launch_stream_collide(const Dev &D, const void *Ain, void *Aout, int mode, int parity, cudaStream_t s);
 // Binary (SASS) architecture of the loaded stream-collide kernel, as
 // cudaFuncGetAttributes reports it (major * 10 + minor).
 cudaError_t stream_collide_binary_version(int *version);
 // Near-tile bitmap of this step (clears it first).
-cudaError_t launch_near_mask(const Dev &D, cudaStream_t s);
+cudaError_t launch_near_mask(const Dev &D, int parity, cudaStream_t s);
 // Direct addressing (the paper's comparison for its index array): a per-
 // particle preparation (owner-map clear, centres, zeroed sums) and one thread
 // per lattice node testing its eight neighbours.
@@ -878,63 +915,71 @@ cudaError_t launch_links_direct(const Dev &D, void *A, const int *own_cur, int *
 // Warp tiles per row of the near-tile bitmap for a storage and pitch.
 int near_tiles_per_row(int storage, int pitch);
 // Nodes the stream-collide kernel leaves to the general path: the first and
-// last rows (y = 0, ny - 1) and the listed newborn nodes.
+// last rows (y = 0, ny - 1) and the newborn nodes among those the particles
+// left.
 cudaError_t launch_boundary(const Dev &D, const void *Ain, void *Aout, const int *own_cur, int parity,
                             cudaStream_t s);
 // mode 0: fluid at rest (unit density, T_init) then collide; mode 1: collide
 // the pre-collision values read from Ain at each node.
-cudaError_t launch_init_collide(const Dev &D, const void *Ain, void *Aout, float T_init, int mode,
+// (parity: of the step the state precedes, here and in launch_fields).
+cudaError_t launch_init_collide(const Dev &D, const void *Ain, void *Aout, float T_init, int mode, int parity,
                                 cudaStream_t s);
 cudaError_t launch_fields(const Dev &D, const void *A, int row0, int rows, float *rho, float *ux,
-                          float *uy, float *T, cudaStream_t s);
+                          float *uy, float *T, int parity, cudaStream_t s);
 cudaError_t launch_links(const Dev &D, void *A, const int *own_cur, int *own_nxt, int parity,
                          cudaStream_t s);
 // Shared memory of the link kernel for zones of side N; prepare_links sets the
 // kernel's shared-memory limit and D.link_ahead (call outside stream capture).
-size_t link_smem_bytes(int N, int storage);
-// Whether the link kernel holds a zone of side N (tile rows of at most 64
-// columns, shared memory within 200 KB).
-bool link_zone_supported(int N, int storage);
+size_t link_smem_bytes(int N);
+// Whether the link kernel holds a zone of side N (window rows of at most 64
+// columns).
+bool link_zone_supported(int N);
 cudaError_t prepare_links(Dev &D);
-// Particle update, then the raster of the new positions into own_nxt.
+// Particle update, then the raster of the new positions.
 cudaError_t launch_particles(const Dev &D, int parity, int *own_nxt, cudaStream_t s);
-// runs (may be null): where each particle's zone-row runs go, for the flags
-// of the next step.
-cudaError_t launch_raster(const Dev &D, int *own, const struct GeomRec *geo, const PartSoA &pos, int2 *runs,
-                          cudaStream_t s);
-// rotate == 0: the flags of one position from scratch; rotate == 1: a step's
-// flags from the row runs of parity (current) and parity ^ 1 (new).
-cudaError_t launch_flags(const Dev &D, const int *own_cur, const int *own_nxt, int rotate, int parity,
-                         cudaStream_t s);
-// The newborn list of a restored state, from its flags (the list is empty).
-cudaError_t launch_collect_newborn(const Dev &D, cudaStream_t s);
-cudaError_t launch_pack_particles(const Dev &D, lbm_particle *out, cudaStream_t s);
-// Geometry records of the current state (into cur, nxt and prev) and of the
-// previous positions (into prev), for init and restore.
+// Raster of the positions of a parity into its row runs and cleared node bits
+// (bits) and owner map (own; every particle marked crowded); either may be
+// left out.
+cudaError_t launch_raster(const Dev &D, int *own, bool bits, int parity, cudaStream_t s);
+// The whole owner map (own: -1 everywhere before) of the positions of a parity.
+cudaError_t launch_owner(const Dev &D, int *own, int parity, cudaStream_t s);
+// A state image's flag map [ny][pitch] from the node bits before a step of
+// `parity`, and back.
+cudaError_t launch_flags_out(const Dev &D, uint8_t *flags, int parity, cudaStream_t s);
+cudaError_t launch_flags_in(const Dev &D, const uint8_t *flags, int parity, cudaStream_t s);
+cudaError_t launch_pack_particles(const Dev &D, lbm_particle *out, int parity, cudaStream_t s);
+// Geometry records of both parities' positions and the constants of the
+// update, for init and restore.
 cudaError_t launch_geom_init(const Dev &D, cudaStream_t s);
 // Screening grids: both cleared (the first step's link kernel enters the
 // current positions).
 cudaError_t launch_cells_init(const Dev &D, cudaStream_t s);
 // The link kernel's CTA order from the current positions (descending y).
-cudaError_t launch_link_order(const Dev &D, cudaStream_t s);
+cudaError_t launch_link_order(const Dev &D, int parity, cudaStream_t s);
 
 // Batched step kernels over an InstArgs table (one grid over all instances;
 // `start` holds the n + 1 block offsets of the launch, `total` its blocks).
-enum BatchPhase { kBLinks = 0, kBParticles, kBRaster, kBFlags, kBStream, kBBoundary, kBatchPhases };
+enum BatchPhase { kBLinks = 0, kBParticles, kBRefill, kBStream, kBBoundary, kBatchPhases };
 constexpr int kBoundaryBlocksPerInstance = 8;
+// The link kernel of a batch: warps per particle, its shared memory and the
+// distance of its prefetch.
+struct LinkPlan {
+    int team = 4, ahead = 1;
+    size_t smem = 0;
+};
 void batch_blocks(const Dev &D, dim3 sc_block, int out[kBatchPhases]);
-cudaError_t prepare_links_batch(int zone_max, int storage, size_t *smem, int *ahead);
+cudaError_t prepare_links_batch(int zone_max, int np, int storage, LinkPlan *plan);
 cudaError_t launch_links_batch(const InstArgs *I, const int *start, int n, int total, int storage, int parity,
-                               int ahead, size_t smem, cudaStream_t s);
+                               const LinkPlan &plan, cudaStream_t s);
 cudaError_t launch_particles_batch(const InstArgs *I, const int *start, int n, int total, int parity,
                                    cudaStream_t s);
-cudaError_t launch_raster_batch(const InstArgs *I, const int *start, int n, int total, int parity, cudaStream_t s);
-cudaError_t launch_flags_batch(const InstArgs *I, const int *start, int n, int total, int parity, cudaStream_t s);
 cudaError_t launch_stream_collide_batch(const InstArgs *I, const ScInst *sc, const int *bucket, int shift, int n,
                                         int total, int storage, int parity, dim3 block, int resident,
                                         cudaStream_t s);
+// The general path over a batch: first and last rows, or (refill) the nodes
+// the particles left.
 cudaError_t launch_boundary_batch(const InstArgs *I, const int *start, int n, int total, int storage, int parity,
-                                  cudaStream_t s);
+                                  bool refill, cudaStream_t s);
 int stream_collide_batch_resident(int storage, dim3 block);
 // The staged stream-collide over a batch (BF16 / FP16 storage): sc and
 // bucket built for the 128 x 1 tile shape; counter: two zeroed words of
