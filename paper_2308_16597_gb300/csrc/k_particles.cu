@@ -24,7 +24,6 @@ namespace lbm {
 namespace {
 
 constexpr int kBoxThreads = 128;
-constexpr int kPartThreads = 256;
 constexpr double kPi = 3.14159265358979323846;
 
 __device__ __forceinline__ bool inside(const Dev &D, int i, int j)
@@ -52,7 +51,7 @@ __host__ __device__ inline int link_tile_wx(int N) { return N + 4; }
 // Shared memory of a CTA: its record, the fluid and owner row masks [wy] (u64
 // each) and the list of links (at most one per slot).
 struct alignas(16) LinkTeam {
-    EllFrame ell;  // an ellipse's FP64 frame
+    EllLink ell;   // an ellipse's FP64 frame
     int n;         // links found
     unsigned over; // a line with two links
 };
@@ -247,10 +246,10 @@ __device__ __forceinline__ void links_body(const Dev &D, T *A, const int *__rest
     if (tid == kThreads - 1) {
         D.pos4[p] = make_float4(Gp->xh, Gp->yh, Gp->xl, Gp->yl);
         D.prc[p] = make_float2(Gp->r, Gp->C);
-        if (Gp->r < 0.f) {
-            const PartSoA &P = D.part[parity];
-            S.ell = ell_frame(P.x[p], P.y[p], P.th[p], P.r[p], P.b[p]);
-        }
+    }
+    if (warp == kTeam - 1 && lane < 8 && Gp->r < 0.f) {
+        const PartSoA &P = D.part[parity];
+        ell_link_entry(S.ell, lane, ell_frame_cs(P.x[p], P.y[p], D.cs[parity][p], P.r[p], P.b[p]));
     }
     // L2 prefetch of the bit rows of particle pa, the one a residency wave
     // later in launch order (none: pa < 0)
@@ -462,32 +461,41 @@ __device__ __forceinline__ double repulsion(double gap, double s, double eps, do
 // Total force = hydrodynamic (assembled from the link sums) + buoyant weight
 // -(rho_p - rho_f) pi r^2 g y-hat + repulsion (walls, and every other disk
 // with C_ab the mean of the two force scales C = pi r^2 (rho_p - rho_f) g).
-// Each block takes 8 particles: warp w screens particle w against the
+// Each block takes kPB particles: warp w screens particle w against the
 // particles listed in the 3 x 3 cells of the screening grid around its cell
 // (filled with the step's starting positions by the link kernel; every
 // pair in reach is among them), or, when a cell of that grid overflowed,
-// against all particles in shared-memory tiles of 1600, and evaluates the
+// against all particles in shared-memory tiles of kPartTile, and evaluates the
 // pairs in reach from double-float centre differences, summed in 64-bit
 // fixed point so that the result is the same whichever way the pairs were
 // found and in whatever order; lane l of warp 0 then sums, integrates and
 // stores particle l in FP64 (its constants 1/M, 1/I, W and C, and its
 // geometry record, staged by the last warp while the others screen), and
-// warp w rasters particle w.  Small
-// blocks let four of them share an SM, so that the latency of one block's
-// loads and FP64 tail overlaps the others' work.  Integration:
+// warp w rasters particle w.  Integration:
 // U' = U + F/M, X' = X + (U + U')/2, Omega' = Omega + T/I,
 // theta' = theta + (Omega + Omega')/2 with M = rho_p pi r^2 and I = M r^2 / 2
 // (M = rho_p pi r b and I = M (r^2 + b^2) / 4 for an ellipse).
-constexpr int kPartTile = 1600;
-constexpr int kPartPerBlock = kPartThreads / 32;
+//
+// Bound by the latency of the chain (screening, FP64 tail, raster) and by the
+// SM's FP64 pipe (2 lanes a clock), so kPB is the smallest of 1, 2, 4, 8 that
+// gives each SM one block: few particles spread over all SMs, many share a
+// tail (one warp's FP64 instructions serve kPB particles).  No thread divides
+// in FP64 for a constant, cos and sin of an orientation are kept with the
+// state, an ellipse's supports are worked out at walls only, and the tail's
+// inputs are copied asynchronously.  Update, us (CUDA events), before / after:
+// 129 ellipses 37.1 / 19.7, 6 ellipses 22.9 / 14.7, 8 disks 13.0 / 12.5, 4800
+// disks 19.2 / 15.8 (with kPB = 4 there 16.9, 16: 22, 32: 29).
+constexpr int kPartTile = 512;
+constexpr int kPartMax = 8;
+constexpr int part_ctas(int pb) { return 32 / pb > 16 ? 16 : 32 / pb; } // 64 registers a thread
 
 // Support distance of particle p along the unit vector (nx, ny): its radius
 // for a disk.
-__device__ __forceinline__ double support_of(const PartSoA &P, int p, double nx, double ny)
+__device__ __forceinline__ double support_of(const Dev &D, int parity, int p, double nx, double ny)
 {
-    const double r = P.r[p], b = P.b[p];
+    const double r = D.part[parity].r[p], b = D.part[parity].b[p];
     if (!is_ellipse(r, b)) return r;
-    return ell_support(ell_frame(0.0, 0.0, P.th[p], r, b), nx, ny);
+    return ell_support(ell_frame_cs(0.0, 0.0, D.cs[parity][p], r, b), nx, ny);
 }
 
 // Pair repulsion on particle a from particle b when either is an ellipse, in
@@ -498,7 +506,8 @@ __device__ __noinline__ void pair_force_ellipse(const Dev &D, int parity, int a,
     const PartSoA &P = D.part[parity];
     const double dx = P.x[a] - P.x[b], dy = P.y[a] - P.y[b];
     const double dist = sqrt(dx * dx + dy * dy);
-    const double gap = dist - support_of(P, a, -dx / dist, -dy / dist) - support_of(P, b, dx / dist, dy / dist);
+    const double gap = dist - support_of(D, parity, a, -dx / dist, -dy / dist) -
+                       support_of(D, parity, b, dx / dist, dy / dist);
     if (gap > D.s_rep) return;
     auto scale = [&](int p) {
         const double r = P.r[p], pb = P.b[p];
@@ -574,7 +583,7 @@ __device__ __forceinline__ void write_runs(const Dev &D, int *own, const Box &B,
 // estimated from the quadratic's roots (FP32) and settled with the predicate
 // at the ends only: FP32 outside the rounding band, the exact FP64 form
 // inside it.
-__device__ __noinline__ void ellipse_run(const Dev &D, const Box B, const GeomRec G, double x, double y, double th,
+__device__ __noinline__ void ellipse_run(const Dev &D, const Box B, const GeomRec G, double x, double y, double2 cs,
                                          double r, double pb, int j, int &lo_out, int &hi_out)
 {
     lo_out = 1;
@@ -585,7 +594,7 @@ __device__ __noinline__ void ellipse_run(const Dev &D, const Box B, const GeomRe
     auto inside = [&](int i) -> bool {
         const int side = ell_side_df(i, j, F);
         if (side) return side < 0;
-        return in_ellipse(i, j, ell_frame(x, y, th, r, pb));
+        return in_ellipse(i, j, ell_frame_cs(x, y, cs, r, pb));
     };
     const float c = F.c, s = F.s;
     const float A2 = c * c * F.b2 + s * s * F.a2; // dx^2 coefficient
@@ -657,7 +666,7 @@ __device__ __forceinline__ void run_minus(int lo, int hi, int xlo, int xhi, F &&
 // its old nodes lie in the rows of its new zone): the nodes it left are
 // listed for the refilling.
 __device__ __forceinline__ void raster_one(const Dev &D, int par, int *own, const GeomRec &G, double x, double y,
-                                           double r, double th, double pb, int p, bool bits, const int2 *old,
+                                           double r, double2 cs, double pb, int p, bool bits, const int2 *old,
                                            int Y0_old)
 {
     const int lane = threadIdx.x & 31;
@@ -667,7 +676,7 @@ __device__ __forceinline__ void raster_one(const Dev &D, int par, int *own, cons
         const int j = B.Y0 + b0 + lane;
         int lo = 1, hi = 0;
         if (b0 + lane < B.N) {
-            if (G.r < 0.f) ellipse_run(D, B, G, x, y, th, r, pb, j, lo, hi);
+            if (G.r < 0.f) ellipse_run(D, B, G, x, y, cs, r, pb, j, lo, hi);
             else disk_run(D, B, G, x, y, r, j, lo, hi);
             if (in_bounds(D, (long long)p * D.zone_max + b0 + lane, (long long)D.np * D.zone_max))
                 runs[b0 + lane] = make_int2(lo, hi);
@@ -693,17 +702,28 @@ __device__ __forceinline__ void raster_one(const Dev &D, int par, int *own, cons
 
 // Support distances of an ellipse along the wall normals x-hat and y-hat
 // (kept out of line: the disk path does not carry its registers).
-__device__ __noinline__ void wall_supports(double th, double r, double b, double &hx, double &hy)
+__device__ __noinline__ void wall_supports(double2 cs, double r, double b, double &hx, double &hy)
 {
-    const EllFrame E = ell_frame(0.0, 0.0, th, r, b);
+    const EllFrame E = ell_frame_cs(0.0, 0.0, cs, r, b);
     hx = ell_support(E, 1.0, 0.0);
     hy = ell_support(E, 0.0, 1.0);
+}
+
+// Asynchronous copy of kBytes (8 or 16, both addresses aligned to it) into
+// shared memory.
+template <int kBytes>
+__device__ __forceinline__ void copy_async(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src),
+                 "n"(kBytes)
+                 : "memory");
 }
 
 // New state of a particle as the raster needs it.
 struct RasterIn {
     GeomRec G;
-    double x, y, r, th, b;
+    double x, y, r, b;
+    double2 cs; // cos and sin of theta (an ellipse)
 };
 
 // Constants of the update of a particle (they depend only on its shape and
@@ -754,14 +774,18 @@ __device__ __forceinline__ void particle_tail(const Dev &D, int b, int parity, l
     const double Cb = pk.w;
     Fy -= pk.z;
     double hx = r, hy = r;
-    if (ell) wall_supports(th, r, pb, hx, hy);
     // A wall gap takes the FP64 repulsion only where the FP32 centre of the
     // current geometry record puts it within the threshold plus a margin
     // (mar) far above that centre's rounding error (half an FP32 spacing,
     // 2.4e-4 at 4096): elsewhere the repulsion is zero either way, and GB300
     // runs FP64 at a small fraction of its FP32 rate.
-    const float mar = 1e-3f + 2.4e-7f * (float)(D.nx + D.ny), near = (float)D.s_rep + mar;
-    const float hxf = (float)hx, hyf = (float)hy, nxf = (float)D.nx, nyf = (float)D.ny;
+    const float mar = 1e-3f + 2.4e-7f * (float)(D.nx + D.ny), near = D.s_repf + mar;
+    const float rf0 = (float)r, nxf = (float)D.nx, nyf = (float)D.ny;
+    // an ellipse reaches at most r along a wall normal: its support distances
+    // are worked out where that may be within the threshold
+    if (ell && (fminf(Gc.xh, nxf - 1.f - Gc.xh) + 0.5f - rf0 <= near || fminf(Gc.yh, nyf - 1.f - Gc.yh) + 0.5f - rf0 <= near))
+        wall_supports(D.cs[parity][b], r, pb, hx, hy);
+    const float hxf = (float)hx, hyf = (float)hy;
     if (!D.per_x) {
         if ((Gc.xh + 0.5f) - hxf <= near) Fx += repulsion((x + 0.5) - hx, D.s_rep, D.eps_w, Cb);
         if ((nxf - 0.5f - Gc.xh) - hxf <= near) Fx -= repulsion(((double)D.nx - 0.5 - x) - hx, D.s_rep, D.eps_w, Cb);
@@ -801,14 +825,21 @@ __device__ __forceinline__ void particle_tail(const Dev &D, int b, int parity, l
     // (both parities hold r, rho, T and b)
     const PartSoA &nxt = D.part[parity ^ 1];
     nxt.x[b] = x; nxt.y[b] = y; nxt.ux[b] = ux; nxt.uy[b] = uy; nxt.th[b] = th; nxt.om[b] = om;
-    const GeomRec Gn = move_geom(Gc, x, y, r, pb, th, ux, uy, om);
+    double2 cs = make_double2(1.0, 0.0);
+    if (ell) {
+        cos_sin_rn(th, cs.x, cs.y);
+        D.cs[parity ^ 1][b] = cs;
+    }
+    const GeomRec Gn = move_geom(Gc, x, y, r, ell, cs, ux, uy, om);
     D.geo[parity ^ 1][b] = Gn;
     out.G = Gn;
-    out.x = x; out.y = y; out.r = r; out.th = th; out.b = pb;
+    out.x = x; out.y = y; out.r = r; out.cs = cs; out.b = pb;
 }
 
+template <int kPB>
 __device__ __forceinline__ void particles_body(const Dev &D, int parity, int *own_nxt, const int blk)
 {
+    constexpr int kPartPerBlock = kPB, kPartThreads = 32 * kPB;
     __shared__ float4 sp[kPartTile];
     __shared__ float2 sc[kPartTile];
     __shared__ long long sred[2][kPartPerBlock];
@@ -822,25 +853,24 @@ __device__ __forceinline__ void particles_body(const Dev &D, int parity, int *ow
     // link sums) while every warp screens, so that the FP64 tail starts
     // without a global round trip
     __shared__ double s_cur[kPartPerBlock][kPartFields];
-    __shared__ LinkSums s_ls[kPartPerBlock];
-    __shared__ GeomRec s_geo[kPartPerBlock];
-    __shared__ double4 s_pk[kPartPerBlock];
+    __shared__ __align__(16) LinkSums s_ls[kPartPerBlock];
+    __shared__ __align__(16) GeomRec s_geo[kPartPerBlock];
+    __shared__ __align__(32) double4 s_pk[kPartPerBlock];
     if (warp == kPartPerBlock - 1) {
-        for (int t = lane; t < kPartPerBlock * kPartFields; t += 32) {
-            const int q = t / kPartFields, f = t - q * kPartFields, bq = blk * kPartPerBlock + q;
-            if (bq < D.np) s_cur[q][f] = D.part[parity].x[(long long)f * D.np + bq];
+        // asynchronous copies: the warp goes on to its screening at once
+        const int b0 = blk * kPartPerBlock, nb = min(kPartPerBlock, D.np - b0);
+        for (int t = lane; t < nb * kPartFields; t += 32) {
+            const int q = t / kPartFields, f = t - q * kPartFields;
+            copy_async<8>(&s_cur[q][f], D.part[parity].x + (long long)f * D.np + b0 + q);
         }
-        static_assert(sizeof(GeomRec) == 64, "a geometry record is 16 words");
-        for (int t = lane; t < kPartPerBlock * 16; t += 32) {
-            const int q = t >> 4, w = t & 15, bq = blk * kPartPerBlock + q;
-            if (bq < D.np) reinterpret_cast<int *>(&s_geo[q])[w] = reinterpret_cast<const int *>(&D.geo[parity][bq])[w];
+        static_assert(sizeof(GeomRec) == 64 && sizeof(LinkSums) == 64, "records of four 16-byte words");
+        for (int t = lane; t < nb * 4; t += 32) {
+            copy_async<16>(reinterpret_cast<char *>(s_geo) + 16 * t, reinterpret_cast<const char *>(D.geo[parity] + b0) + 16 * t);
+            if (!D.direct)
+                copy_async<16>(reinterpret_cast<char *>(s_ls) + 16 * t, reinterpret_cast<const char *>(D.lsum + b0) + 16 * t);
         }
-        if (lane < kPartPerBlock && blk * kPartPerBlock + lane < D.np) s_pk[lane] = D.pconst[blk * kPartPerBlock + lane];
-        if (!D.direct)
-            for (int t = lane; t < kPartPerBlock * 8; t += 32) {
-                const int q = t >> 3, w = t & 7, bq = blk * kPartPerBlock + q;
-                if (bq < D.np) reinterpret_cast<long long *>(&s_ls[q])[w] = reinterpret_cast<const long long *>(&D.lsum[bq])[w];
-            }
+        for (int t = lane; t < nb * 2; t += 32)
+            copy_async<16>(reinterpret_cast<char *>(s_pk) + 16 * t, reinterpret_cast<const char *>(D.pconst + b0) + 16 * t);
     }
     float4 pa = make_float4(0.f, 0.f, 0.f, 0.f);
     float2 ca = make_float2(1.f, 0.f);
@@ -848,7 +878,7 @@ __device__ __forceinline__ void particles_body(const Dev &D, int parity, int *ow
         pa = D.pos4[a];
         ca = D.prc[a];
     }
-    const float s_rep = (float)D.s_rep, inv_eps = (float)(1.0 / D.eps_w);
+    const float s_rep = D.s_repf, inv_eps = D.inv_eps;
     long long sx = 0, sy = 0; // pair repulsion, fixed point
     const int *grid = D.cells[parity];
     const int gx = D.cell_gx, gy = D.cell_gy, ncell = gx * gy;
@@ -907,6 +937,7 @@ __device__ __forceinline__ void particles_body(const Dev &D, int parity, int *ow
         sred[0][warp] = sx;
         sred[1][warp] = sy;
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     const int b = blk * kPartPerBlock + lane;
     if (warp == 0 && lane < kPartPerBlock && b < D.np)
@@ -919,7 +950,7 @@ __device__ __forceinline__ void particles_body(const Dev &D, int parity, int *ow
         const RasterIn &R = sras[warp];
         crowd = __any_sync(0xffffffffu, crowd);
         if (lane == 0) D.crowd[parity ^ 1][a] = crowd;
-        raster_one(D, parity ^ 1, crowd ? own_nxt : nullptr, R.G, R.x, R.y, R.r, R.th, R.b, a, true,
+        raster_one(D, parity ^ 1, crowd ? own_nxt : nullptr, R.G, R.x, R.y, R.r, R.cs, R.b, a, true,
                    D.runs[parity] + (long long)a * D.zone_max, s_geo[warp].Y0);
     }
 }
@@ -940,7 +971,7 @@ __device__ __forceinline__ void raster_body(const Dev &D, int *own, bool bits, i
     if (p >= D.np) return;
     const PartSoA &P = D.part[par];
     if (own && (threadIdx.x & 31) == 0) D.crowd[par][p] = 1;
-    raster_one(D, par, own, D.geo[par][p], P.x[p], P.y[p], P.r[p], P.th[p], P.b[p], p, bits, nullptr, 0);
+    raster_one(D, par, own, D.geo[par][p], P.x[p], P.y[p], P.r[p], D.cs[par][p], P.b[p], p, bits, nullptr, 0);
 }
 
 // Near-tile bitmap: every warp tile (one row, 32 V nodes) that meets a
@@ -1084,9 +1115,10 @@ __global__ void __launch_bounds__(32 * kTeam, link_ctas(kTeam))
     links_body<T, kTeam>(D, A, own, own_nxt, parity, __ldg(D.lorder + b),
                          b + ahead < D.np ? __ldg(D.lorder + b + ahead) : -1);
 }
-__global__ void __launch_bounds__(kPartThreads, 4) k_particles(const Dev D, int parity, int *own_nxt)
+template <int kPB>
+__global__ void __launch_bounds__(32 * kPB, part_ctas(kPB)) k_particles(const Dev D, int parity, int *own_nxt)
 {
-    particles_body(D, parity, own_nxt, (int)blockIdx.x);
+    particles_body<kPB>(D, parity, own_nxt, (int)blockIdx.x);
 }
 __global__ void __launch_bounds__(kBoxThreads)
     k_raster(const Dev D, int *own, bool bits, int parity)
@@ -1145,14 +1177,15 @@ __global__ void __launch_bounds__(32 * kTeam, link_ctas(kTeam))
     links_body<T, kTeam>(sD, static_cast<T *>(a.A[par]), a.own[par], a.own[par ^ 1], par, b,
                          b + ahead < sD.np ? b + ahead : -1);
 }
-__global__ void __launch_bounds__(kPartThreads, 4)
+template <int kPB>
+__global__ void __launch_bounds__(32 * kPB, part_ctas(kPB))
     k_particles_batch(const InstArgs *__restrict__ I, const int *__restrict__ start, int n, int parity)
 {
     __shared__ Dev sD;
     const int i = batch_find(start, n, (int)blockIdx.x);
     copy_dev(sD, I[i].D);
     const int par = parity ^ I[i].poff;
-    particles_body(sD, par, I[i].own[par ^ 1], (int)blockIdx.x - __ldg(start + i));
+    particles_body<kPB>(sD, par, I[i].own[par ^ 1], (int)blockIdx.x - __ldg(start + i));
 }
 // Geometry records of both parities' states.
 __global__ void k_geom_init(const Dev D)
@@ -1161,6 +1194,9 @@ __global__ void k_geom_init(const Dev D)
     if (a >= D.np) return;
     for (int q = 0; q < 2; ++q) {
         const PartSoA &P = D.part[q];
+        double2 cs;
+        cos_sin_rn(P.th[a], cs.x, cs.y);
+        D.cs[q][a] = cs;
         D.geo[q][a] = make_geom(P.x[a], P.y[a], P.r[a], P.b[a], P.th[a], P.ux[a], P.uy[a], P.om[a], P.T[a], P.rho[a],
                                 D.rho_f, D.g);
     }
@@ -1243,6 +1279,24 @@ int sm_count()
     return sms;
 }
 
+template <typename F>
+cudaError_t part_dispatch(int pb, F &&f)
+{
+    switch (pb) {
+    case 1: return f(std::integral_constant<int, 1>{});
+    case 2: return f(std::integral_constant<int, 2>{});
+    case 4: return f(std::integral_constant<int, 4>{});
+    default: return f(std::integral_constant<int, 8>{});
+    }
+}
+// Particles per block of the update (see particles_body).
+int part_per_block(int np, int sms)
+{
+    int pb = 1;
+    while (pb < kPartMax && np > pb * sms) pb *= 2;
+    return pb;
+}
+
 // Shared-memory limit of a link kernel for zones of side N, and the CTAs of it
 // that the GPU holds at once (the distance of its prefetch).
 template <typename K>
@@ -1263,10 +1317,12 @@ cudaError_t prepare_links(Dev &D)
 {
     D.link_ahead = 1;
     D.link_team = 4;
+    D.part_pb = 8;
     if (D.np == 0) return cudaSuccess;
     const int sms = sm_count();
     if (!sms) return cudaErrorUnknown;
     D.link_team = link_team(D.np, sms);
+    D.part_pb = part_per_block(D.np, sms);
     return link_dispatch(D.storage, D.link_team, [&](auto t, auto team) {
         return prepare_link_kernel(k_links<decltype(t), decltype(team)::value>, decltype(team)::value, D.zone_max, sms,
                                    &D.link_ahead);
@@ -1292,6 +1348,7 @@ cudaError_t prepare_links_batch(int zone_max, int np, int storage, LinkPlan *pla
     const int sms = sm_count();
     if (!sms) return cudaErrorUnknown;
     plan->team = link_team(np, sms);
+    plan->part_pb = part_per_block(np, sms);
     plan->smem = link_smem_bytes(zone_max);
     return link_dispatch(storage, plan->team, [&](auto t, auto team) {
         return prepare_link_kernel(k_links_batch<decltype(t), decltype(team)::value>, decltype(team)::value, zone_max,
@@ -1310,20 +1367,23 @@ cudaError_t launch_links_batch(const InstArgs *I, const int *start, int n, int t
     });
 }
 
-cudaError_t launch_particles_batch(const InstArgs *I, const int *start, int n, int total, int parity,
+cudaError_t launch_particles_batch(const InstArgs *I, const int *start, int n, int total, int parity, int pb,
                                    cudaStream_t s)
 {
     if (total <= 0) return cudaSuccess;
-    k_particles_batch<<<total, kPartThreads, 0, s>>>(I, start, n, parity);
-    return cudaGetLastError();
+    return part_dispatch(pb, [&](auto t) {
+        constexpr int kPB = decltype(t)::value;
+        k_particles_batch<kPB><<<total, 32 * kPB, 0, s>>>(I, start, n, parity);
+        return cudaGetLastError();
+    });
 }
 
 // Blocks of each batched step kernel for one instance.
-void batch_blocks(const Dev &D, dim3 sc_block, int out[kBatchPhases])
+void batch_blocks(const Dev &D, dim3 sc_block, int part_pb, int out[kBatchPhases])
 {
     const int V = D.storage == LBM_STORE_FP32 ? 1 : 2;
     out[kBLinks] = D.np;
-    out[kBParticles] = (D.np + kPartPerBlock - 1) / kPartPerBlock;
+    out[kBParticles] = (D.np + part_pb - 1) / part_pb;
     out[kBRefill] = (D.np + kBoxThreads - 1) / kBoxThreads;
     out[kBStream] = ((D.pitch / V + (int)sc_block.x - 1) / (int)sc_block.x) *
                     ((D.ny + (int)sc_block.y - 1) / (int)sc_block.y);
@@ -1363,8 +1423,11 @@ cudaError_t launch_links_direct(const Dev &D, void *A, const int *own_cur, int *
 cudaError_t launch_particles(const Dev &D, int parity, int *own_nxt, cudaStream_t s)
 {
     if (D.np == 0) return cudaSuccess;
-    k_particles<<<(D.np + kPartPerBlock - 1) / kPartPerBlock, kPartThreads, 0, s>>>(D, parity, own_nxt);
-    return cudaGetLastError();
+    return part_dispatch(D.part_pb, [&](auto pb) {
+        constexpr int kPB = decltype(pb)::value;
+        k_particles<kPB><<<(D.np + kPB - 1) / kPB, 32 * kPB, 0, s>>>(D, parity, own_nxt);
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_raster(const Dev &D, int *own, bool bits, int parity, cudaStream_t s)

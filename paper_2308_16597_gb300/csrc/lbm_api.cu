@@ -115,6 +115,7 @@ void layout(const lbm_domain *d, const lbm_particle *p, int32_t n, int storage, 
     L.pos4 = take((size_t)n * sizeof(float4));
     L.prc = take((size_t)n * sizeof(float2));
     L.lsum = take((size_t)n * sizeof(LinkSums));
+    for (int b = 0; b < 2; ++b) L.cs[b] = take((size_t)n * sizeof(double2));
     for (int b = 0; b < 2; ++b) L.geo[b] = take((size_t)n * sizeof(GeomRec));
     L.pconst = take((size_t)n * sizeof(double4));
     L.lorder = take((size_t)n * sizeof(int));
@@ -382,6 +383,8 @@ void fill_dev(lbm_handle *h)
     D.rho_f = P.rho_f;
     D.eps_w = P.eps_w;
     D.s_rep = P.s_rep;
+    D.s_repf = (float)P.s_rep;
+    D.inv_eps = (float)(1.0 / P.eps_w);
     D.fixed = (P.flags & LBM_FLAG_FIXED_PARTICLES) ? 1 : 0;
     D.bits = reinterpret_cast<unsigned *>(ws + L.bits);
     D.bpitch = L.bpitch;
@@ -408,6 +411,7 @@ void fill_dev(lbm_handle *h)
     D.a_elems = (long long)kPop * L.ps + (long long)(kDistTailPad / storage_bytes(D.storage));
     D.prc = reinterpret_cast<float2 *>(ws + L.prc);
     D.lsum = reinterpret_cast<LinkSums *>(ws + L.lsum);
+    for (int b = 0; b < 2; ++b) D.cs[b] = reinterpret_cast<double2 *>(ws + L.cs[b]);
     for (int b = 0; b < 2; ++b) D.geo[b] = reinterpret_cast<GeomRec *>(ws + L.geo[b]);
     D.pconst = reinterpret_cast<double4 *>(ws + L.pconst);
     D.lorder = reinterpret_cast<int *>(ws + L.lorder);

@@ -86,7 +86,7 @@ int upload_starts(lbm_batch *b)
     for (int ph = 0; ph < kBatchPhases; ++ph) b->total[ph] = 0;
     for (int i = 0; i < b->n; ++i) {
         int blocks[kBatchPhases];
-        batch_blocks(b->hs[i]->D, tile_shape(b->tile), blocks);
+        batch_blocks(b->hs[i]->D, tile_shape(b->tile), b->links.part_pb, blocks);
         for (int ph = 0; ph < kBatchPhases; ++ph) {
             st[(size_t)ph * (b->n + 1) + i] = b->total[ph];
             b->total[ph] += blocks[ph];
@@ -147,7 +147,7 @@ int enqueue_batch_step(lbm_batch *b, int par, cudaStream_t st)
     const InstArgs *I = b->d_inst;
     const int n = b->n;
     BCK(b, launch_links_batch(I, starts(b, kBLinks), n, b->total[kBLinks], b->storage, par, b->links, st));
-    BCK(b, launch_particles_batch(I, starts(b, kBParticles), n, b->total[kBParticles], par, st));
+    BCK(b, launch_particles_batch(I, starts(b, kBParticles), n, b->total[kBParticles], par, b->links.part_pb, st));
     BCK(b, cudaEventRecord(b->fork, st));
     BCK(b, cudaStreamWaitEvent(b->side, b->fork, 0));
     BCK(b, launch_boundary_batch(I, starts(b, kBBoundary), n, b->total[kBBoundary], b->storage, par, false, b->side));

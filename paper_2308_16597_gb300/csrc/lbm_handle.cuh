@@ -14,7 +14,7 @@ struct Layout {
     long long ps = 0;
     size_t nslots = 0;
     size_t A[2], own[2], bits, slot_node, slot_q, slot_base, part[2], crowd[2], force, pos4, prc, lsum,
-        geo[2], pconst, lorder, status, pack, stage, left, near, dsum, cells[2], runs[2], total;
+        geo[2], cs[2], pconst, lorder, status, pack, stage, left, near, dsum, cells[2], runs[2], total;
     int bpitch = 0, left_cap = 0;
     int cell_gx = 1, cell_gy = 1; // cell grid of the pair screening
     double cell_side = 1.0;

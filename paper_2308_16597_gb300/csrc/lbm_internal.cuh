@@ -124,10 +124,12 @@ struct Dev {
     float ksc[12];
     float Twall[4];
     double g, rho_f, eps_w, s_rep;
+    float s_repf, inv_eps; // s_rep and 1 / eps_w in FP32
     int fixed;
     int zone_max;      // largest zone side N over the particles (sizes the link kernel's tile)
     int link_ahead;    // link-kernel CTAs resident on the GPU (distance of its L2 prefetch)
     int link_team;     // its warps per particle
+    int part_pb;       // particles per block of the particle update
     // device buffers.  What a step reads and writes of the particles and of
     // the nodes they hold lies in pairs by step parity: with par that of the
     // step, [par] is the state it starts from and [par ^ 1] that one step
@@ -159,6 +161,7 @@ struct Dev {
     int sc_staged;         // whole-lattice stream-collide through the staged kernel (else one block per tile)
     int sc_extra_tx;       // bytes the staged kernel announces beyond its copies (tests of its bounded waits)
     struct GeomRec *geo[2]; // [np] by parity: FP32/int geometry of the positions
+    double2 *cs[2];    // [np] by parity: cos and sin of theta (an ellipse's)
     double4 *pconst;   // [np]: constants of the update (1/M, 1/I, weight W, repulsion scale C)
     int *lorder;       // [np]: the link kernel's CTA order (particles by descending y)
     // pair screening: a grid of square cells of side 1 / cell_inv >= 2 r_max
@@ -295,15 +298,23 @@ __device__ __forceinline__ void cos_sin_rn(double theta, double &c, double &s)
 struct EllFrame {
     double x, y, c, s, a2, b2;
 };
-__device__ __forceinline__ EllFrame ell_frame(double x, double y, double th, double r, double b)
+// (cs: cos and sin of theta, from cos_sin_rn)
+__device__ __forceinline__ EllFrame ell_frame_cs(double x, double y, double2 cs, double r, double b)
 {
     EllFrame E;
     E.x = x;
     E.y = y;
-    cos_sin_rn(th, E.c, E.s);
+    E.c = cs.x;
+    E.s = cs.y;
     E.a2 = __dmul_rn(r, r);
     E.b2 = __dmul_rn(b, b);
     return E;
+}
+__device__ __forceinline__ EllFrame ell_frame(double x, double y, double th, double r, double b)
+{
+    double2 cs;
+    cos_sin_rn(th, cs.x, cs.y);
+    return ell_frame_cs(x, y, cs, r, b);
 }
 // (dx, dy) in the body frame: u along the major axis, v along the minor one.
 __device__ __forceinline__ void ell_uv(const EllFrame &E, double dx, double dy, double &u, double &v)
@@ -327,21 +338,54 @@ __device__ __forceinline__ bool in_ellipse(int i, int j, const EllFrame &E)
 // i.e. P2 t^2 + 2 P1 t + P0 = 0, as t = P0 / (-P1 + sqrt(P1^2 - P2 P0))
 // (P0 > 0 outside, P1 < 0 towards the ellipse: no cancellation).  Also
 // returns d = (i, j) - centre rounded to FP32.
-__device__ __forceinline__ float link_q_ellipse(int i, int j, int k, const EllFrame &E, float &dxf, float &dyf)
+// e: e_k in the body frame and P2 = F's quadratic coefficient along it.
+struct EllDir {
+    double u, v, p2;
+};
+__device__ __forceinline__ EllDir ell_dir(const EllFrame &E, int k)
+{
+    EllDir e;
+    ell_uv(E, (double)ex(k), (double)ey(k), e.u, e.v);
+    e.p2 = ell_form(E, e.u, e.v);
+    return e;
+}
+__device__ __forceinline__ float link_q_ellipse(int i, int j, const EllFrame &E, const EllDir &e, double ab, float &dxf,
+                                                float &dyf)
 {
     const double dx = __dsub_rn((double)i, E.x), dy = __dsub_rn((double)j, E.y);
-    double du, dv, eu, ev;
+    double du, dv;
     ell_uv(E, dx, dy, du, dv);
-    ell_uv(E, (double)ex(k), (double)ey(k), eu, ev);
-    const double P2 = ell_form(E, eu, ev);
-    const double P1 = __dadd_rn(__dmul_rn(__dmul_rn(du, eu), E.b2), __dmul_rn(__dmul_rn(dv, ev), E.a2));
-    const double P0 = __dsub_rn(ell_form(E, du, dv), __dmul_rn(E.a2, E.b2));
-    double disc = __dsub_rn(__dmul_rn(P1, P1), __dmul_rn(P2, P0));
+    const double P1 = __dadd_rn(__dmul_rn(__dmul_rn(du, e.u), E.b2), __dmul_rn(__dmul_rn(dv, e.v), E.a2));
+    const double P0 = __dsub_rn(ell_form(E, du, dv), ab);
+    double disc = __dsub_rn(__dmul_rn(P1, P1), __dmul_rn(e.p2, P0));
     if (disc < 0.0) disc = 0.0;
     double t = __ddiv_rn(P0, __dadd_rn(-P1, __dsqrt_rn(disc)));
     dxf = (float)dx;
     dyf = (float)dy;
     return (float)(t > 1.0 ? 1.0 : t);
+}
+__device__ __forceinline__ float link_q_ellipse(int i, int j, int k, const EllFrame &E, float &dxf, float &dyf)
+{
+    return link_q_ellipse(i, j, E, ell_dir(E, k), __dmul_rn(E.a2, E.b2), dxf, dyf);
+}
+// The frame with what its links share: a^2 b^2 and the eight directions
+// (a fifth of a link's FP64 operations), filled by eight threads.
+struct EllLink {
+    EllFrame E;
+    double ab;
+    EllDir dir[8];
+};
+__device__ __forceinline__ void ell_link_entry(EllLink &L, int t, const EllFrame &E)
+{
+    if (t == 0) {
+        L.E = E;
+        L.ab = __dmul_rn(E.a2, E.b2);
+    }
+    L.dir[t] = ell_dir(E, t + 1);
+}
+__device__ __forceinline__ float link_q_ellipse(int i, int j, int k, const EllLink &L, float &dxf, float &dyf)
+{
+    return link_q_ellipse(i, j, L.E, L.dir[k - 1], L.ab, dxf, dyf);
 }
 // Outward normal at an offset (dx, dy) from the centre, unnormalised: the
 // gradient of u^2 / a^2 + v^2 / b^2 (up to a factor 2) in lattice axes.
@@ -560,18 +604,16 @@ __device__ __forceinline__ GeomRec make_geom(double x, double y, double r, doubl
 // that depend only on its shape, density and temperature (r, C, the zone
 // side, r^2 of a disk, 2 w_k T_w) are those of its record G at any other
 // position, so the result has the same bits as make_geom.
-__device__ __forceinline__ GeomRec move_geom(GeomRec G, double x, double y, double r, double b, double th, double ux,
+__device__ __forceinline__ GeomRec move_geom(GeomRec G, double x, double y, double r, bool ell, double2 cs, double ux,
                                              double uy, double om)
 {
     G.xh = (float)x;
     G.xl = (float)(x - (double)G.xh);
     G.yh = (float)y;
     G.yl = (float)(y - (double)G.yh);
-    if (is_ellipse(r, b)) {
-        double c, s;
-        cos_sin_rn(th, c, s);
-        G.w0 = (float)c;
-        G.w1 = (float)s;
+    if (ell) {
+        G.w0 = (float)cs.x;
+        G.w1 = (float)cs.y;
     }
     G.X0 = (int)floor(x - r) - 1;
     G.Y0 = (int)floor(y - r) - 1;
@@ -962,16 +1004,16 @@ cudaError_t launch_link_order(const Dev &D, int parity, cudaStream_t s);
 enum BatchPhase { kBLinks = 0, kBParticles, kBRefill, kBStream, kBBoundary, kBatchPhases };
 constexpr int kBoundaryBlocksPerInstance = 8;
 // The link kernel of a batch: warps per particle, its shared memory and the
-// distance of its prefetch.
+// distance of its prefetch; particles per block of the update.
 struct LinkPlan {
-    int team = 4, ahead = 1;
+    int team = 4, part_pb = 8, ahead = 1;
     size_t smem = 0;
 };
-void batch_blocks(const Dev &D, dim3 sc_block, int out[kBatchPhases]);
+void batch_blocks(const Dev &D, dim3 sc_block, int part_pb, int out[kBatchPhases]);
 cudaError_t prepare_links_batch(int zone_max, int np, int storage, LinkPlan *plan);
 cudaError_t launch_links_batch(const InstArgs *I, const int *start, int n, int total, int storage, int parity,
                                const LinkPlan &plan, cudaStream_t s);
-cudaError_t launch_particles_batch(const InstArgs *I, const int *start, int n, int total, int parity,
+cudaError_t launch_particles_batch(const InstArgs *I, const int *start, int n, int total, int parity, int pb,
                                    cudaStream_t s);
 cudaError_t launch_stream_collide_batch(const InstArgs *I, const ScInst *sc, const int *bucket, int shift, int n,
                                         int total, int storage, int parity, dim3 block, int resident,

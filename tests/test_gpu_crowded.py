@@ -39,13 +39,13 @@ def test_overlapping_particles(shape, r, cols, rows):
         parts["omega"] = rng.normal(0, 2e-3, n)
     # the columns move towards each other in pairs (slowly: the fluid between
     # them has to leave)
-    parts["ux"] = np.where(k % cols % 2, -0.04, 0.04)
-    parts["uy"] = rng.uniform(-0.01, 0.01, n)
+    parts["ux"] = np.where(k % cols % 2, -0.02, 0.02)
+    parts["uy"] = rng.uniform(-0.005, 0.005, n)
     nx, ny = int(pitch * cols + 14), int(pitch * rows + 11)
     prm = W.base_params(0.05, 0.71, 1e-6, eps_w=1e9)
     sim = lbm.Simulation(W.cavity(nx, ny), parts, prm)
     shared = 0
-    for step in range(10):
+    for step in range(20):
         p0 = sim.particles()
         sim.step(1)
         p1 = sim.particles()
