@@ -96,8 +96,9 @@ extern "C" {
  * block per row tile reading its pulled values straight from global memory,
  * instead of the default staged kernel (persistent blocks, row tiles copied
  * into shared memory by bulk asynchronous copies two tiles ahead).
- * Bit-identical results; for comparisons.  FP32 storage always takes the
- * one-block-per-tile kernel, which is the faster of the two there. */
+ * Bit-identical results; for comparisons.  FP32 storage, and lattices of
+ * fewer than about 1.8 million nodes, always take the one-block-per-tile
+ * kernel, which is the faster of the two there. */
 #define LBM_FLAG_SC_UNSTAGED 32u
 /* Tests only (BF16 or FP16 storage): the staged stream-collide kernel
  * announces one byte more than its copies bring, so its bounded waits run

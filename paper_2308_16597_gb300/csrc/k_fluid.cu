@@ -820,7 +820,7 @@ template <typename T, int V, bool kInst = false>
 struct StTail {
     unsigned long long *full;
     int4 *stile, *snext;
-    int *chunk; // thread 0's claim state: the index of the last tile handed out, tiles left in its chunk
+    int *chunk; // thread 0's claim state: the index of the last tile handed out, tiles left in its chunk, claims made
     __device__ explicit StTail(unsigned char *sm)
     {
         full = reinterpret_cast<unsigned long long *>(sm + kStStages * StGeo<T, V, kInst>::STAGE_B);
@@ -829,7 +829,7 @@ struct StTail {
         chunk = reinterpret_cast<int *>(snext + 2);
     }
 };
-static_assert(kStStages * 8 <= 32 && 32 + (kStStages + 2) * 16 + 8 <= 128, "staged stream-collide: tail layout");
+static_assert(kStStages * 8 <= 32 && 32 + (kStStages + 2) * 16 + 12 <= 128, "staged stream-collide: tail layout");
 
 // The copy a thread issues for every tile, fixed for the launch: copy c
 // (planes 0..13, then the node bits, then in a batch the tile's instance record)
@@ -902,14 +902,21 @@ __device__ __forceinline__ void st_issue(const Dev &D, const T *__restrict__ Ain
 // Tiles claimed per step of the work counter: consecutive tiles, the first
 // looked up, the others found from it (next column, next row, or, at the
 // end of an instance, looked up), so the counter's round trip and the
-// lookup's dependent loads come once per kStChunk tiles.
+// lookup's dependent loads come once per chunk.  Chunks of kStChunk where
+// every block gets several of them, else smaller ones, since the blocks that
+// take one chunk more than the others end last (step of a 2000 x 1000 BF16
+// lattice, 6.6 tiles a block: 26.7 us with chunks of four, 25.5 with one).
 constexpr int kStChunk = 4;
+inline int staged_chunk(int tiles, int resident)
+{
+    return tiles >= 8 * kStChunk * resident ? kStChunk : tiles >= 16 * resident ? 2 : 1;
+}
 
 // The staged loop over the tiles a policy P hands out: P::decode(it) maps a
 // tile index to a tile (int4: instance, row, first column; row -1 past the
 // end), P::next(t, it) gives tile it from tile it - 1, P::dev / ain / aout
-// give an instance's state and buffers, P::ctr the work counter (in chunks
-// of kStChunk tiles) and the done count after it, P::err the error word a
+// give an instance's state and buffers, P::chunk the tiles per claim, P::ctr
+// the work counter (in chunks) and the done count after it, P::err the error word a
 // timeout is recorded in.
 template <typename T, int V, typename P>
 __device__ __forceinline__ void staged_body(const P &pol)
@@ -923,12 +930,16 @@ __device__ __forceinline__ void staged_body(const P &pol)
     const int tid = threadIdx.x;
     const StLane L = st_lane<T, V, kInst>(sm);
     unsigned *ctr = pol.ctr();
-    // thread 0: the tile after `last`, the last one it handed out
+    // thread 0: the tile after `last`, the last one it handed out.  A block's
+    // first chunks, those of the prologue, are its own by its index; the
+    // counter hands out the rest.
+    const int own = (kStStages + pol.chunk - 1) / pol.chunk;
     auto claim = [&](int4 last) {
         int it = t.chunk[0], left = t.chunk[1];
         if (left == 0) {
-            it = (int)atomicAdd(ctr, 1u) * kStChunk;
-            left = kStChunk;
+            const int c = t.chunk[2]++;
+            it = (c < own ? (int)(blockIdx.x + c * gridDim.x) : (int)(atomicAdd(ctr, 1u) + own * gridDim.x)) * pol.chunk;
+            left = pol.chunk;
             last = pol.decode(it);
         } else {
             last = pol.next(last, ++it);
@@ -943,7 +954,7 @@ __device__ __forceinline__ void staged_body(const P &pol)
     if (tid == 0) {
         for (int s = 0; s < kStStages; ++s) mbar_init(smem_addr(t.full + s), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        t.chunk[1] = 0;
+        t.chunk[1] = t.chunk[2] = 0;
         int4 tile = make_int4(0, 0, 0, 0);
         for (int s = 0; s < kStStages; ++s) {
             tile = tile.y < 0 ? tile : claim(tile);
@@ -1051,7 +1062,7 @@ struct StSingle {
     const Dev &D;
     const T *Ain;
     T *Aout;
-    int ntx, nitems, parity;
+    int ntx, nitems, parity, chunk;
     __device__ int4 decode(int it) const
     {
         if (it >= nitems) return make_int4(0, -1, 0, 0);
@@ -1087,7 +1098,7 @@ struct StBatch {
     const InstArgs *__restrict__ I;
     const ScInst *__restrict__ sc;
     const int *__restrict__ bucket;
-    int shift, n, total, parity;
+    int shift, n, total, parity, chunk;
     unsigned *counter;
     __device__ int4 decode(int it) const
     {
@@ -1119,18 +1130,18 @@ struct StBatch {
 template <typename T, int V>
 __global__ void __launch_bounds__(kSCThreads, LBM_ST_MINB)
     k_stream_collide_staged(const Dev D, const T *__restrict__ Ain, T *__restrict__ Aout, int ntx, int nitems,
-                            int parity)
+                            int parity, int chunk)
 {
-    staged_body<T, V>(StSingle<T, V>{D, Ain, Aout, ntx, nitems, parity});
+    staged_body<T, V>(StSingle<T, V>{D, Ain, Aout, ntx, nitems, parity, chunk});
 }
 
 template <typename T, int V>
 __global__ void __launch_bounds__(kSCThreads, LBM_ST_MINB)
     k_stream_collide_staged_batch(const InstArgs *__restrict__ I, const ScInst *__restrict__ sc,
-                                  const int *__restrict__ bucket, int shift, int n, int total, int parity,
+                                  const int *__restrict__ bucket, int shift, int n, int total, int parity, int chunk,
                                   unsigned *counter)
 {
-    staged_body<T, V>(StBatch<T, V>{I, sc, bucket, shift, n, total, parity, counter});
+    staged_body<T, V>(StBatch<T, V>{I, sc, bucket, shift, n, total, parity, chunk, counter});
 }
 
 template <typename T>
@@ -1286,9 +1297,18 @@ int staged_resident(K kernel, int smem)
 
 // The staged kernel's grid: as many blocks as the GPU holds at once (they
 // claim tiles from the work counter, so blocks that start late, behind the
-// boundary kernel's, take fewer).
+// boundary kernel's, take fewer).  *run: whether it is the one to run, namely
+// with kStagedTiles tiles or more per block: below that its blocks' start (a
+// barrier, the first tiles' copies) and their uneven last tiles cost more
+// than they hide, and a lattice in L2 has less latency to hide.  BF16 step
+// without particles, staged / one block per tile, us: 256^2 10.4 / 6.1,
+// 700^2 15.3 / 8.6, 1000^2 16.8 / 13.9, 1531 x 1021 (5.0 tiles a block)
+// 20.7 / 20.3, 2000 x 1000 (6.6) 25.5 / 29.6, 2000^2 44.9 / 49.0, 4000^2
+// 144 / 172.  (LBM_FLAG_TEST_WAIT_TIMEOUT always takes it: that is what the
+// flag tests.)
+constexpr int kStagedTiles = 6;
 template <typename T, int V>
-cudaError_t stream_collide_staged(const Dev &D, const void *Ain, void *Aout, int parity, cudaStream_t s)
+cudaError_t stream_collide_staged(const Dev &D, const void *Ain, void *Aout, int parity, cudaStream_t s, bool *run)
 {
     using G = StGeo<T, V>;
     static int resident = 0;
@@ -1296,8 +1316,10 @@ cudaError_t stream_collide_staged(const Dev &D, const void *Ain, void *Aout, int
         return cudaErrorInvalidValue;
     const int ntx = (D.pitch + G::W - 1) / G::W;
     const int nitems = ntx * D.ny;
+    *run = nitems >= kStagedTiles * resident || D.sc_extra_tx;
+    if (!*run) return cudaSuccess;
     k_stream_collide_staged<T, V><<<min(resident, nitems), kSCThreads, G::SMEM_B, s>>>(
-        D, static_cast<const T *>(Ain), static_cast<T *>(Aout), ntx, nitems, parity);
+        D, static_cast<const T *>(Ain), static_cast<T *>(Aout), ntx, nitems, parity, staged_chunk(nitems, resident));
     return cudaGetLastError();
 }
 
@@ -1309,8 +1331,8 @@ cudaError_t stream_collide_staged_batch(const InstArgs *I, const ScInst *sc, con
     static int resident = 0;
     if (!resident && !(resident = staged_resident(k_stream_collide_staged_batch<T, V>, G::SMEM_B)))
         return cudaErrorInvalidValue;
-    k_stream_collide_staged_batch<T, V><<<min(resident, total), kSCThreads, G::SMEM_B, s>>>(I, sc, bucket, shift, n,
-                                                                                          total, parity, counter);
+    k_stream_collide_staged_batch<T, V><<<min(resident, total), kSCThreads, G::SMEM_B, s>>>(
+        I, sc, bucket, shift, n, total, parity, staged_chunk(total, resident), counter);
     return cudaGetLastError();
 }
 
@@ -1322,7 +1344,11 @@ cudaError_t stream_collide_t(const Dev &D, const void *Ain, void *Aout, int mode
     case kSCNear: return stream_collide_m<T, V, kSCNear>(D, Ain, Aout, parity, s);
     default:
         if constexpr (V == 2) // FP32 is never staged (see fill_dev)
-            if (D.sc_staged) return stream_collide_staged<T, V>(D, Ain, Aout, parity, s);
+            if (D.sc_staged) {
+                bool run = false;
+                const cudaError_t e = stream_collide_staged<T, V>(D, Ain, Aout, parity, s, &run);
+                if (e != cudaSuccess || run) return e;
+            }
         return stream_collide_m<T, V, kSCAll>(D, Ain, Aout, parity, s);
     }
 }
