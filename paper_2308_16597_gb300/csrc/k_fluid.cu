@@ -394,10 +394,6 @@ __device__ __forceinline__ bool tile_near(const Dev &D, int y, int t)
     return (__ldg(D.near + (b >> 5)) >> (b & 31)) & 1u;
 }
 
-// Stream-collide kernel, V consecutive nodes per thread (one vector load and
-// one vector store per plane); FP32 runs V = 1, the 16-bit storages V = 2 so
-// that every load still moves four bytes.  mode selects all warp tiles, or
-// only those away from / within reach of this step's particles.
 // Look-ahead target of a grid launch: the block `ahead` places later in
 // launch order, ahead = ahead_y grid rows + ahead_x blocks (ahead_x < gx).
 __device__ __forceinline__ void ahead_block(const Blk &blk, int ahead_y, int ahead_x, int &bx, int &by)
@@ -414,9 +410,10 @@ __device__ __forceinline__ void ahead_block(const Blk &blk, int ahead_y, int ahe
 // issue one bulk L2 prefetch each of the 14 source row segments of block
 // (bx, by) of a grid over D (in a pass, only of rows holding that pass's
 // tiles).
-template <typename T, int V, int mode>
+template <typename T, int mode>
 __device__ __forceinline__ void prefetch_block(const Dev &D, const T *__restrict__ Ain, int bx, int by)
 {
+    constexpr int V = kScNodes;
     constexpr int kAl = 16 / (int)sizeof(T); // elements per 16 bytes
     const int span = (int)blockDim.x * V;   // nodes of a row per block
     if (threadIdx.x < kPop && threadIdx.y == 0) {
@@ -446,184 +443,96 @@ __device__ __forceinline__ void prefetch_block(const Dev &D, const T *__restrict
     }
 }
 
-template <typename T, int V, bool kSharedFlags>
-__device__ __forceinline__ void sc_tail(const Dev &D, const T *__restrict__ Ain, T *__restrict__ Aout,
-                                        float (&c)[V][kPop], int x0, int y, int parity, const uint2 *sbits);
-
-// pf_x < 0: no look-ahead prefetch here (the caller issues its own).
-template <typename T, int V, int mode = kSCAll>
-__device__ __forceinline__ void sc_body(const Dev &D, const T *__restrict__ Ain, T *__restrict__ Aout, int pf_x,
-                                        int pf_y, int parity, const Blk blk)
+// Two neighbouring nodes x, x + 1 of row y whose pulled values c holds (in
+// the kernel's scale): the side nodes' wall or seam planes, the collision of
+// both at once on paired FP32 instructions, zeros for solid nodes and the
+// padding past nx.  now / before: bits 0 and 1 for solid now and when the step
+// began.  gen: newborn nodes, and the first and last rows' (edge): k_boundary
+// writes them.  Returns false for a non-physical state of a node kept here.
+template <typename T>
+__device__ __forceinline__ bool pair_update(const Dev &D, const T *__restrict__ Ain, float (&c)[2][kPop], int x, int y,
+                                            unsigned now, unsigned before, bool edge, bool (&gen)[2])
 {
-    using VW = typename Vec<T, V>::W;
-    const int lane = threadIdx.x & 31;
-    if (pf_x >= 0) prefetch_block<T, V, mode>(D, Ain, pf_x, pf_y);
-    const int x0 = (blk.x * (int)blockDim.x + (int)threadIdx.x) * V;
-    const int y = blk.y * (int)blockDim.y + (int)threadIdx.y;
-    if (y >= D.ny) return; // uniform across the warp: blockDim.x is a multiple of 32
-    // a warp wholly past the pitch (where the grid's last block of a row
-    // overhangs it) has no node: it returns before its first load
-    if (x0 - lane * V >= D.pitch) return;
-    if constexpr (mode != kSCAll)
-        if (tile_near(D, y, (x0 - (lane * V)) / (32 * V)) != (mode == kSCNear))
-            return; // the other pass's tile (uniform across the warp)
-    const bool act = x0 < D.pitch; // the pitch is a multiple of 32, so all V nodes are in the row
-    float c[V][kPop];
-    // A warp off the first and last row (the common case) pulls without any
-    // wall, seam or range test.  In the first and last warp of a row, the
-    // reads past the row's ends (x = -1, x >= nx, lanes past the pitch: at
-    // most 32 V + 1 elements, since a warp starts below the pitch) land in
-    // the previous plane (every plane with e_x = 1 has index p >= 1), the
-    // next row or the buffer's tail pad, so they stay inside the buffer; the
-    // values they bring feed only the planes of the side nodes x = 0 and
-    // x = nx - 1 that pull across a wall or seam, which the general pull
-    // replaces below, and the padding past nx, which is zeroed.
-    // (The fluid nodes of the first and last rows are k_boundary's: nothing
-    // is pulled for them.)
-    if (y >= 1 && y + 1 < D.ny) {
-        const T *b0 = Ain + (long long)y * D.pitch + x0;
-#pragma unroll
-        for (int p = 0; p < kPop; ++p) {
-            const int d = pdir(p);
-            const int dx = ex(d), dy = ey(d);
-            const T *src = b0 + (long long)p * D.ps - (long long)dy * D.pitch;
-            const long long e = (long long)(src - Ain); // element index, for the bounds checks
-            float v[V];
-            if (in_bounds(D, e, D.a_elems - V + 1)) VecIo<T, V>::unpack(__ldg(reinterpret_cast<const VW *>(src)), v);
-            else {
-#pragma unroll
-                for (int k = 0; k < V; ++k) v[k] = 0.f;
-            }
-            if (dx == 0) {
-#pragma unroll
-                for (int k = 0; k < V; ++k) c[k][p] = v[k];
-            } else if (dx == 1) { // pull from x - 1
-                float l = __shfl_up_sync(kFull, v[V - 1], 1);
-                if (lane == 0) l = in_bounds(D, e - 1, D.a_elems) ? Io<T>::ld(__ldg(src - 1)) : 0.f;
-                c[0][p] = l;
-#pragma unroll
-                for (int k = 1; k < V; ++k) c[k][p] = v[k - 1];
-            } else { // pull from x + 1
-                float r = __shfl_down_sync(kFull, v[0], 1);
-                if (lane == 31) r = in_bounds(D, e + V, D.a_elems) ? Io<T>::ld(__ldg(src + V)) : 0.f;
-#pragma unroll
-                for (int k = 0; k + 1 < V; ++k) c[k][p] = v[k + 1];
-                c[V - 1][p] = r;
-            }
-        }
-    } else {
-#pragma unroll
-        for (int p = 0; p < kPop; ++p)
-#pragma unroll
-            for (int k = 0; k < V; ++k) c[k][p] = 0.f;
-    }
-    if (!act) return;
-    sc_tail<T, V, false>(D, Ain, Aout, c, x0, y, parity, nullptr);
-}
-
-// The part of a stream-collide update after the interior pulls, for the V
-// nodes x0 .. x0 + V - 1 of row y whose pulled values c holds: the side
-// nodes' wall or seam planes, the collision, the stores and the numeric
-// check.  The word pair of the nodes' bits is *sbits (shared memory) or,
-// without kSharedFlags, read from the node bits where it is used (an address
-// computed earlier and held cost the one-block-per-tile kernels registers).
-template <typename T, int V, bool kSharedFlags>
-__device__ __forceinline__ void sc_tail(const Dev &D, const T *__restrict__ Ain, T *__restrict__ Aout,
-                                        float (&c)[V][kPop], int x0, int y, int parity, const uint2 *sbits)
-{
-    using VW = typename Vec<T, V>::W;
     constexpr float kIo = Io<T>::kScaled ? kHalfScale : 1.f; // the side pulls' values in the kernel's scale
-    const bool interior = y >= 1 && y + 1 < D.ny;
     // The nodes x = 0 and x = nx - 1 of the rows between the first and the
     // last: the planes that pull across a side wall or the periodic seam
     // take the wall rule or the far side's value (side_pull: the general
     // pull that k_boundary applies to the first and last rows, restricted
-    // to that case, inlined: as a call it cost the 16-bit kernel 4 us of
+    // to that case, inlined: as a call it cost a 16-bit kernel 4 us of
     // its 180 through register allocation); every other plane
     // is the fast path's.  This warp thus writes whole sectors at the row's
     // ends, and the side columns need no scattered pass of their own.
-    if (interior) {
-        if (x0 == 0) {
+    if (!edge) {
+        if (x == 0) {
 #pragma unroll
             for (int p = 0; p < kPop; ++p)
                 if (ex(pdir(p)) == 1) c[0][p] = side_pull(D, Ain, 0, y, p) * kIo;
         }
-        const int kl = D.nx - 1 - x0;
+        const int kl = D.nx - 1 - x;
 #pragma unroll
-        for (int k = 0; k < V; ++k)
+        for (int k = 0; k < 2; ++k)
             if (k == kl) {
 #pragma unroll
                 for (int p = 0; p < kPop; ++p)
                     if (ex(pdir(p)) == -1) c[k][p] = side_pull(D, Ain, D.nx - 1, y, p) * kIo;
             }
     }
-    bool ok = true, gen[V], anygen = false;
-    // solid now; newborn: solid when the step began only
-    const uint2 bits = kSharedFlags
-                           ? *sbits
-                           : __ldg(reinterpret_cast<const uint2 *>(D.bits) + (long long)y * D.bpitch + (x0 >> 5));
-    const unsigned now = (parity ? bits.x : bits.y) >> (x0 & 31), before = (parity ? bits.y : bits.x) >> (x0 & 31);
-    const bool edge = y == 0 || y == D.ny - 1;
-    if constexpr (V == 2) {
-        // both nodes collided at once on paired FP32 instructions; solid
-        // nodes (and the padding past nx) are zeroed after
-        bool fluid[2];
+    bool fluid[2];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            fluid[k] = x0 + k < D.nx && !((now >> k) & 1u);
-            // newborn nodes and the first and last rows belong to k_boundary,
-            // which writes them
-            gen[k] = fluid[k] && (((before >> k) & 1u) || edge);
-            anygen |= gen[k];
-        }
-        float2 cc[kPop];
+    for (int k = 0; k < 2; ++k) {
+        fluid[k] = x + k < D.nx && !((now >> k) & 1u);
+        gen[k] = fluid[k] && (((before >> k) & 1u) || edge);
+    }
+    float2 cc[kPop];
 #pragma unroll
-        for (int p = 0; p < kPop; ++p) cc[p] = make_float2(c[0][p], c[1][p]);
-        bool ok0, ok1;
-        collide_t<float2, Io<T>::kScaled>(D, cc, ok0, ok1);
+    for (int p = 0; p < kPop; ++p) cc[p] = make_float2(c[0][p], c[1][p]);
+    bool ok0, ok1;
+    collide_t<float2, Io<T>::kScaled>(D, cc, ok0, ok1);
+#pragma unroll
+    for (int p = 0; p < kPop; ++p) {
+        c[0][p] = cc[p].x;
+        c[1][p] = cc[p].y;
+    }
+    if (!(fluid[0] && fluid[1])) { // solid nodes and the padding past nx hold zeros
 #pragma unroll
         for (int p = 0; p < kPop; ++p) {
-            c[0][p] = cc[p].x;
-            c[1][p] = cc[p].y;
-        }
-        if (!(fluid[0] && fluid[1])) { // solid nodes and the padding past nx hold zeros
-#pragma unroll
-            for (int p = 0; p < kPop; ++p) {
-                if (!fluid[0]) c[0][p] = 0.f;
-                if (!fluid[1]) c[1][p] = 0.f;
-            }
-        }
-        ok = (!fluid[0] || gen[0] || ok0) && (!fluid[1] || gen[1] || ok1);
-    } else {
-#pragma unroll
-        for (int k = 0; k < V; ++k) {
-            gen[k] = false;
-            if (x0 + k < D.nx && !((now >> k) & 1u)) {
-                // newborn nodes and the first and last rows belong to
-                // k_boundary, which writes them
-                gen[k] = ((before >> k) & 1u) || edge;
-                if (!gen[k]) ok &= collide(D, c[k]);
-            } else {
-#pragma unroll
-                for (int p = 0; p < kPop; ++p) c[k][p] = 0.f;
-            }
-            anygen |= gen[k];
+            if (!fluid[0]) c[0][p] = 0.f;
+            if (!fluid[1]) c[1][p] = 0.f;
         }
     }
+    return (!fluid[0] || gen[0] || ok0) && (!fluid[1] || gen[1] || ok1);
+}
+
+// The word pair of node (x, y)'s bits, in the order of *now and *before.
+__device__ __forceinline__ void node_bits(uint2 w, int parity, int x, unsigned *now, unsigned *before)
+{
+    *now = (parity ? w.x : w.y) >> (x & 31);
+    *before = (parity ? w.y : w.x) >> (x & 31);
+}
+
+// Collides and stores the nodes x0, x0 + 1 of row y whose pulled values c
+// holds; bits: their word pair.
+template <typename T>
+__device__ __forceinline__ void pair_store(const Dev &D, const T *__restrict__ Ain, T *__restrict__ Aout,
+                                           float (&c)[2][kPop], int x0, int y, int parity, uint2 bits)
+{
+    using VW = typename Vec<T, 2>::W;
+    unsigned now, before;
+    node_bits(bits, parity, x0, &now, &before);
+    bool gen[2];
+    const bool ok = pair_update<T>(D, Ain, c, x0, y, now, before, y == 0 || y == D.ny - 1, gen);
     const long long d0 = (long long)y * D.pitch + x0;
     T *dst = Aout + d0;
-    if (!anygen) {
+    if (!(gen[0] || gen[1])) {
 #pragma unroll
         for (int p = 0; p < kPop; ++p) {
-            float v[V];
-#pragma unroll
-            for (int k = 0; k < V; ++k) v[k] = c[k][p];
-            if (in_bounds(D, d0 + (long long)p * D.ps, D.a_elems - V + 1))
-                *reinterpret_cast<VW *>(dst + (long long)p * D.ps) = VecIo<T, V>::pack(v);
+            const float v[2] = {c[0][p], c[1][p]};
+            if (in_bounds(D, d0 + (long long)p * D.ps, D.a_elems - 1))
+                *reinterpret_cast<VW *>(dst + (long long)p * D.ps) = VecIo<T, 2>::pack(v);
         }
     } else {
 #pragma unroll
-        for (int k = 0; k < V; ++k)
+        for (int k = 0; k < 2; ++k)
             if (!gen[k]) {
 #pragma unroll
                 for (int p = 0; p < kPop; ++p)
@@ -632,6 +541,76 @@ __device__ __forceinline__ void sc_tail(const Dev &D, const T *__restrict__ Ain,
             }
     }
     if (!ok) atomicOr(&D.status->err, kErrNumeric);
+}
+
+// Stream-collide of one block, kScNodes nodes a thread (one vector load and
+// store per plane).  mode selects all warp tiles, or only those away from /
+// within reach of this step's particles.  pf_x < 0: no look-ahead prefetch
+// here.
+template <typename T, int mode = kSCAll>
+__device__ __forceinline__ void sc_body(const Dev &D, const T *__restrict__ Ain, T *__restrict__ Aout, int pf_x,
+                                        int pf_y, int parity, const Blk blk)
+{
+    constexpr int kN = kScNodes;
+    static_assert(kN == 2, "a thread collides a pair of nodes");
+    if (pf_x >= 0) prefetch_block<T, mode>(D, Ain, pf_x, pf_y);
+    const int lane = threadIdx.x & 31;
+    const int x0 = (blk.x * (int)blockDim.x + (int)threadIdx.x) * kN;
+    const int y = blk.y * (int)blockDim.y + (int)threadIdx.y;
+    if (y >= D.ny) return; // uniform across the warp: blockDim.x is a multiple of 32
+    // a warp wholly past the pitch (where the grid's last block of a row
+    // overhangs it) has no node: it returns before its first load
+    if (x0 - lane * kN >= D.pitch) return;
+    if constexpr (mode != kSCAll)
+        if (tile_near(D, y, (x0 - (lane * kN)) / (32 * kN)) != (mode == kSCNear))
+            return; // the other pass's tile (uniform across the warp)
+    const bool act = x0 < D.pitch; // the pitch is a multiple of 32, so all kN nodes are in the row
+    // A warp off the first and last row (the common case) pulls without any
+    // wall, seam or range test.  In the first and last warp of a row, the
+    // reads past the row's ends (x = -1, x >= nx, lanes past the pitch: at
+    // most 33 elements, since a warp starts at least 32 nodes below
+    // the pitch) land in the previous plane (every plane with e_x = 1 has
+    // index p >= 1), the next row or the buffer's tail pad, so they stay
+    // inside the buffer; the values they bring feed only the planes of the
+    // side nodes x = 0 and x = nx - 1 that pull across a wall or seam, which
+    // pair_update replaces, and the padding past nx, which is zeroed.
+    // (The fluid nodes of the first and last rows are k_boundary's: nothing
+    // is pulled for them.)
+    const bool interior = y >= 1 && y + 1 < D.ny;
+    const T *b0 = Ain + (long long)y * D.pitch + x0;
+    auto source = [&](int p) { return b0 + (long long)p * D.ps - (long long)ey(pdir(p)) * D.pitch; };
+    auto inside = [&](const T *s, int n) { return in_bounds(D, s - Ain, D.a_elems - n + 1); };
+    using VW = typename Vec<T, 2>::W;
+    float c[2][kPop];
+    if (interior) {
+#pragma unroll
+        for (int p = 0; p < kPop; ++p) {
+            const int dx = ex(pdir(p));
+            const T *src = source(p);
+            float v[2] = {0.f, 0.f};
+            if (inside(src, 2)) VecIo<T, 2>::unpack(__ldg(reinterpret_cast<const VW *>(src)), v);
+            if (dx == 0) {
+                c[0][p] = v[0];
+                c[1][p] = v[1];
+            } else if (dx == 1) { // pull from x - 1
+                float l = __shfl_up_sync(kFull, v[1], 1);
+                if (lane == 0) l = inside(src - 1, 1) ? Io<T>::ld(__ldg(src - 1)) : 0.f;
+                c[0][p] = l;
+                c[1][p] = v[0];
+            } else { // pull from x + 1
+                float r = __shfl_down_sync(kFull, v[0], 1);
+                if (lane == 31) r = inside(src + 2, 1) ? Io<T>::ld(__ldg(src + 2)) : 0.f;
+                c[0][p] = v[1];
+                c[1][p] = r;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int p = 0; p < kPop; ++p) c[0][p] = c[1][p] = 0.f;
+    }
+    if (act)
+        pair_store<T>(D, Ain, Aout, c, x0, y, parity,
+                      __ldg(reinterpret_cast<const uint2 *>(D.bits) + (long long)y * D.bpitch + (x0 >> 5)));
 }
 
 // General path, beside the stream-collide kernel (it reads only the previous
@@ -685,20 +664,27 @@ __device__ __forceinline__ void boundary_body(const Dev &D, const T *__restrict_
     if (!ok) atomicOr(&D.status->err, kErrNumeric);
 }
 
-// Blocks per SM that measured best on the 4000^2 benchmark: FP32 10 (48
-// registers; 268 us against 272 with 8 and 279 with 12), 16-bit storage 9
-// (at most 56 registers, a few spilled: BF16 180.8 us against 184.6 with 8
-// and 181.8 with 10; the kernel waits on L2 latency as much as on issue, so
-// the ninth block's warps outweigh the spills).
-template <typename T, int V, int mode>
-__global__ void __launch_bounds__(kSCThreads, V == 1 ? 10 : 9)
-    k_stream_collide(const Dev D, const T *__restrict__ Ain, T *__restrict__ Aout, int ahead_y, int ahead_x,
-                     int parity)
+// Two nodes a thread, collided on paired FP32 instructions, and blocks per SM
+// as measured (step without particles, us): FP32 8 (64 registers; 4000^2
+// with the prefetch below: 279 with 6, 7 or 8, 289 with 9), 16-bit storage 9
+// (at most 56 registers).  FP32 with one node a thread (10 blocks) and with
+// two: 777 x 513 9.2 / 7.2, 1000^2 24.4 / 17.8, 1000 x 2000 39.5 / 37.2, 2000^2
+// 72.6 / 70.6, 4000^2 268 / 259 (1.03 of the copy bandwidth): from L2 the kernel is
+// bound by instruction issue, from HBM by the loads in flight.  16-bit
+// storage with four nodes a thread (8-byte loads): 1000^2 12.7, 1531 x 1021
+// 19.7, 700^2 8.9, against 13.1, 18.7, 8.1 with two.
+// The prefetch (ahead_y >= 0) pays where a block's 4-byte loads leave the
+// memory latency uncovered: 16-bit storage beyond L2 (2000^2 48.7 against
+// 54.7 us, but 1000^2 13.9 against 13.1).
+constexpr int sc_ctas(int elem) { return elem == 4 ? 8 : 9; }
+template <typename T, int mode>
+__global__ void __launch_bounds__(kSCThreads, sc_ctas(sizeof(T)))
+    k_stream_collide(const Dev D, const T *__restrict__ Ain, T *__restrict__ Aout, int ahead_y, int ahead_x, int parity)
 {
     const Blk blk = this_blk();
-    int bx, by;
-    ahead_block(blk, ahead_y, ahead_x, bx, by);
-    sc_body<T, V, mode>(D, Ain, Aout, bx, by, parity, blk);
+    int bx = -1, by = 0;
+    if (sizeof(T) == 2 && ahead_y >= 0) ahead_block(blk, ahead_y, ahead_x, bx, by);
+    sc_body<T, mode>(D, Ain, Aout, bx, by, parity, blk);
 }
 
 
@@ -923,8 +909,8 @@ __device__ __forceinline__ void staged_body(const P &pol)
 {
     constexpr bool kInst = P::kInst;
     using G = StGeo<T, V, kInst>;
-    using E = Elem<T>;
     using VW = typename Vec<T, V>::W;
+    static_assert(V == 2, "a thread collides a pair of nodes");
     extern __shared__ __align__(128) unsigned char sm[];
     const StTail<T, V, kInst> t(sm);
     const int tid = threadIdx.x;
@@ -994,9 +980,7 @@ __device__ __forceinline__ void staged_body(const P &pol)
                 for (int p = 0; p < kPop; ++p) {
                     const int dx = ex(pdir(p));
                     const T *seg = reinterpret_cast<const T *>(sb + p * G::SEG_B) + G::H + tid * V;
-                    if constexpr (V == 1) {
-                        c[0][p] = E::ld(seg[-dx]);
-                    } else {
+                    {
                         float a[2];
                         VecIo<T, V>::unpack(*reinterpret_cast<const VW *>(seg), a);
                         if (dx == 0) {
@@ -1025,8 +1009,8 @@ __device__ __forceinline__ void staged_body(const P &pol)
                     ain = pol.ain(tile.x);
                     aout = pol.aout(tile.x);
                 }
-                sc_tail<T, V, true>(D, ain, aout, c, x0, y, kInst ? pol.parity ^ rec->poff : pol.parity,
-                                    reinterpret_cast<const uint2 *>(sb + G::BITS_OFF) + (tid * V >> 5));
+                pair_store<T>(D, ain, aout, c, x0, y, kInst ? pol.parity ^ rec->poff : pol.parity,
+                              reinterpret_cast<const uint2 *>(sb + G::BITS_OFF)[tid * V >> 5]);
             }
         }
         if (tid == 0) t.snext[(k + 1) & 1] = claimed;
@@ -1160,20 +1144,22 @@ __global__ void __launch_bounds__(128)
 // instances (often one of a later instance: prefetching only within the
 // block's own instance left most blocks of small instances without a
 // prefetch).
-template <typename T, int V>
-__global__ void __launch_bounds__(kSCThreads, V == 1 ? 10 : 9) // as k_stream_collide (BF16 ensemble: 0.516 against 0.522 ms per step with 8)
+template <typename T>
+__global__ void __launch_bounds__(kSCThreads, sc_ctas(sizeof(T)))
     k_stream_collide_batch(const InstArgs *__restrict__ I, const ScInst *__restrict__ sc,
                            const int *__restrict__ bucket, int shift, int n, int total, int parity, int resident)
 {
     // the look-ahead target is the block `resident` places later in the
-    // launch over all instances, which is often in a later instance
+    // launch over all instances, which is often in a later instance (FP32 too:
+    // a block's own lookups come before its loads; 64 cavities 493 against
+    // 524 us without it)
     const int tg = (int)blockIdx.x + resident;
     if (threadIdx.x < kPop && threadIdx.y == 0 && tg < total) {
         const int j = sc_find(sc, bucket, shift, n, tg);
         const InstArgs &t = I[j];
         int bx, by;
         sc_tile(sc + j, tg, bx, by);
-        prefetch_block<T, V, kSCAll>(t.D, static_cast<const T *>(t.A[parity ^ t.poff]), bx, by);
+        prefetch_block<T, kSCAll>(t.D, static_cast<const T *>(t.A[parity ^ t.poff]), bx, by);
     }
     const int i = sc_find(sc, bucket, shift, n, (int)blockIdx.x);
     const InstArgs &a = I[i];
@@ -1181,7 +1167,7 @@ __global__ void __launch_bounds__(kSCThreads, V == 1 ? 10 : 9) // as k_stream_co
     sc_tile(sc + i, (int)blockIdx.x, bx, by);
     const Blk blk{bx, by, 0, 0}; // the grid extents are not used by the body
     const int par = parity ^ a.poff;
-    sc_body<T, V>(a.D, static_cast<const T *>(a.A[par]), static_cast<T *>(a.A[par ^ 1]), -1, 0, par, blk);
+    sc_body<T>(a.D, static_cast<const T *>(a.A[par]), static_cast<T *>(a.A[par ^ 1]), -1, 0, par, blk);
 }
 
 template <typename T, int kWhat>
@@ -1260,7 +1246,11 @@ __global__ void k_fields(const Dev D, const S *__restrict__ A, int row0, float *
 
 namespace {
 
-template <typename T, int V, int mode>
+// A 16-bit lattice of more nodes than this (56 bytes a node in both buffers)
+// does not stay in L2's 126 MB.
+constexpr long long kPrefetchNodes = 1700000;
+
+template <typename T, int mode>
 cudaError_t stream_collide_m(const Dev &D, const void *Ain, void *Aout, int parity, cudaStream_t s)
 {
     static int resident = 0;
@@ -1268,17 +1258,18 @@ cudaError_t stream_collide_m(const Dev &D, const void *Ain, void *Aout, int pari
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide<T, V, mode>, kSCThreads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide<T, mode>, kSCThreads, 0);
         resident = max(1, sms * per_sm);
     }
-    const int tx = D.pitch / V; // threads per row (the pitch is a multiple of 32)
+    const int tx = D.pitch / kScNodes; // threads per row (the pitch is a multiple of 32)
     int bx = ((tx + 31) / 32) * 32;
     if (bx > kSCThreads) bx = kSCThreads;
     const int by = kSCThreads / bx;
     dim3 block(bx, by);
     dim3 grid((tx + bx - 1) / bx, (D.ny + by - 1) / by);
-    k_stream_collide<T, V, mode><<<grid, block, 0, s>>>(D, static_cast<const T *>(Ain), static_cast<T *>(Aout),
-                                                        resident / (int)grid.x, resident % (int)grid.x, parity);
+    const bool pf = sizeof(T) == 2 && (long long)D.pitch * D.ny > kPrefetchNodes;
+    k_stream_collide<T, mode><<<grid, block, 0, s>>>(D, static_cast<const T *>(Ain), static_cast<T *>(Aout),
+                                                     pf ? resident / (int)grid.x : -1, resident % (int)grid.x, parity);
     return cudaGetLastError();
 }
 
@@ -1336,20 +1327,20 @@ cudaError_t stream_collide_staged_batch(const InstArgs *I, const ScInst *sc, con
     return cudaGetLastError();
 }
 
-template <typename T, int V>
+template <typename T>
 cudaError_t stream_collide_t(const Dev &D, const void *Ain, void *Aout, int mode, int parity, cudaStream_t s)
 {
     switch (mode) {
-    case kSCFar: return stream_collide_m<T, V, kSCFar>(D, Ain, Aout, parity, s);
-    case kSCNear: return stream_collide_m<T, V, kSCNear>(D, Ain, Aout, parity, s);
+    case kSCFar: return stream_collide_m<T, kSCFar>(D, Ain, Aout, parity, s);
+    case kSCNear: return stream_collide_m<T, kSCNear>(D, Ain, Aout, parity, s);
     default:
-        if constexpr (V == 2) // FP32 is never staged (see fill_dev)
+        if constexpr (sizeof(T) == 2) // FP32 is never staged (see fill_dev)
             if (D.sc_staged) {
                 bool run = false;
-                const cudaError_t e = stream_collide_staged<T, V>(D, Ain, Aout, parity, s, &run);
+                const cudaError_t e = stream_collide_staged<T, 2>(D, Ain, Aout, parity, s, &run);
                 if (e != cudaSuccess || run) return e;
             }
-        return stream_collide_m<T, V, kSCAll>(D, Ain, Aout, parity, s);
+        return stream_collide_m<T, kSCAll>(D, Ain, Aout, parity, s);
     }
 }
 
@@ -1392,16 +1383,16 @@ cudaError_t fields_t(const Dev &D, const void *A, int row0, int rows, float *rho
 
 int near_tiles_per_row(int storage, int pitch)
 {
-    const int span = 32 * (storage == LBM_STORE_FP32 ? 1 : 2);
-    return (pitch + span - 1) / span;
+    (void)storage;
+    return (pitch + 32 * kScNodes - 1) / (32 * kScNodes);
 }
 
 cudaError_t launch_stream_collide(const Dev &D, const void *Ain, void *Aout, int mode, int parity, cudaStream_t s)
 {
     switch (D.storage) {
-    case LBM_STORE_FP32: return stream_collide_t<float, 1>(D, Ain, Aout, mode, parity, s);
-    case LBM_STORE_BF16: return stream_collide_t<__nv_bfloat16, 2>(D, Ain, Aout, mode, parity, s);
-    case LBM_STORE_FP16: return stream_collide_t<__half, 2>(D, Ain, Aout, mode, parity, s);
+    case LBM_STORE_FP32: return stream_collide_t<float>(D, Ain, Aout, mode, parity, s);
+    case LBM_STORE_BF16: return stream_collide_t<__nv_bfloat16>(D, Ain, Aout, mode, parity, s);
+    case LBM_STORE_FP16: return stream_collide_t<__half>(D, Ain, Aout, mode, parity, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -1409,7 +1400,7 @@ cudaError_t launch_stream_collide(const Dev &D, const void *Ain, void *Aout, int
 cudaError_t stream_collide_binary_version(int *version)
 {
     cudaFuncAttributes a{};
-    const cudaError_t e = cudaFuncGetAttributes(&a, k_stream_collide<float, 1, kSCAll>);
+    const cudaError_t e = cudaFuncGetAttributes(&a, k_stream_collide<float, kSCAll>);
     if (e == cudaSuccess) *version = a.binaryVersion;
     return e;
 }
@@ -1432,14 +1423,13 @@ cudaError_t launch_stream_collide_batch(const InstArgs *I, const ScInst *sc, con
     if (total <= 0) return cudaSuccess;
     switch (storage) {
     case LBM_STORE_FP32:
-        k_stream_collide_batch<float, 1><<<total, block, 0, s>>>(I, sc, bucket, shift, n, total, parity, resident);
+        k_stream_collide_batch<float><<<total, block, 0, s>>>(I, sc, bucket, shift, n, total, parity, resident);
         break;
     case LBM_STORE_BF16:
-        k_stream_collide_batch<__nv_bfloat16, 2>
-            <<<total, block, 0, s>>>(I, sc, bucket, shift, n, total, parity, resident);
+        k_stream_collide_batch<__nv_bfloat16><<<total, block, 0, s>>>(I, sc, bucket, shift, n, total, parity, resident);
         break;
     case LBM_STORE_FP16:
-        k_stream_collide_batch<__half, 2><<<total, block, 0, s>>>(I, sc, bucket, shift, n, total, parity, resident);
+        k_stream_collide_batch<__half><<<total, block, 0, s>>>(I, sc, bucket, shift, n, total, parity, resident);
         break;
     default: return cudaErrorInvalidValue;
     }
@@ -1488,12 +1478,10 @@ int stream_collide_batch_resident(int storage, dim3 block)
     const int nt = (int)(block.x * block.y);
     switch (storage) {
     case LBM_STORE_BF16:
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_batch<__nv_bfloat16, 2>, nt, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_batch<__nv_bfloat16>, nt, 0);
         break;
-    case LBM_STORE_FP16:
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_batch<__half, 2>, nt, 0);
-        break;
-    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_batch<float, 1>, nt, 0);
+    case LBM_STORE_FP16: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_batch<__half>, nt, 0); break;
+    default: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_stream_collide_batch<float>, nt, 0);
     }
     return max(1, sms * per_sm);
 }

@@ -974,7 +974,7 @@ __device__ __forceinline__ void raster_body(const Dev &D, int *own, bool bits, i
     raster_one(D, par, own, D.geo[par][p], P.x[p], P.y[p], P.r[p], D.cs[par][p], P.b[p], p, bits, nullptr, 0);
 }
 
-// Near-tile bitmap: every warp tile (one row, 32 V nodes) that meets a
+// Near-tile bitmap: every warp tile (one row, 32 kScNodes nodes) that meets a
 // particle's zone at the current position widened by kNearMargin nodes.  One
 // thread per particle and zone row; the bitmap is cleared beforehand.
 __global__ void __launch_bounds__(128) k_near_mask(const Dev D, int span, int parity)
@@ -1381,11 +1381,10 @@ cudaError_t launch_particles_batch(const InstArgs *I, const int *start, int n, i
 // Blocks of each batched step kernel for one instance.
 void batch_blocks(const Dev &D, dim3 sc_block, int part_pb, int out[kBatchPhases])
 {
-    const int V = D.storage == LBM_STORE_FP32 ? 1 : 2;
     out[kBLinks] = D.np;
     out[kBParticles] = (D.np + part_pb - 1) / part_pb;
     out[kBRefill] = (D.np + kBoxThreads - 1) / kBoxThreads;
-    out[kBStream] = ((D.pitch / V + (int)sc_block.x - 1) / (int)sc_block.x) *
+    out[kBStream] = ((D.pitch / kScNodes + (int)sc_block.x - 1) / (int)sc_block.x) *
                     ((D.ny + (int)sc_block.y - 1) / (int)sc_block.y);
     out[kBBoundary] = kBoundaryBlocksPerInstance;
 }
@@ -1395,7 +1394,7 @@ cudaError_t launch_near_mask(const Dev &D, int parity, cudaStream_t s)
     const size_t words = ((size_t)D.ny * D.near_tpr + 31) / 32;
     cudaError_t e = cudaMemsetAsync(D.near, 0, words * sizeof(unsigned), s);
     if (e != cudaSuccess || D.np == 0) return e;
-    const int span = 32 * (D.storage == LBM_STORE_FP32 ? 1 : 2);
+    const int span = 32 * kScNodes;
     const long long threads = (long long)D.np * (D.zone_max + 2 * kNearMargin);
     k_near_mask<<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(D, span, parity);
     return cudaGetLastError();

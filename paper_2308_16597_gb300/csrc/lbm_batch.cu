@@ -96,7 +96,7 @@ int upload_starts(lbm_batch *b)
     // stream-collide: per-instance records (first block, tiles per row and
     // the exact reciprocal of the latter) and buckets of 2^shift blocks,
     // each holding the instance its first block belongs to
-    const int V = b->storage == LBM_STORE_FP32 ? 1 : 2;
+    const int V = kScNodes;
     const int tx = (int)tile_shape(b->tile).x;
     std::vector<ScInst> sc(b->n);
     for (int i = 0; i < b->n; ++i) {

@@ -68,6 +68,8 @@ struct Elem<__half> {
     __host__ __device__ static float ld(__half v) { return __half2float(v) * (1.f / kHalfScale); }
     __host__ __device__ static __half st(float v) { return __float2half_rn(v * kHalfScale); }
 };
+// Nodes of a row per thread of the stream-collide.
+constexpr int kScNodes = 2;
 // Indices of Dev::ksc.
 enum { kScC1 = 0, kScC2, kScB4, kScB7, kScC7, kScC8, kScG2, kScThree, kScBfx, kNumSc };
 // Bytes per stored population.
@@ -139,7 +141,7 @@ struct Dev {
     int2 *left;        // [left_cap]: the nodes particles left this step: (j * nx + i, particle)
     int left_cap;
     int2 *runs[2];     // [np][zone_max] by step parity: each zone row's run (lo, hi) of nodes inside the particle
-    unsigned *near;    // bit per warp tile (row, 32 V nodes) within reach of a particle this step
+    unsigned *near;    // bit per warp tile (row, 32 kScNodes nodes) within reach of a particle this step
     int near_tpr;      // warp tiles per row of that bitmap
     long long nslots;  // slots of the fixed index array
     long long a_elems; // elements of each distribution buffer, its tail pad included
