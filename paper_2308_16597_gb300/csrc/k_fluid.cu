@@ -681,9 +681,11 @@ template <typename T, int mode>
 __global__ void __launch_bounds__(kSCThreads, sc_ctas(sizeof(T)))
     k_stream_collide(const Dev D, const T *__restrict__ Ain, T *__restrict__ Aout, int ahead_y, int ahead_x, int parity)
 {
-    const Blk blk = this_blk();
+    Blk blk = this_blk();
     int bx = -1, by = 0;
     if (sizeof(T) == 2 && ahead_y >= 0) ahead_block(blk, ahead_y, ahead_x, bx, by);
+    // every other sweep from the last row down, where the last one ended
+    if (sizeof(T) == 4 && parity && D.sweep) blk.y = blk.gy - 1 - blk.y;
     sc_body<T, mode>(D, Ain, Aout, bx, by, parity, blk);
 }
 

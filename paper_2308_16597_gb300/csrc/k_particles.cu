@@ -1110,10 +1110,12 @@ __global__ void __launch_bounds__(32 * kTeam, link_ctas(kTeam))
             int *__restrict__ own_nxt, int parity, int ahead)
 {
     // CTAs in the link order (descending y, the rows stream-collide wrote
-    // last first)
+    // last first; after a sweep from the last row down, the reverse: so the
+    // rows the next sweep begins with are gathered last)
     const int b = (int)blockIdx.x;
-    links_body<T, kTeam>(D, A, own, own_nxt, parity, __ldg(D.lorder + b),
-                         b + ahead < D.np ? __ldg(D.lorder + b + ahead) : -1);
+    const bool rev = D.sweep && parity;
+    auto at = [&](int i) { return __ldg(D.lorder + (rev ? D.np - 1 - i : i)); };
+    links_body<T, kTeam>(D, A, own, own_nxt, parity, at(b), b + ahead < D.np ? at(b + ahead) : -1);
 }
 template <int kPB>
 __global__ void __launch_bounds__(32 * kPB, part_ctas(kPB)) k_particles(const Dev D, int parity, int *own_nxt)

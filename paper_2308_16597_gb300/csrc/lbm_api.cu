@@ -427,6 +427,20 @@ void fill_dev(lbm_handle *h)
     }
 }
 
+// Whether the FP32 stream-collide sweeps the rows up and down in turn: a step
+// then finds the rows that the last one wrote last in L2, which pays where the
+// planes do not fit L2 (126 MB) anyway and the links in between do not sweep it
+// (they move about 5 KB per unit of radius; 32 MB at most).  Step, us, one
+// direction / in turn: without particles 1000^2 18.1 / 16.2, 1500^2 41.9 / 36.9,
+// 3000^2 147.2 / 143.0; 1500^2 with 500 disks r = 10 64.2 / 62.2, 2000^2 with
+// 300 89.1 / 86.9; but with 1200 99.8 / 99.6, in its upper half 98.6 / 99.1, and
+// 3000^2 with 2500 200.4 / 202.6.
+bool sweeps(const lbm_handle *h, double radii)
+{
+    const double bytes = 2.0 * kPop * sizeof(float) * (double)h->L.pitch * h->d.ny;
+    return h->prm.storage == LBM_STORE_FP32 && bytes > 96e6 && 5e3 * radii <= 32e6;
+}
+
 // Upload a particle array into the current state (and the copies the step
 // keeps), then build the owner map and flags of those positions.
 int upload_particles(lbm_handle *h, const lbm_particle *p)
@@ -548,7 +562,12 @@ int lbm_init(lbm_handle **out, const lbm_domain *d, const lbm_particle *p, int32
     h->stream = static_cast<cudaStream_t>(stream);
     fill_dev(h);
     h->D.zone_max = 0;
-    for (int a = 0; a < n; ++a) h->D.zone_max = std::max(h->D.zone_max, zone_size(p[a].r));
+    double radii = 0.0;
+    for (int a = 0; a < n; ++a) {
+        h->D.zone_max = std::max(h->D.zone_max, zone_size(p[a].r));
+        radii += p[a].r;
+    }
+    h->D.sweep = sweeps(h, radii) ? 1 : 0;
     auto fail = [&](int code) {
         lbm_destroy(h);
         return code;

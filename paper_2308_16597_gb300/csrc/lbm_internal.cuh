@@ -161,6 +161,7 @@ struct Dev {
     struct DirectSums *dsum; // [np]: the same sums accumulated by atomics (direct addressing)
     int direct;            // links found by the node-parallel scan instead of the index array
     int sc_staged;         // whole-lattice stream-collide through the staged kernel (else one block per tile)
+    int sweep;             // FP32 stream-collide sweeps the rows up and down in turn
     int sc_extra_tx;       // bytes the staged kernel announces beyond its copies (tests of its bounded waits)
     struct GeomRec *geo[2]; // [np] by parity: FP32/int geometry of the positions
     double2 *cs[2];    // [np] by parity: cos and sin of theta (an ellipse's)

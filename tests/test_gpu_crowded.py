@@ -69,3 +69,27 @@ def test_overlapping_particles(shape, r, cols, rows):
     assert np.array_equal(sim.get_state(), other.get_state()) and np.array_equal(sim.owner(), other.owner())
     sim.close()
     other.close()
+
+
+@pytest.mark.parametrize("n,periodic_x", [(0, 0), (40, 0), (40, 1)])
+def test_sweeps_in_turn_equal_one_direction(n, periodic_x):
+    """An FP32 lattice beyond L2 with few particles is swept up and down in
+    turn; the same lattice in a batch always upwards.  Bit for bit."""
+    nx, ny = 929, 1021
+    rng = np.random.default_rng(n)
+    lo = 9.0 + W.S_REP
+    parts = W.rsa_disks(rng, n, 9.0, lo + 1, nx - lo - 2, lo, ny - lo - 1, min_gap=W.S_REP + 1.0) if n else None
+    if n:
+        parts["rho"], parts["T"] = 1.5, 1.0
+        parts["ux"], parts["uy"] = rng.normal(0, 0.03, (2, n))
+    dom = W.cavity(nx, ny, T_wall=(0.2, 0.9, 0.4, 0.0), periodic_x=periodic_x)
+    sims = [lbm.Simulation(dom, parts, W.base_params(0.03, 0.71, 1e-4)) for _ in range(2)]
+    b = lbm.Batch(sims[1:])
+    for steps in (1, 12):
+        sims[0].step(steps)
+        b.step(steps)
+        b.sync()
+        assert np.array_equal(sims[0].get_state(), sims[1].get_state())
+    b.close()
+    for s in sims:
+        s.close()
