@@ -1349,13 +1349,15 @@ cudaError_t stream_collide_t(const Dev &D, const void *Ain, void *Aout, int mode
 template <typename T>
 cudaError_t boundary_t(const Dev &D, const void *Ain, void *Aout, const int *own_cur, int parity, cudaStream_t s)
 {
-    static int blocks = 0;
-    if (!blocks) {
+    static int most = 0;
+    if (!most) {
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        blocks = max(1, 2 * sms);
+        most = max(1, 2 * sms);
     }
+    // a node of the two rows a thread, and room for two nodes left a particle
+    const int blocks = min(most, (2 * D.nx + 2 * D.np + 127) / 128);
     k_boundary<T><<<blocks, 128, 0, s>>>(D, static_cast<const T *>(Ain), static_cast<T *>(Aout), own_cur, parity);
     return cudaGetLastError();
 }

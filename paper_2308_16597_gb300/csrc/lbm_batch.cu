@@ -228,7 +228,15 @@ int lbm_batch_create(lbm_batch **out, lbm_handle *const *hs, int32_t n, void *d_
     b->poff.assign(n, 0);
     b->n = n;
     b->storage = hs[0]->D.storage;
-    b->tile = b->storage == LBM_STORE_FP32 ? 0 : kStagedTile; // until lbm_batch_autotune picks
+    // until lbm_batch_autotune picks: with 16-bit storage the staged kernel
+    // from about a million and a half nodes on, as for a single lattice (BF16
+    // step, staged / 64 x 2 tiles, us: 0.8 million nodes 39.8 / 31.3, 2.0 million
+    // 55.7 / 55.8)
+    {
+        long long nodes = 0;
+        for (int i = 0; i < n; ++i) nodes += (long long)hs[i]->D.pitch * hs[i]->D.ny;
+        b->tile = b->storage == LBM_STORE_FP32 ? 0 : nodes >= 1500000 || hs[0]->D.sc_extra_tx ? kStagedTile : 1;
+    }
     b->parity = 0; // instance i runs at parity b->parity ^ poff[i]
     b->stream = static_cast<cudaStream_t>(stream);
     char *ws = static_cast<char *>(d_workspace);

@@ -2,7 +2,7 @@
 lattice of 6 row tiles or more per resident block, and batches.  Against the
 one-block-per-tile kernel, bit for bit, with tile counts around the chunk
 rule's lines (claims of 1, 2 and 4 tiles; the last claims past the end), ragged
-widths, and a batch of one lattice far below the single-lattice line."""
+widths, and small lattices beside a large one."""
 import numpy as np
 import pytest
 
@@ -38,14 +38,15 @@ def test_large_lattices_equal_the_unstaged_kernel(nx, ny, per, storage):
 
 @pytest.mark.parametrize("storage", [lbm.LBM_STORE_BF16, lbm.LBM_STORE_FP16])
 @pytest.mark.parametrize("nx,ny", [(4, 4), (70, 50), (257, 33), (300, 1301)])
-def test_batch_of_one_small_lattice_equals_it_alone(nx, ny, storage):
-    dom = W.cavity(nx, ny, T_wall=(0.3, 0.8, 1.0, 0.1))
+def test_small_lattices_in_a_staged_batch_equal_themselves_alone(nx, ny, storage):
+    dom, big = W.cavity(nx, ny, T_wall=(0.3, 0.8, 1.0, 0.1)), W.cavity(1300, 1200)
     a, b = start(dom, nx, ny, storage, 0), start(dom, nx, ny, storage, 0)
-    bt = lbm.Batch([a])  # the staged kernel, until autotune picks
+    c = lbm.Simulation(big, None, W.base_params(0.03, 0.71, 0.0), storage=storage)
+    bt = lbm.Batch([a, c])  # large enough for the staged kernel
     bt.step(5)
     bt.sync()
     b.step(5)
     assert np.array_equal(a.get_state(), b.get_state())
     bt.close()
-    a.close()
-    b.close()
+    for s in (a, b, c):
+        s.close()
