@@ -7,14 +7,13 @@
 // ping-ponged between two buffers.  A plane row is read once and written once
 // per step: 112 (FP32) or 56 (16-bit) algorithmic bytes per node.
 //
-// One thread per node.  A pull from x - 1 or x + 1 takes the value from the
-// neighbouring lane by a warp shuffle (one scalar load at the warp edge), so
-// the x-shifted planes cost no extra HBM traffic.  The nodes of the cavity
-// frame (walls, periodic seams) and newborn nodes take a general (scalar)
-// path in a second, small kernel (k_boundary) that runs concurrently with
-// the streaming kernel and keeps that code and its registers out of it.
-// With 16-bit storage a thread holds two nodes, collided together on paired
-// FP32 instructions.
+// Two neighbouring nodes per thread, collided together on paired FP32
+// instructions.  A pull from x - 1 or x + 1 takes the value from the
+// thread's other node or the neighbouring lane, by a warp shuffle (one scalar
+// load at the warp edge), so the x-shifted planes cost no extra HBM traffic.
+// The fluid nodes of the first and last rows and newborn nodes take a general
+// (scalar) path in a second, small kernel (k_boundary) that runs concurrently
+// with the streaming kernel and keeps that code and its registers out of it.
 #include "lbm_internal.cuh"
 
 namespace lbm {
@@ -300,21 +299,21 @@ __device__ __noinline__ void flush_counters(const Dev &D, int parity, const unsi
 } // namespace
 
 // ---------------------------------------------------------------------------
-// Stream-collide kernel.  One thread per node; a block covers 128 consecutive
-// nodes of a row and blocks are launched in row order, so the blocks resident
-// at any moment read and write a compact band of rows of every plane.  Each
-// plane is read with one 4-byte load per thread at the pulled position: the
-// x - e_x shift is taken from the neighbouring lane by a warp shuffle (one
-// extra scalar load at the warp edge), so every plane row crosses HBM once.
+// Stream-collide kernel.  A block of 128 threads covers 256 consecutive nodes
+// of a row (or the same share of two or four rows of a narrow lattice) and
+// blocks are launched in row order, so the blocks resident at any moment read
+// and write a compact band of rows of every plane.  Each plane is read with one
+// vector load per thread at the pulled position: the x - e_x shift is taken
+// within the thread or from the neighbouring lane (one extra scalar load at
+// the warp edge), so every plane row crosses HBM once.
 //
-// Look-ahead prefetch: lanes 0..13 of every block issue one bulk L2 prefetch
-// each (cp.async.bulk.prefetch.L2) of the 14 source row segments of the block
+// Look-ahead prefetch (16-bit storage beyond L2, and batches; see sc_ctas):
+// lanes 0..13 of every block issue one bulk L2 prefetch each
+// (cp.async.bulk.prefetch.L2) of the 14 source row segments of the block
 // `ahead` positions later in launch order, where `ahead` is the number of
 // blocks resident on the GPU.  By the time that block runs its loads hit L2,
 // so the memory latency of one wave overlaps the collisions of the previous
-// wave without holding registers.  (On the 4000^2 benchmark case, when it
-// was introduced: 0.73 of the copy bandwidth against 0.56 without it, about
-// 53 us per launch.)
+// wave without holding registers.
 // ---------------------------------------------------------------------------
 constexpr int kSCThreads = 128;
 
@@ -714,7 +713,7 @@ __global__ void __launch_bounds__(kSCThreads, sc_ctas(sizeof(T)))
 // plane pulling from x - 1, which has index p >= 1, so the previous plane or
 // row lies there; x = pitch .. pitch + H - 1 for one pulling from x + 1, the
 // next row, plane or the buffer's tail pad) feed only the side nodes' wall or
-// seam planes, which sc_tail replaces, and the zeroed padding.  The first and
+// seam planes, which pair_update replaces, and the zeroed padding.  The first and
 // last rows read clamped source rows: every fluid node there belongs to
 // k_boundary, and the others are stored as zeros.
 //
