@@ -1103,7 +1103,10 @@ __global__ void __launch_bounds__(128)
 // 82.3.)  With many particles it is bound by its scattered accesses: the
 // loads and stores of the links alone, from a kernel that does nothing else,
 // take 61 us for 4800 disks in 4000^2 from HBM, in any layout of the planes.
-constexpr int link_ctas(int team) { return team == 4 ? 8 : 3; }
+// Sixteen for zones of more than 32 rows while there is a particle per SM or
+// fewer: their lines and links then take one round instead of two (129 ellipses
+// with zones of 53 rows: 20.3 -> 18.1 us).
+constexpr int link_ctas(int team) { return team == 4 ? 8 : team == 8 ? 3 : 1; }
 template <typename T, int kTeam>
 __global__ void __launch_bounds__(32 * kTeam, link_ctas(kTeam))
     k_links(const Dev D, T *A, const int *__restrict__ own,
@@ -1263,15 +1266,22 @@ template <typename F>
 auto link_dispatch(int storage, int team, F &&f)
 {
     auto by_team = [&](auto t) {
-        return team == 4 ? f(t, std::integral_constant<int, 4>{}) : f(t, std::integral_constant<int, 8>{});
+        return team == 4   ? f(t, std::integral_constant<int, 4>{})
+               : team == 8 ? f(t, std::integral_constant<int, 8>{})
+                           : f(t, std::integral_constant<int, 16>{});
     };
     return storage == LBM_STORE_BF16   ? by_team(__nv_bfloat16{})
            : storage == LBM_STORE_FP16 ? by_team(__half{})
                                        : by_team(float{});
 }
 
-// Warps per particle for np particles (see link_ctas).
-int link_team(int np, int sms) { return np <= link_ctas(8) * sms ? 8 : 4; }
+// Warps per particle for np particles with zones of at most N rows (see
+// link_ctas).
+int link_team(int np, int N, int sms)
+{
+    if (np <= sms && N > 32) return 16;
+    return np <= link_ctas(8) * sms ? 8 : 4;
+}
 int sm_count()
 {
     int dev = 0, sms = 0;
@@ -1323,7 +1333,7 @@ cudaError_t prepare_links(Dev &D)
     if (D.np == 0) return cudaSuccess;
     const int sms = sm_count();
     if (!sms) return cudaErrorUnknown;
-    D.link_team = link_team(D.np, sms);
+    D.link_team = link_team(D.np, D.zone_max, sms);
     D.part_pb = part_per_block(D.np, sms);
     return link_dispatch(D.storage, D.link_team, [&](auto t, auto team) {
         return prepare_link_kernel(k_links<decltype(t), decltype(team)::value>, decltype(team)::value, D.zone_max, sms,
@@ -1349,7 +1359,7 @@ cudaError_t prepare_links_batch(int zone_max, int np, int storage, LinkPlan *pla
 {
     const int sms = sm_count();
     if (!sms) return cudaErrorUnknown;
-    plan->team = link_team(np, sms);
+    plan->team = link_team(np, zone_max, sms);
     plan->part_pb = part_per_block(np, sms);
     plan->smem = link_smem_bytes(zone_max);
     return link_dispatch(storage, plan->team, [&](auto t, auto team) {
