@@ -55,14 +55,22 @@ struct alignas(16) LinkTeam {
     int n;         // links found
     unsigned over; // a line with two links
 };
-size_t link_smem_bytes(int N)
+constexpr int kLinkZoneMax = 60; // zone side: window rows of at most 64 columns
+constexpr size_t link_smem(int N)
 {
-    const size_t b = sizeof(LinkTeam) + (size_t)2 * link_tile_wy(N) * sizeof(unsigned long long) +
+    const size_t b = sizeof(LinkTeam) + (size_t)2 * (N + 4) * sizeof(unsigned long long) +
                      (size_t)(12 * N - 12) * sizeof(int);
     return (b + 15) / 16 * 16;
 }
+// A kernel's dynamic shared memory is limited per function and process, not per
+// handle, so the link kernels leave that limit alone (a handle that lowered it
+// to its own zones would have later launches of one with larger zones refused):
+// beside the kernels' static arrays (below 2 KB) every zone fits the default.
+static_assert(link_smem(kLinkZoneMax) <= 46 * 1024, "the link kernels' shared memory exceeds the default limit");
+size_t link_smem_bytes(int N) { return link_smem(N); }
 
-bool link_zone_supported(int N) { return link_tile_wx(N) <= 64; }
+bool link_zone_supported(int N) { return N <= kLinkZoneMax; }
+static_assert(kLinkZoneMax + 4 <= 64, "the masks of a window row are 64-bit words");
 
 // Counts (and overflow flag) of the screening grid of the next step, which
 // the next step's link kernel fills: block p of the np blocks of a
@@ -1309,16 +1317,14 @@ int part_per_block(int np, int sms)
     return pb;
 }
 
-// Shared-memory limit of a link kernel for zones of side N, and the CTAs of it
-// that the GPU holds at once (the distance of its prefetch).
+// CTAs of a link kernel for zones of side N that the GPU holds at once (the
+// distance of its prefetch).
 template <typename K>
-cudaError_t prepare_link_kernel(K fn, int team, int N, int sms, int *ahead)
+cudaError_t link_resident(K fn, int team, int N, int sms, int *ahead)
 {
-    const int smem = (int)link_smem_bytes(N);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
     int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * team, smem)) != cudaSuccess) return e;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 32 * team, link_smem_bytes(N));
+    if (e != cudaSuccess) return e;
     *ahead = max(1, sms * per_sm);
     return cudaSuccess;
 }
@@ -1336,7 +1342,7 @@ cudaError_t prepare_links(Dev &D)
     D.link_team = link_team(D.np, D.zone_max, sms);
     D.part_pb = part_per_block(D.np, sms);
     return link_dispatch(D.storage, D.link_team, [&](auto t, auto team) {
-        return prepare_link_kernel(k_links<decltype(t), decltype(team)::value>, decltype(team)::value, D.zone_max, sms,
+        return link_resident(k_links<decltype(t), decltype(team)::value>, decltype(team)::value, D.zone_max, sms,
                                    &D.link_ahead);
     });
 }
@@ -1363,7 +1369,7 @@ cudaError_t prepare_links_batch(int zone_max, int np, int storage, LinkPlan *pla
     plan->part_pb = part_per_block(np, sms);
     plan->smem = link_smem_bytes(zone_max);
     return link_dispatch(storage, plan->team, [&](auto t, auto team) {
-        return prepare_link_kernel(k_links_batch<decltype(t), decltype(team)::value>, decltype(team)::value, zone_max,
+        return link_resident(k_links_batch<decltype(t), decltype(team)::value>, decltype(team)::value, zone_max,
                                    sms, &plan->ahead);
     });
 }

@@ -974,7 +974,8 @@ cudaError_t launch_fields(const Dev &D, const void *A, int row0, int rows, float
 cudaError_t launch_links(const Dev &D, void *A, const int *own_cur, int *own_nxt, int parity,
                          cudaStream_t s);
 // Shared memory of the link kernel for zones of side N; prepare_links sets the
-// kernel's shared-memory limit and D.link_ahead (call outside stream capture).
+// link kernel's and the update's shapes and D.link_ahead (call outside stream
+// capture).
 size_t link_smem_bytes(int N);
 // Whether the link kernel holds a zone of side N (window rows of at most 64
 // columns).
