@@ -202,7 +202,7 @@ const char *lbm_strerror(int code);
 
 /* ---- inspection and checkpoint hooks (tests, serving) ------------------- */
 /* Owner map [ny][nx] int32 (host): particle id whose disk holds the node, or
- * -1 for fluid.  Synchronises. */
+ * -1 for fluid.  Synchronises; writes no device memory. */
 int lbm_get_owner(lbm_handle *h, int32_t *out);
 /* Fixed index array of the last step (Sec. 3), host copies: per particle
  * 12N - 12 slots in the order e1..e8, and within a direction by line index
@@ -220,7 +220,8 @@ int lbm_get_slots(lbm_handle *h, int32_t *node, float *q, int64_t cap, int64_t *
  * and plane_stride = pitch * ny rounded up to a multiple of 64; the owner map
  * (int32 [ny][nx]); the node flags (uint8 [ny][pitch]); the particle state as
  * 10 arrays of n doubles (x, y, ux, uy, theta, omega, r, rho, T, b); the previous
- * positions (2 arrays of n doubles).  Synchronises. */
+ * positions (2 arrays of n doubles).  Synchronises; lbm_get_state writes no
+ * device memory. */
 int lbm_state_bytes(lbm_handle *h, size_t *bytes);
 int lbm_get_state(lbm_handle *h, void *host_buf, size_t bytes);
 int lbm_set_state(lbm_handle *h, const void *host_buf, size_t bytes);

@@ -1138,28 +1138,8 @@ __global__ void __launch_bounds__(kBoxThreads)
 {
     raster_body(D, own, bits, parity, (int)blockIdx.x);
 }
-// The whole owner map (-1 before) from the row runs of a parity.
-__global__ void __launch_bounds__(kBoxThreads) k_owner(const Dev D, int *own, int parity)
-{
-    const int p = (int)blockIdx.x * (kBoxThreads / 32) + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (p >= D.np) return;
-    const Box B = box_of(D.geo[parity][p]);
-    for (int b0 = 0; b0 < B.N; b0 += 32) {
-        int2 run = make_int2(1, 0);
-        if (b0 + lane < B.N) run = D.runs[parity][(long long)p * D.zone_max + b0 + lane];
-        write_runs(D, own, B, b0, run.x, run.y, p);
-    }
-}
-// A state image's flag map from the node bits before a step of `parity`, a
-// thread per node, and back, a thread per word.
-__global__ void k_flags_out(const Dev D, uint8_t *flags, int parity)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-    if (i >= D.pitch) return;
-    flags[(long long)j * D.pitch + i] = solid_at(D, i, j, parity)       ? kSolid
-                                        : solid_at(D, i, j, parity ^ 1) ? kNewborn
-                                                                        : kFluid;
-}
+// The node bits before a step of `parity` from a state image's flag map, a
+// thread per word.
 __global__ void k_flags_in(const Dev D, const uint8_t *flags, int parity)
 {
     const int w = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
@@ -1477,20 +1457,6 @@ cudaError_t launch_cells_init(const Dev &D, cudaStream_t s)
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
-}
-
-cudaError_t launch_owner(const Dev &D, int *own, int parity, cudaStream_t s)
-{
-    if (D.np == 0) return cudaSuccess;
-    const int per = kBoxThreads / 32;
-    k_owner<<<(D.np + per - 1) / per, kBoxThreads, 0, s>>>(D, own, parity);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_flags_out(const Dev &D, uint8_t *flags, int parity, cudaStream_t s)
-{
-    k_flags_out<<<dim3((D.pitch + 127) / 128, D.ny), 128, 0, s>>>(D, flags, parity);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_flags_in(const Dev &D, const uint8_t *flags, int parity, cudaStream_t s)

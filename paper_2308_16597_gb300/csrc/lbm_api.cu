@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <unordered_map>
 #include <vector>
@@ -110,13 +111,11 @@ void layout(const lbm_domain *d, const lbm_particle *p, int32_t n, int storage, 
     L.slot_q = take(L.nslots * sizeof(float));
     L.slot_base = take((size_t)(n + 1) * sizeof(int));
     for (int b = 0; b < 2; ++b) L.part[b] = take((size_t)kPartFields * n * sizeof(double));
-    for (int b = 0; b < 2; ++b) L.crowd[b] = take((size_t)n * sizeof(int));
     L.force = take((size_t)3 * n * sizeof(double));
     L.pos4 = take((size_t)n * sizeof(float4));
     L.prc = take((size_t)n * sizeof(float2));
     L.lsum = take((size_t)n * sizeof(LinkSums));
     for (int b = 0; b < 2; ++b) L.cs[b] = take((size_t)n * sizeof(double2));
-    for (int b = 0; b < 2; ++b) L.geo[b] = take((size_t)n * sizeof(GeomRec));
     L.pconst = take((size_t)n * sizeof(double4));
     L.lorder = take((size_t)n * sizeof(int));
     L.status = take(sizeof(Status));
@@ -129,8 +128,14 @@ void layout(const lbm_domain *d, const lbm_particle *p, int32_t n, int storage, 
     for (int a = 0; a < n; ++a) zmax = std::max(zmax, zone_size(p[a].r));
     L.left_cap = std::max(1024, 4 * n * zmax);
     L.left = take((size_t)L.left_cap * sizeof(int2));
-    // each zone row's run of inside nodes, at the current and the next positions
-    for (int b = 0; b < 2; ++b) L.runs[b] = take((size_t)n * std::max(zmax, 1) * sizeof(int2));
+    // by step parity: whether a particle may share nodes, its geometry record,
+    // and each zone row's run of its nodes (side by side: read_maps copies them
+    // at once)
+    for (int b = 0; b < 2; ++b) {
+        L.crowd[b] = take((size_t)n * sizeof(int));
+        L.geo[b] = take((size_t)n * sizeof(GeomRec));
+        L.runs[b] = take((size_t)n * std::max(zmax, 1) * sizeof(int2));
+    }
     L.near = take(((size_t)d->ny * near_tiles_per_row(storage, L.pitch) + 31) / 32 * sizeof(unsigned));
     L.dsum = take((size_t)n * sizeof(DirectSums));
     // cell grid of the pair screening: side 2 r_max + s + 2 (every pair in
@@ -463,12 +468,16 @@ int upload_particles(lbm_handle *h, const lbm_particle *p)
 // What the kernels keep of the positions beside the particle state: geometry
 // records, screening grids, link order, row runs and the owner map (whole:
 // every particle counts as crowded until it has moved); bits: the node bits
-// too.  The maps of the other parity, which the next step clears over the
-// zones one step back, hold nothing.
-int rebuild_maps(lbm_handle *h, bool bits)
+// too; owner (host, may be null): a state image's owner map, which the raster
+// goes over.  The maps of the other parity, which the next step clears over
+// the zones one step back, hold nothing.
+int rebuild_maps(lbm_handle *h, bool bits, const void *owner = nullptr)
 {
-    const size_t nn = (size_t)h->d.nx * h->d.ny;
-    for (int b = 0; b < 2; ++b) CK(h, cudaMemsetAsync(h->own[b], 0xff, nn * sizeof(int), h->stream));
+    const size_t own_b = (size_t)h->d.nx * h->d.ny * sizeof(int);
+    for (int b = 0; b < 2; ++b) {
+        if (owner && b == h->parity) CK(h, cudaMemcpyAsync(h->own[b], owner, own_b, cudaMemcpyHostToDevice, h->stream));
+        else CK(h, cudaMemsetAsync(h->own[b], 0xff, own_b, h->stream));
+    }
     if (bits) CK(h, cudaMemsetAsync(h->D.bits, 0, (size_t)bits_words(h->L.bpitch, h->d.ny) * sizeof(unsigned), h->stream));
     if (h->np == 0) return LBM_OK;
     CK(h, cudaMemsetAsync(h->D.crowd[h->parity ^ 1], 0, h->np * sizeof(int), h->stream));
@@ -480,31 +489,57 @@ int rebuild_maps(lbm_handle *h, bool bits)
     return LBM_OK;
 }
 
-// The owner map of the current positions and, after it, a state image's flag
-// map, made in the distribution buffer that the next step overwrites;
-// release_maps zeroes what they took of it (its gaps between the planes hold
-// zeros).
-struct Maps {
-    int *own;
-    uint8_t *flags;
-    size_t bytes;
-};
-int make_maps(lbm_handle *h, Maps &m)
+// The owner map of the current positions (own, host [ny][nx]) and a state
+// image's flag map (flags, host [ny][pitch]; may be null), with the stream
+// waited for.  Nothing on the device is written: the owner map there, which
+// holds the crowded particles' nodes, takes the others' row runs here (they
+// share no node), and the flags are spelled out from the node bits.
+int read_maps(lbm_handle *h, void *own, uint8_t *flags)
 {
-    const size_t own_b = round_up((size_t)h->d.nx * h->d.ny * sizeof(int), kAlign);
-    const size_t flag_b = (size_t)h->L.pitch * h->d.ny;
-    char *base = static_cast<char *>(h->A[h->parity ^ 1]);
-    m.own = reinterpret_cast<int *>(base);
-    m.flags = reinterpret_cast<uint8_t *>(base + own_b);
-    m.bytes = own_b + flag_b;
-    CK(h, cudaMemsetAsync(m.own, 0xff, own_b, h->stream));
-    CK(h, launch_owner(h->D, m.own, h->parity, h->stream));
-    CK(h, launch_flags_out(h->D, m.flags, h->parity, h->stream));
-    return LBM_OK;
-}
-int release_maps(lbm_handle *h, const Maps &m)
-{
-    CK(h, cudaMemsetAsync(m.own, 0, m.bytes, h->stream));
+    const int par = h->parity, n = h->np, nx = h->d.nx, ny = h->d.ny, zmax = h->D.zone_max;
+    const Layout &L = h->L;
+    std::unique_ptr<char[]> rec, bits;
+    CK(h, cudaMemcpyAsync(own, h->own[par], (size_t)nx * ny * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    if (n > 0) {
+        const size_t bytes = L.runs[par] + (size_t)n * zmax * sizeof(int2) - L.crowd[par];
+        rec.reset(new (std::nothrow) char[bytes]);
+        if (!rec) return LBM_ENOSPC;
+        CK(h, cudaMemcpyAsync(rec.get(), h->ws + L.crowd[par], bytes, cudaMemcpyDeviceToHost, h->stream));
+    }
+    if (flags) {
+        const size_t bytes = (size_t)bits_words(L.bpitch, ny) * sizeof(unsigned);
+        bits.reset(new (std::nothrow) char[bytes]);
+        if (!bits) return LBM_ENOSPC;
+        CK(h, cudaMemcpyAsync(bits.get(), h->D.bits, bytes, cudaMemcpyDeviceToHost, h->stream));
+    }
+    CK(h, cudaStreamSynchronize(h->stream));
+    if (n > 0) {
+        const int *crowd = reinterpret_cast<const int *>(rec.get());
+        const GeomRec *geo = reinterpret_cast<const GeomRec *>(rec.get() + (L.geo[par] - L.crowd[par]));
+        const int2 *runs = reinterpret_cast<const int2 *>(rec.get() + (L.runs[par] - L.crowd[par]));
+        for (int p = 0; p < n; ++p) {
+            if (crowd[p]) continue;
+            for (int r = 0; r < std::min(geo[p].N, zmax); ++r) {
+                const int j = geo[p].Y0 + r;
+                if (j < 0 || j >= ny) continue;
+                const int2 run = runs[(size_t)p * zmax + r];
+                const int lo = std::max(run.x, 0), hi = std::min(run.y, nx - 1);
+                char *row = static_cast<char *>(own) + (size_t)j * nx * sizeof(int); // (of any alignment)
+                for (int i = lo; i <= hi; ++i) std::memcpy(row + (size_t)i * sizeof(int), &p, sizeof(int));
+            }
+        }
+    }
+    if (flags) {
+        const unsigned *w = reinterpret_cast<const unsigned *>(bits.get());
+        for (int j = 0; j < ny; ++j, w += 2 * L.bpitch)
+            for (int i = 0; i < L.pitch; i += 32) {
+                const unsigned now = w[2 * (i >> 5) + par], before = w[2 * (i >> 5) + (par ^ 1)];
+                uint8_t *f = flags + (size_t)j * L.pitch + i;
+                if (!(now | before)) std::memset(f, kFluid, 32);
+                else
+                    for (int b = 0; b < 32; ++b) f[b] = (now >> b & 1u) ? kSolid : (before >> b & 1u) ? kNewborn : kFluid;
+            }
+    }
     return LBM_OK;
 }
 
@@ -741,12 +776,8 @@ int lbm_destroy(lbm_handle *h)
 int lbm_get_owner(lbm_handle *h, int32_t *out)
 {
     if (!h || !out) return LBM_EINVAL;
-    Maps m;
-    int rc = make_maps(h, m);
-    if (rc) return rc;
-    CK(h, cudaMemcpyAsync(out, m.own, (size_t)h->d.nx * h->d.ny * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    if ((rc = release_maps(h, m))) return rc;
-    return sync_status(h);
+    const int rc = read_maps(h, out, nullptr);
+    return rc ? rc : sync_status(h);
 }
 
 int lbm_get_slots(lbm_handle *h, int32_t *node, float *q, int64_t cap, int64_t *count)
@@ -788,15 +819,14 @@ int lbm_get_state(lbm_handle *h, void *buf, size_t bytes)
     if (!h || !buf || bytes < state_parts(h, sz)) return LBM_EINVAL;
     int rc = sync_status(h);
     if (rc) return rc;
-    Maps m;
-    if ((rc = make_maps(h, m))) return rc;
-    const void *src[5] = {h->A[h->parity], m.own, m.flags, h->D.part[h->parity].x, h->D.part[h->parity ^ 1].x};
-    char *o = static_cast<char *>(buf);
+    const void *src[5] = {h->A[h->parity], nullptr, nullptr, h->D.part[h->parity].x, h->D.part[h->parity ^ 1].x};
+    char *o = static_cast<char *>(buf), *dst[5];
     for (int i = 0; i < 5; ++i) {
-        if (sz[i]) CK(h, cudaMemcpyAsync(o, src[i], sz[i], cudaMemcpyDeviceToHost, h->stream));
+        if (sz[i] && src[i]) CK(h, cudaMemcpyAsync(o, src[i], sz[i], cudaMemcpyDeviceToHost, h->stream));
+        dst[i] = o;
         o += sz[i];
     }
-    if ((rc = release_maps(h, m))) return rc;
+    if ((rc = read_maps(h, dst[1], reinterpret_cast<uint8_t *>(dst[2])))) return rc;
     return sync_status(h);
 }
 
@@ -822,10 +852,9 @@ int lbm_set_state(lbm_handle *h, const void *buf, size_t bytes)
     if (h->np > 0) {
         CK(h, cudaMemcpyAsync(h->D.part[par ^ 1].x, h->D.part[par].x, sz[3], cudaMemcpyDeviceToDevice, h->stream));
         CK(h, cudaMemcpyAsync(h->D.part[par ^ 1].x, part[4], sz[4], cudaMemcpyHostToDevice, h->stream));
-        int rc = rebuild_maps(h, false);
-        if (rc) return rc;
-        CK(h, cudaMemcpyAsync(h->own[par], part[1], sz[1], cudaMemcpyHostToDevice, h->stream));
     }
+    const int rc = rebuild_maps(h, false, part[1]);
+    if (rc) return rc;
     return sync_status(h);
 }
 

@@ -987,11 +987,8 @@ cudaError_t launch_particles(const Dev &D, int parity, int *own_nxt, cudaStream_
 // (bits) and owner map (own; every particle marked crowded); either may be
 // left out.
 cudaError_t launch_raster(const Dev &D, int *own, bool bits, int parity, cudaStream_t s);
-// The whole owner map (own: -1 everywhere before) of the positions of a parity.
-cudaError_t launch_owner(const Dev &D, int *own, int parity, cudaStream_t s);
-// A state image's flag map [ny][pitch] from the node bits before a step of
-// `parity`, and back.
-cudaError_t launch_flags_out(const Dev &D, uint8_t *flags, int parity, cudaStream_t s);
+// The node bits before a step of `parity` from a state image's flag map
+// [ny][pitch].
 cudaError_t launch_flags_in(const Dev &D, const uint8_t *flags, int parity, cudaStream_t s);
 cudaError_t launch_pack_particles(const Dev &D, lbm_particle *out, int parity, cudaStream_t s);
 // Geometry records of both parities' positions and the constants of the
