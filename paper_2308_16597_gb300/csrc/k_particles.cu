@@ -185,11 +185,11 @@ __device__ __forceinline__ unsigned transpose32(unsigned x, int lane)
 //  2. links.  Along any line of the zone (Sec. 3: the rows, the columns and
 //     the two families of diagonals) the particle's nodes are one run, and
 //     the only nodes that can be linked to it there are the two next to the
-//     run's ends, one per direction: a warp per family brings the row masks
-//     to a lane per line (shears and 32 x 32 bit transposes), takes the
-//     run's ends, looks the two nodes up in the fluid masks and appends the
-//     links to a list; a line without a link empties its slot of the index
-//     array;
+//     run's ends, one per direction: a warp per family (teams of one or two
+//     warps take the families in turn) brings the row masks to a lane per
+//     line (shears and 32 x 32 bit transposes), takes the run's ends, looks
+//     the two nodes up in the fluid masks and appends the links to a list; a
+//     line without a link empties its slot of the index array;
 //  3. each link: its slot of the index array, wall fraction q, curved
 //     bounce-back of f and g (Sec. 2.3) from the populations read at x_f,
 //     x_f - e_k and x_f - 2 e_k, written into the solid node x_f + e_k
@@ -231,7 +231,7 @@ __device__ __forceinline__ void links_body(const Dev &D, T *A, const int *__rest
     if (warp == 0)
         for (int r = lane; r < wy; r += 32) Fm[r] = fluid_row(D, parity, XA, YA + r, wx > 32);
     if (!crowded) {
-        if (warp == 1)
+        if (warp == 1 % kTeam)
             for (int r = lane; r < wy; r += 32) {
                 unsigned long long m = 0ull;
                 if (r >= 2 && r < N + 2) {
@@ -241,15 +241,28 @@ __device__ __forceinline__ void links_body(const Dev &D, T *A, const int *__rest
                 Om[r] = m;
             }
     } else {
-        for (int r = warp; r < wy; r += kTeam) {
-            const int j = YA + r, i = XA + lane;
-            const int lo = inside(D, i, j) ? own[(long long)j * D.nx + i] : -1;
-            const int hi = wx > 32 && inside(D, i + 32, j) ? own[(long long)j * D.nx + i + 32] : -1;
-            const unsigned ol = __ballot_sync(F, lo == p), oh = __ballot_sync(F, hi == p);
-            if (lane == 0) Om[r] = ((unsigned long long)oh << 32) | ol;
+        // four zone rows' loads of a warp in flight before the first ballot
+        constexpr int kU = kTeam < 4 ? 4 : 8;
+        for (int b0 = warp; b0 < N; b0 += kU * kTeam) {
+            int lo[kU], hi[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int b = b0 + u * kTeam, j = Y0 + b, i = X0 + lane;
+                if (b >= N) break;
+                const int *row = own + (long long)j * D.nx;
+                lo[u] = inside(D, i, j) ? row[i] : -1;
+                hi[u] = N > 32 && inside(D, i + 32, j) ? row[i + 32] : -1;
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int b = b0 + u * kTeam;
+                if (b >= N) break;
+                const unsigned ol = __ballot_sync(F, lo[u] == p), oh = N > 32 ? __ballot_sync(F, hi[u] == p) : 0u;
+                if (lane == 0) Om[b + 2] = (((unsigned long long)oh << 32) | ol) << 2;
+            }
         }
     }
-    if (warp == 2) clear_zone_bits(D, parity, p, lane);
+    if (warp == 2 % kTeam) clear_zone_bits(D, parity, p, lane);
     clear_zone_owner(D, own_nxt, parity, p, tid, kThreads);
     if (tid == kThreads - 1) {
         D.pos4[p] = make_float4(Gp->xh, Gp->yh, Gp->xl, Gp->yl);
@@ -261,7 +274,7 @@ __device__ __forceinline__ void links_body(const Dev &D, T *A, const int *__rest
     }
     // L2 prefetch of the bit rows of particle pa, the one a residency wave
     // later in launch order (none: pa < 0)
-    if (warp == 3 && pa >= 0) {
+    if (warp == 3 % kTeam && pa >= 0) {
         const GeomRec *Ga = D.geo[parity] + pa;
         const int xa = Ga->X0 - 2, ya = Ga->Y0 - 2;
         for (int r = lane; r < link_tile_wy(D.zone_max); r += 32) {
@@ -274,12 +287,13 @@ __device__ __forceinline__ void links_body(const Dev &D, T *A, const int *__rest
 
     // ---- 2. links: the rows, the columns, the diagonals of constant a - b,
     // those of constant a + b; lane l of a round takes line i
-    {
-        const int f = warp & 3, M = 2 * N - 3, lines = f < 2 ? N : M;
+    constexpr int kFam = kTeam < 4 ? kTeam : 4; // families taken side by side
+    for (int f = warp % kFam; f < 4; f += kFam) {
+        const int M = 2 * N - 3, lines = f < 2 ? N : M;
         const int kf = f < 2 ? f + 1 : f + 3;                   // direction into the run's start: 1, 2, 5, 6
         const int sf = f == 0 ? 0 : f == 1 ? N : f == 2 ? 4 * N : 4 * N + M; // its slots; those of the end follow
         const int sb = sf + (f < 2 ? 2 * N : 2 * M);
-        for (int i0 = 32 * (warp >> 2); i0 < lines; i0 += 8 * kTeam) {
+        for (int i0 = 32 * (warp / kFam); i0 < lines; i0 += 32 * (kTeam / kFam)) {
             const int i = i0 + lane;
             // the particle's nodes on line i: bit t, the row b of the node
             // (its column a on a row)
@@ -1103,18 +1117,29 @@ __global__ void __launch_bounds__(128)
 }
 
 // ---- single-instance kernels
-// Warps per particle, one CTA each: eight while that is a single wave (three
-// CTAs of 80 registers per SM), else four (eight CTAs of 64 registers).  Link
-// kernel, us, eight / four (CUDA events): 8 disks 9.9 / 11.9, 300 disks
-// 12.1 / 14.2, 129 ellipses 21.3 / 23.0, 4800 disks 84.7 / 72.1.  (One warp per
-// particle, four particles per CTA: 75.4 with 4800 disks; 12 CTAs per SM:
-// 82.3.)  With many particles it is bound by its scattered accesses: the
-// loads and stores of the links alone, from a kernel that does nothing else,
-// take 61 us for 4800 disks in 4000^2 from HBM, in any layout of the planes.
+// Warps per particle, one CTA each (link_team): eight while that is a single
+// wave (three CTAs of 80 registers per SM), else four (eight CTAs of 64
+// registers).  Link kernel, us, eight / four (CUDA events): 8 disks 9.9 / 11.9,
+// 300 disks 12.1 / 14.2, 129 ellipses 21.3 / 23.0, 4800 disks 84.7 / 72.1.
+// (12 CTAs per SM: 82.3.)  With many particles it is bound by its scattered
+// accesses: the loads and stores of the links alone, from a kernel that does
+// nothing else, take 61 us for 4800 disks in 4000^2 from HBM, in any layout of
+// the planes.
 // Sixteen for zones of more than 32 rows while there is a particle per SM or
-// fewer: their lines and links then take one round instead of two (129 ellipses
-// with zones of 53 rows: 20.3 -> 18.1 us).
-constexpr int link_ctas(int team) { return team == 4 ? 8 : team == 8 ? 3 : 1; }
+// fewer: their lines and links then take one round instead of two.  Disks with
+// zones of 34, 43 and 60 rows, eight / sixteen: 1 particle 12.0 / 10.7,
+// 12.6 / 10.6, 14.6 / 12.5; 152 particles (one per SM) 12.1 / 10.8, 12.2 / 11.3,
+// 14.8 / 13.5; 153 particles 12.3 / 14.6, 13.0 / 14.9, 15.2 / 18.1.
+// One or two where many particles with small zones would wait for their turn:
+// a CTA's chain of dependent loads is as long for a small zone, so what counts
+// is how many particles an SM holds at once (32, 16 or 8).  Disks 0.3 or 4
+// apart, one / two / four: zones of 5 rows, 27,556 of them 79 / 109 / 207;
+// 9 rows, 24,649 106 / 117 / 223; 11 rows, 6,724 38 / 39 / 49; 13 rows, 44,521
+// 222 / 243 / 336; 23 rows, 21,025 231 / 211 / 255; 31 rows, 8,464
+// 160 / 139 / 154.  Below the lines of link_team four are as good or better:
+// 11 rows, 3,136 particles (21 per SM) 34 / 34 / 31; 23 rows, 5,329 (35 per SM)
+// 98 / 83 / 81; 43 rows, 5,184 208 / 159 / 152.
+constexpr int link_ctas(int team) { return team <= 4 ? 32 / team : team == 8 ? 3 : 1; }
 template <typename T, int kTeam>
 __global__ void __launch_bounds__(32 * kTeam, link_ctas(kTeam))
     k_links(const Dev D, T *A, const int *__restrict__ own,
@@ -1254,7 +1279,9 @@ template <typename F>
 auto link_dispatch(int storage, int team, F &&f)
 {
     auto by_team = [&](auto t) {
-        return team == 4   ? f(t, std::integral_constant<int, 4>{})
+        return team == 1   ? f(t, std::integral_constant<int, 1>{})
+               : team == 2 ? f(t, std::integral_constant<int, 2>{})
+               : team == 4 ? f(t, std::integral_constant<int, 4>{})
                : team == 8 ? f(t, std::integral_constant<int, 8>{})
                            : f(t, std::integral_constant<int, 16>{});
     };
@@ -1268,6 +1295,8 @@ auto link_dispatch(int storage, int team, F &&f)
 int link_team(int np, int N, int sms)
 {
     if (np <= sms && N > 32) return 16;
+    if (np > 32 * sms && N <= 12) return 1;
+    if (np > 56 * sms && N <= 40) return 2;
     return np <= link_ctas(8) * sms ? 8 : 4;
 }
 int sm_count()
