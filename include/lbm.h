@@ -309,7 +309,8 @@ int lbm_link_forces_noalloc(float *d_dist, int64_t plane_stride, int32_t pitch,
  *                        32x4 threads: choices 0-2) and, with BF16 or FP16
  *                        storage, the staged kernel (choice 3, the default
  *                        there from 1.5 million nodes on, choice 1 below;
- *                        choice 0 is the FP32 default) on the batch,
+ *                        choice 0 is the FP32 default, choice 2 where no
+ *                        lattice is wider than 64 nodes) on the batch,
  *                        `reps` launches each, without changing any state,
  *                        and keeps the fastest; *choice receives its index
  *                        and *best_ms its mean time per launch (either may

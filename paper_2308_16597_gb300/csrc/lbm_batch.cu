@@ -231,11 +231,18 @@ int lbm_batch_create(lbm_batch **out, lbm_handle *const *hs, int32_t n, void *d_
     // until lbm_batch_autotune picks: with 16-bit storage the staged kernel
     // from about a million and a half nodes on, as for a single lattice (BF16
     // step, staged / 64 x 2 tiles, us: 0.8 million nodes 39.8 / 31.3, 2.0 million
-    // 55.7 / 55.8)
+    // 55.7 / 55.8); with FP32 128 x 1 threads, or 32 x 4 where no row holds more
+    // than the 64 nodes of 32 threads (step, 128 x 1 / 32 x 4, us: 8 lattices of
+    // 30 x 3000 42.7 / 28.0, of 64 x 3000 45.4 / 34.6)
     {
         long long nodes = 0;
-        for (int i = 0; i < n; ++i) nodes += (long long)hs[i]->D.pitch * hs[i]->D.ny;
-        b->tile = b->storage == LBM_STORE_FP32 ? 0 : nodes >= 1500000 || hs[0]->D.sc_extra_tx ? kStagedTile : 1;
+        int widest = 0;
+        for (int i = 0; i < n; ++i) {
+            nodes += (long long)hs[i]->D.pitch * hs[i]->D.ny;
+            widest = std::max(widest, hs[i]->D.pitch);
+        }
+        if (b->storage == LBM_STORE_FP32) b->tile = widest <= 32 * kScNodes ? 2 : 0;
+        else b->tile = nodes >= 1500000 || hs[0]->D.sc_extra_tx ? kStagedTile : 1;
     }
     b->parity = 0; // instance i runs at parity b->parity ^ poff[i]
     b->stream = static_cast<cudaStream_t>(stream);
