@@ -607,9 +607,7 @@ __device__ __forceinline__ void sc_body(const Dev &D, const T *__restrict__ Ain,
 #pragma unroll
         for (int p = 0; p < kPop; ++p) c[0][p] = c[1][p] = 0.f;
     }
-    if (act)
-        pair_store<T>(D, Ain, Aout, c, x0, y, parity,
-                      __ldg(reinterpret_cast<const uint2 *>(D.bits) + (long long)y * D.bpitch + (x0 >> 5)));
+    if (act) pair_store<T>(D, Ain, Aout, c, x0, y, parity, bits_pair(D, x0, y));
 }
 
 // General path, beside the stream-collide kernel (it reads only the previous
@@ -872,7 +870,7 @@ __device__ __forceinline__ void st_issue(const Dev &D, const T *__restrict__ Ain
         return;
     }
     if (L.c == kPop) { // the tile's node bits (rows are padded to whole tiles' words)
-        bulk_to_smem(dst, D.bits + bit_word(D, xs, y, 0), (unsigned)G::BITS_B, b);
+        bulk_to_smem(dst, bits_src(D, bit_word(D, xs, y, 0), G::BITS_B / 4), (unsigned)G::BITS_B, b);
         return;
     }
     int ys = y - ((L.meta & 3) - 1);

@@ -110,8 +110,7 @@ __device__ __forceinline__ void clear_zone_bits(const Dev &D, int parity, int p,
     for (int r = lane; r < N; r += 32) {
         const int j = Y0 + r;
         if (j < 0 || j >= D.ny) continue;
-        unsigned *row = D.bits + (long long)j * D.bpitch * 2 + (parity ^ 1);
-        for (int w = w0; w <= w1; ++w) row[2 * w] = 0u;
+        for (int w = w0; w <= w1; ++w) bits_put(D, bit_word(D, 32 * w, j, parity ^ 1), 0u);
     }
 }
 // (Whole block of nthreads threads.)
@@ -126,9 +125,17 @@ __device__ __forceinline__ void clear_zone_owner(const Dev &D, int *__restrict__
         if (j < 0 || j >= D.ny) continue;
         for (int c = tid & 31; c < N; c += 32) {
             const int i = X0 + c;
-            if (i >= 0 && i < D.nx) own_nxt[(long long)j * D.nx + i] = -1;
+            if (i >= 0 && i < D.nx && in_bounds(D, (long long)j * D.nx + i, (long long)D.nx * D.ny))
+                own_nxt[(long long)j * D.nx + i] = -1;
         }
     }
+}
+
+// Run of zone row r of particle p (empty: lo > hi) at a parity.
+__device__ __forceinline__ int2 run_at(const Dev &D, int parity, int p, int r)
+{
+    const long long i = (long long)p * D.zone_max + r;
+    return in_bounds(D, i, (long long)D.np * D.zone_max) ? D.runs[parity][i] : make_int2(1, 0);
 }
 
 // Row masks of the link kernel's window, 64 columns from XA: the fluid nodes
@@ -137,9 +144,8 @@ __device__ __forceinline__ void clear_zone_owner(const Dev &D, int *__restrict__
 __device__ __forceinline__ unsigned long long fluid_row(const Dev &D, int parity, int XA, int j, bool wide)
 {
     if (j < 0 || j >= D.ny) return 0ull;
-    const unsigned *row = D.bits + (long long)j * D.bpitch * 2 + parity;
     const int w0 = XA >> 5, sh = XA & 31; // XA may be negative: words before the row are not fluid
-    auto word = [&](int w) -> unsigned { return w >= 0 && w < D.bpitch ? ~row[2 * w] : 0u; };
+    auto word = [&](int w) -> unsigned { return w >= 0 && w < D.bpitch ? ~bits_get(D, bit_word(D, 32 * w, j, parity)) : 0u; };
     const unsigned a = word(w0), b = word(w0 + 1), c = wide ? word(w0 + 2) : 0u;
     unsigned long long m = ((unsigned long long)__funnelshift_r(b, c, sh) << 32) | __funnelshift_r(a, b, sh);
     const int in = D.nx - XA; // columns inside the domain
@@ -235,7 +241,7 @@ __device__ __forceinline__ void links_body(const Dev &D, T *A, const int *__rest
             for (int r = lane; r < wy; r += 32) {
                 unsigned long long m = 0ull;
                 if (r >= 2 && r < N + 2) {
-                    const int2 run = D.runs[parity][(long long)p * D.zone_max + r - 2];
+                    const int2 run = run_at(D, parity, p, r - 2);
                     if (run.x <= run.y) m = ((2ull << (run.y - XA)) - 1ull) & (~0ull << (run.x - XA));
                 }
                 Om[r] = m;
@@ -280,7 +286,7 @@ __device__ __forceinline__ void links_body(const Dev &D, T *A, const int *__rest
         for (int r = lane; r < link_tile_wy(D.zone_max); r += 32) {
             const int j = ya + r;
             if (j >= 0 && j < D.ny)
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(D.bits + bit_word(D, max(xa, 0), j, 0)) : "memory");
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(bits_src(D, bit_word(D, max(xa, 0), j, 0), 1)) : "memory");
         }
     }
     __syncthreads();
@@ -683,12 +689,12 @@ __device__ __forceinline__ void run_minus(int lo, int hi, int xlo, int xhi, F &&
 // Raster of one particle by one warp, a lane per zone row: the row's run
 // (lo, hi) of inside nodes, empty when lo > hi, kept by parity; its node bits
 // (bits; at most three words a row, by atomic or); for a crowded particle
-// its nodes in the owner map (own not null).  old (may be null): its runs
-// one step back, from zone row Y0_old (a particle moves less than a node, so
-// its old nodes lie in the rows of its new zone): the nodes it left are
-// listed for the refilling.
+// its nodes in the owner map (own not null).  moved: its runs one step back
+// are those of the other parity, from zone row Y0_old (a particle moves less
+// than a node, so its old nodes lie in the rows of its new zone): the nodes
+// it left are listed for the refilling.
 __device__ __forceinline__ void raster_one(const Dev &D, int par, int *own, const GeomRec &G, double x, double y,
-                                           double r, double2 cs, double pb, int p, bool bits, const int2 *old,
+                                           double r, double2 cs, double pb, int p, bool bits, bool moved,
                                            int Y0_old)
 {
     const int lane = threadIdx.x & 31;
@@ -703,14 +709,13 @@ __device__ __forceinline__ void raster_one(const Dev &D, int par, int *own, cons
             if (in_bounds(D, (long long)p * D.zone_max + b0 + lane, (long long)D.np * D.zone_max))
                 runs[b0 + lane] = make_int2(lo, hi);
             if (bits && lo <= hi) {
-                unsigned *row = D.bits + (long long)j * D.bpitch * 2 + par;
                 for (int w = lo >> 5; w <= hi >> 5; ++w) {
                     const int c0 = max(lo - 32 * w, 0), c1 = min(hi - 32 * w, 31);
-                    atomicOr(row + 2 * w, (~0u << c0) & (~0u >> (31 - c1)));
+                    bits_or(D, bit_word(D, 32 * w, j, par), (~0u << c0) & (~0u >> (31 - c1)));
                 }
             }
-            if (old && j >= Y0_old && j < Y0_old + B.N && j >= 0 && j < D.ny) {
-                const int2 o = old[j - Y0_old];
+            if (moved && j >= Y0_old && j < Y0_old + B.N && j >= 0 && j < D.ny) {
+                const int2 o = run_at(D, par ^ 1, p, j - Y0_old);
                 run_minus(o.x, o.y, lo, hi, [&](int i) {
                     const unsigned at = atomicAdd(&D.status->nb, 1u);
                     if (at < (unsigned)D.left_cap) D.left[at] = make_int2(j * D.nx + i, p);
@@ -972,8 +977,8 @@ __device__ __forceinline__ void particles_body(const Dev &D, int parity, int *ow
         const RasterIn &R = sras[warp];
         crowd = __any_sync(0xffffffffu, crowd);
         if (lane == 0) D.crowd[parity ^ 1][a] = crowd;
-        raster_one(D, parity ^ 1, crowd ? own_nxt : nullptr, R.G, R.x, R.y, R.r, R.cs, R.b, a, true,
-                   D.runs[parity] + (long long)a * D.zone_max, s_geo[warp].Y0);
+        raster_one(D, parity ^ 1, crowd ? own_nxt : nullptr, R.G, R.x, R.y, R.r, R.cs, R.b, a, true, true,
+                   s_geo[warp].Y0);
     }
 }
 
@@ -993,7 +998,7 @@ __device__ __forceinline__ void raster_body(const Dev &D, int *own, bool bits, i
     if (p >= D.np) return;
     const PartSoA &P = D.part[par];
     if (own && (threadIdx.x & 31) == 0) D.crowd[par][p] = 1;
-    raster_one(D, par, own, D.geo[par][p], P.x[p], P.y[p], P.r[p], D.cs[par][p], P.b[p], p, bits, nullptr, 0);
+    raster_one(D, par, own, D.geo[par][p], P.x[p], P.y[p], P.r[p], D.cs[par][p], P.b[p], p, bits, false, 0);
 }
 
 // Near-tile bitmap: every warp tile (one row, 32 kScNodes nodes) that meets a
@@ -1175,8 +1180,8 @@ __global__ void k_flags_in(const Dev D, const uint8_t *flags, int parity)
         now |= (f == kSolid ? 1u : 0u) << b;
         before |= (f == kNewborn ? 1u : 0u) << b;
     }
-    D.bits[bit_word(D, 32 * w, j, parity)] = now;
-    D.bits[bit_word(D, 32 * w, j, parity ^ 1)] = before;
+    bits_put(D, bit_word(D, 32 * w, j, parity), now);
+    bits_put(D, bit_word(D, 32 * w, j, parity ^ 1), before);
 }
 
 // ---- batched kernels: one grid over all instances (InstArgs table, block

@@ -183,8 +183,9 @@ constexpr int kCellCap = 16;
 // index i outside [0, n) and records kErrBounds (LBM_EBOUNDS at the next
 // synchronising call); the caller then skips the access.  The checks stand
 // in for a memory checker: they cover the scattered writes of the particle
-// kernels and every read of the stream-collide fast path.  Without
-// LBM_CHECK the function is constant true and compiles away.
+// kernels, every access to the node bits and row runs, and every read and
+// write of the distributions by the link, stream-collide and boundary kernels.
+// Without LBM_CHECK the function is constant true and compiles away.
 __device__ __forceinline__ bool in_bounds(const Dev &D, long long i, long long n)
 {
 #ifdef LBM_CHECK
@@ -220,12 +221,34 @@ __device__ __forceinline__ long long bit_word(const Dev &D, int x, int y, int pa
 {
     return ((long long)y * D.bpitch + (x >> 5)) * 2 + par;
 }
-__device__ __forceinline__ bool solid_at(const Dev &D, int x, int y, int par)
-{
-    return (D.bits[bit_word(D, x, y, par)] >> (x & 31)) & 1u;
-}
 // Words of the node bits.
 __host__ __device__ inline long long bits_words(int bpitch, int ny) { return (long long)ny * bpitch * 2; }
+// Every access to the node bits, checked in a bounds-checked build: load,
+// store and atomic or of word w, the word pair of node (x, y) (both parities,
+// read-only data of the kernel) and the source of a copy of n words.
+__device__ __forceinline__ bool bits_ok(const Dev &D, long long w) { return in_bounds(D, w, bits_words(D.bpitch, D.ny)); }
+__device__ __forceinline__ unsigned bits_get(const Dev &D, long long w) { return bits_ok(D, w) ? D.bits[w] : 0u; }
+__device__ __forceinline__ void bits_put(const Dev &D, long long w, unsigned v)
+{
+    if (bits_ok(D, w)) D.bits[w] = v;
+}
+__device__ __forceinline__ void bits_or(const Dev &D, long long w, unsigned v)
+{
+    if (bits_ok(D, w)) atomicOr(D.bits + w, v);
+}
+__device__ __forceinline__ uint2 bits_pair(const Dev &D, int x, int y)
+{
+    const long long w = bit_word(D, x, y, 0);
+    return bits_ok(D, w + 1) ? __ldg(reinterpret_cast<const uint2 *>(D.bits + w)) : make_uint2(0u, 0u);
+}
+__device__ __forceinline__ const unsigned *bits_src(const Dev &D, long long w, int n)
+{
+    return bits_ok(D, w) && bits_ok(D, w + n - 1) ? D.bits + w : D.bits;
+}
+__device__ __forceinline__ bool solid_at(const Dev &D, int x, int y, int par)
+{
+    return (bits_get(D, bit_word(D, x, y, par)) >> (x & 31)) & 1u;
+}
 
 // ---------------------------------------------------------------------------
 // Exact FP64 geometry shared by raster, gather and refill.  Every operation is
