@@ -237,12 +237,14 @@ int lbm_batch_create(lbm_batch **out, lbm_handle *const *hs, int32_t n, void *d_
     {
         long long nodes = 0;
         int widest = 0;
+        bool staged = false; // LBM_FLAG_TEST_WAIT_TIMEOUT on an instance: what it tests
         for (int i = 0; i < n; ++i) {
             nodes += (long long)hs[i]->D.pitch * hs[i]->D.ny;
             widest = std::max(widest, hs[i]->D.pitch);
+            staged |= hs[i]->D.sc_extra_tx != 0;
         }
         if (b->storage == LBM_STORE_FP32) b->tile = widest <= 32 * kScNodes ? 2 : 0;
-        else b->tile = nodes >= 1500000 || hs[0]->D.sc_extra_tx ? kStagedTile : 1;
+        else b->tile = nodes >= 1500000 || staged ? kStagedTile : 1;
     }
     b->parity = 0; // instance i runs at parity b->parity ^ poff[i]
     b->stream = static_cast<cudaStream_t>(stream);
