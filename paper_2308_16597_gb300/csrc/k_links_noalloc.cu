@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(kThreads) k_static_gather(View v, unsigned cha
     EllFrame E{};
     if (ell) E = ell_frame(xc, yc, v.P[p].theta, r, v.P[p].b);
     const int N = zone_size(r), cap = 12 * N - 12;
-    const int X0 = (int)floor(xc - r) - 1, Y0 = (int)floor(yc - r) - 1;
+    const int X0 = zone_lo(xc, r), Y0 = zone_lo(yc, r);
     const int base = s.base[p];
     for (int t0 = threadIdx.x; t0 < cap; t0 += kThreads) {
         int k, line;

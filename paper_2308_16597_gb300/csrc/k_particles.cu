@@ -285,7 +285,7 @@ __device__ __forceinline__ void links_body(const Dev &D, T *A, const int *__rest
         const int xa = Ga->X0 - 2, ya = Ga->Y0 - 2;
         for (int r = lane; r < link_tile_wy(D.zone_max); r += 32) {
             const int j = ya + r;
-            if (j >= 0 && j < D.ny)
+            if (j >= 0 && j < D.ny && xa < D.nx)
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(bits_src(D, bit_word(D, max(xa, 0), j, 0), 1)) : "memory");
         }
     }
@@ -636,6 +636,7 @@ __device__ __noinline__ void ellipse_run(const Dev &D, const Box B, const GeomRe
     const int im = (int)floorf(mid + 0.5f);
     const int in = inside(im) ? im : inside(im - 1) ? im - 1 : inside(im + 1) ? im + 1 : INT_MIN;
     if (in == INT_MIN) return; // then no node of the row is inside
+    if (in < xmin || in > xmax) return; // (a centre beyond any lattice: see zone_lo)
     const float h = sqrtf(fmaxf(B1 * B1 - A2 * C0, 0.f)) / A2;
     int lo = max(min(in, (int)ceilf(mid - h)), xmin), hi = min(max(in, (int)floorf(mid + h)), xmax);
     while (lo > xmin && inside(lo - 1)) --lo;
@@ -657,11 +658,12 @@ __device__ __forceinline__ void disk_run(const Dev &D, const Box &B, const GeomR
     if (j < 0 || j >= D.ny) return;
     const DiskDF dk = geom_df(G);
     const int ic = G.ic; // the node of each row nearest the centre
+    const int xmin = B.X0, xmax = B.X0 + B.N - 1;
+    if (ic < xmin || ic > xmax) return; // (a centre beyond any lattice: see zone_lo)
     if (!in_disk_df(ic, j, dk, x, y, r)) return; // then no node of the row is inside
     float dyh, dyl;
     df_offset(j, dk.yh, dk.yl, dyh, dyl);
     const float h = sqrtf(fmaxf(dk.r2h - dyh * dyh, 0.f));
-    const int xmin = B.X0, xmax = B.X0 + B.N - 1;
     int lo = min(ic, (int)ceilf(dk.xh - h)), hi = max(ic, (int)floorf(dk.xh + h));
     lo = max(lo, xmin);
     hi = min(hi, xmax);

@@ -436,6 +436,14 @@ __device__ __forceinline__ double ell_support(const EllFrame &E, double nx, doub
 // integer radii); 12N - 12 fixed slots.
 __host__ __device__ inline int zone_size(double r) { return (int)ceil(2.0 * r) + 3; }
 __host__ __device__ inline int slot_capacity(double r) { return 12 * zone_size(r) - 12; }
+// Its first column or row, for a centre coordinate c.  A centre that is not
+// finite or lies beyond any lattice (a caller's particles in device memory,
+// which no host code checks) gets a zone that no lattice meets, and that leaves
+// room for the offsets of a window (zones of up to 712 nodes): a test such as
+// 0 <= i + 32 && i + 32 < nx keeps out every node outside only while i + 32
+// does not wrap around.
+constexpr int kZoneLeft = -(1 << 29), kZoneRight = 0x7fffffff - 1024;
+__device__ __forceinline__ int zone_lo(double c, double r) { return min(max((int)floor(c - r), kZoneLeft), kZoneRight) - 1; }
 
 // ---------------------------------------------------------------------------
 // Double-float arithmetic in FP32 (an unevaluated sum hi + lo).  GB300 runs
@@ -620,8 +628,8 @@ __device__ __forceinline__ GeomRec make_geom(double x, double y, double r, doubl
     G.r = ell ? -(float)r : (float)r;
     G.C = (float)(3.14159265358979323846 * r * (ell ? b : r) * (rho - rho_f) * g);
     G.N = zone_size(r);
-    G.X0 = (int)floor(x - r) - 1;
-    G.Y0 = (int)floor(y - r) - 1;
+    G.X0 = zone_lo(x, r);
+    G.Y0 = zone_lo(y, r);
     G.ic = (int)floor(x + 0.5);
     G.ux = (float)ux; G.uy = (float)uy; G.om = (float)om; G.wT = (float)(0.2 * T);
     return G;
@@ -641,8 +649,8 @@ __device__ __forceinline__ GeomRec move_geom(GeomRec G, double x, double y, doub
         G.w0 = (float)cs.x;
         G.w1 = (float)cs.y;
     }
-    G.X0 = (int)floor(x - r) - 1;
-    G.Y0 = (int)floor(y - r) - 1;
+    G.X0 = zone_lo(x, r);
+    G.Y0 = zone_lo(y, r);
     G.ic = (int)floor(x + 0.5);
     G.ux = (float)ux; G.uy = (float)uy; G.om = (float)om;
     return G;
