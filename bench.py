@@ -314,6 +314,21 @@ def run_reference(args, wl):
     return 0
 
 
+def stream_collide_form(wl, args):
+    """The stream-collide kernel that runs: with 16-bit storage the staged one from six row tiles of 256 nodes per
+    resident block on (eight blocks per SM), unless asked otherwise; else one block per row tile."""
+    if (getattr(args, "storage", "fp32") == "fp32" or getattr(args, "stream_collide", "staged") == "unstaged"
+            or getattr(args, "overlap", False)):
+        return "one_block_per_tile"
+    try:
+        import torch
+        sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+    except Exception:  # no GPU: a GB300's
+        sms = 152
+    tiles = ((wl.nx + 31) // 32 * 32 + 255) // 256 * wl.ny
+    return "staged" if tiles >= 6 * 8 * sms else "one_block_per_tile"
+
+
 def config_of(wl, args):
     p = wl.particles
     es = 4 if getattr(args, "storage", "fp32") == "fp32" else 2
@@ -322,9 +337,7 @@ def config_of(wl, args):
             "radius": float(p["r"][0]) if len(p) else None,
             "minor_axis": float(p["b"][0]) if len(p) and p["b"][0] > 0 else None,
             "storage": getattr(args, "storage", "fp32"), "links": getattr(args, "links", "index"),
-            # the kernel that ran: FP32 storage always takes one block per row tile
-            "stream_collide": ("one_block_per_tile" if getattr(args, "storage", "fp32") == "fp32"
-                               or getattr(args, "stream_collide", "staged") == "unstaged" else "staged"),
+            "stream_collide": stream_collide_form(wl, args),
             "density_ratio": float(p["rho"][0]) if len(p) else None,
             "parallelism": "replicas%d" % args.gpus,
             "l2": "no flush: each step reads one distribution buffer and writes the other, %.2f GB "

@@ -97,8 +97,10 @@ extern "C" {
  * instead of the default staged kernel (persistent blocks, row tiles copied
  * into shared memory by bulk asynchronous copies two tiles ahead).
  * Bit-identical results; for comparisons.  FP32 storage, and lattices of
- * fewer than about 1.8 million nodes, always take the one-block-per-tile
- * kernel, which is the faster of the two there. */
+ * fewer than six row tiles (256 nodes of a row, or what is left of it) per
+ * resident block of the staged kernel, always take the one-block-per-tile
+ * kernel: on a GB300 that is fewer than 7,296 tiles, 1.8 million nodes where
+ * rows are whole tiles. */
 #define LBM_FLAG_SC_UNSTAGED 32u
 /* Tests only (BF16 or FP16 storage): the staged stream-collide kernel
  * announces one byte more than its copies bring, so its bounded waits run
@@ -242,7 +244,9 @@ int lbm_get_counters(lbm_handle *h, int64_t *out8);
  * brackets every kernel with CUDA events on the handle's stream.
  * lbm_kernel_times synchronises and returns, per kernel kind, the summed
  * milliseconds and launch counts since the last reset (arrays of nk entries
- * in the order of lbm_kernel_name), then resets them. */
+ * in the order of lbm_kernel_name), then resets them.  The kinds
+ * "owner_raster" and "node_flags" belong to earlier forms of the step and stay
+ * zero. */
 int lbm_kernel_timing(lbm_handle *h, int32_t enable);
 int lbm_kernel_times(lbm_handle *h, double *ms, int64_t *launches, int32_t nk);
 int32_t lbm_kernel_count(void);
@@ -260,20 +264,24 @@ int lbm_binary_version(int32_t *version);
  * allocate device memory where they compute particle forces (their device
  * memory belongs to an allocator or pool they cannot extend, or they run in a
  * section where cudaMalloc is not allowed), so they cannot provide the
- * workspace of lbm_init.  It performs the link gather into the fixed index
- * array, the curved bounce-back and the momentum-exchange reduction of one
- * step (the same arithmetic as lbm_step's link kernel) for caller-owned
- * device buffers, and allocates nothing: its index array is a static device
- * array of the library, holding at most 2,097,152 slots (12N - 12 per
- * particle, N = ceil(2r) + 3) and 32,768 particles, 16 MiB + 128 KiB held on
- * every GPU that loads the library until the process exits.
+ * workspace of lbm_init.  It performs the link gather, the curved
+ * bounce-back and the momentum-exchange reduction of one step (the same
+ * arithmetic as lbm_step's link kernel) for caller-owned device buffers, and
+ * allocates nothing: its scratch is a static device array of the library, 16
+ * MiB + 128 KiB held on every GPU that loads the library until the process
+ * exits.  For r_max above 28.5 it holds the fixed index array, up to that the
+ * particles' records (links are then found in row masks and kept on chip);
+ * either way at most 2,097,152 slots (12N - 12 per particle, N = ceil(2 r_max)
+ * + 3) and 32,768 particles are taken.
  *   d_dist        14 FP32 planes in the layout of lbm_get_state (pitch,
  *                 plane_stride in elements), post-collision; its entries at
  *                 solid nodes are overwritten with the bounce-back values.
  *   d_owner       int32 [ny][nx]: particle id per node, -1 for fluid.
  *   d_particles   n particles (device); every radius must be <= r_max, and
  *                 the shapes follow lbm_init's rule (b >= 0; for an ellipse
- *                 1 <= b <= r and |theta| <= 1.6e6).
+ *                 1 <= b <= r and |theta| <= 1.6e6).  A centre that is not
+ *                 finite or lies outside the lattice by more than its zone
+ *                 has no links.
  *   d_forces      output, 3 doubles per particle (Fx, Fy, Tz); NaN for every
  *                 particle when one of them breaks the radius or shape rule
  *                 (checked on the device), NaN for a particle one of whose

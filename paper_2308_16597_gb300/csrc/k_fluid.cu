@@ -321,12 +321,6 @@ constexpr int kSCThreads = 128;
 template <typename T, int V>
 struct Vec;
 template <>
-struct Vec<float, 1> {
-    using W = float;
-    __device__ static void unpack(W w, float *v) { v[0] = w; }
-    __device__ static W pack(const float *v) { return v[0]; }
-};
-template <>
 struct Vec<float, 2> {
     using W = float2;
     __device__ static void unpack(W w, float *v) { v[0] = w.x; v[1] = w.y; }

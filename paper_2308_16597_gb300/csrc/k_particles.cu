@@ -31,14 +31,6 @@ __device__ __forceinline__ bool inside(const Dev &D, int i, int j)
     return i >= 0 && i < D.nx && j >= 0 && j < D.ny;
 }
 
-template <typename T>
-__device__ __forceinline__ T warp_sum(T v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
 } // namespace
 
 // The link kernel's window for zones of side N: the zone plus the two-node
@@ -327,8 +319,9 @@ __device__ __forceinline__ void links_body(const Dev &D, T *A, const int *__rest
                 t1 = 64 - __clzll((long long)m); // after its end
                 lo = fluid(t0);
                 hi = fluid(t1);
-                // two runs (only in an owner map that no raster made): a link
-                // inside would be the line's second
+                // two runs: a particle of higher index owns the nodes between
+                // (none of them is fluid), or the owner map is a restored
+                // image's; a link inside would be the line's second
                 unsigned long long st = m & ~(m << 1), en = m & ~(m >> 1);
                 st &= st - 1ull;
                 en &= ~(1ull << (t1 - 1));
@@ -515,7 +508,7 @@ __device__ __forceinline__ double repulsion(double gap, double s, double eps, do
 // disks 19.2 / 15.8 (with kPB = 4 there 16.9, 16: 22, 32: 29).
 constexpr int kPartTile = 512;
 constexpr int kPartMax = 8;
-constexpr int part_ctas(int pb) { return 32 / pb > 16 ? 16 : 32 / pb; } // 64 registers a thread
+constexpr int part_ctas(int pb) { return 32 / pb > 16 ? 16 : 32 / pb; } // 64 registers a thread (pb = 1: 128)
 
 // Support distance of particle p along the unit vector (nx, ny): its radius
 // for a disk.

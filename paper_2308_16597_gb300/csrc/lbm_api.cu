@@ -399,9 +399,10 @@ void fill_dev(lbm_handle *h)
     D.near = reinterpret_cast<unsigned *>(ws + L.near);
     D.dsum = reinterpret_cast<DirectSums *>(ws + L.dsum);
     D.direct = (P.flags & LBM_FLAG_DIRECT_LINKS) ? 1 : 0;
-    // the staged stream-collide pays with 16-bit storage only (BF16 at
-    // 4000^2: 166.9 against 180.4 us; FP32: 292 or more against 272 us), and
-    // on large lattices (stream_collide_staged)
+    // the staged stream-collide pays with 16-bit storage only (step of a
+    // 4000^2 BF16 lattice without particles 144 against 172 us; FP32 through an
+    // earlier form of it was no faster, its step slower), and on lattices of
+    // many row tiles (stream_collide_staged)
     D.sc_staged = (P.storage != LBM_STORE_FP32 && !(P.flags & LBM_FLAG_SC_UNSTAGED)) ? 1 : 0;
     D.sc_extra_tx = (P.flags & LBM_FLAG_TEST_WAIT_TIMEOUT) ? 1 : 0;
     D.all_pairs = (P.flags & LBM_FLAG_ALL_PAIRS) ? 1 : 0;

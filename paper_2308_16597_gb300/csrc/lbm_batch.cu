@@ -141,7 +141,10 @@ cudaError_t launch_sc(const lbm_batch *b, int par, cudaStream_t st)
 
 // One step of every instance, in the order of lbm_step: links -> particles
 // (and raster) -> stream-collide beside the general path (the first and last
-// rows, and the refilling).
+// rows, and the refilling: two launches of eight blocks an instance and of a
+// block per 128 particles.  One launch for both, with a thread per node of the
+// rows and per particle, measured less: 64 cavities 577.4 / 565.2 us a step
+// FP32 and 415.5 / 405.4 BF16, 16 of them 138.3 / 128.4 and 114.6 / 107.2.)
 int enqueue_batch_step(lbm_batch *b, int par, cudaStream_t st)
 {
     const InstArgs *I = b->d_inst;

@@ -262,21 +262,6 @@ __device__ __forceinline__ bool in_disk(int i, int j, double xc, double yc, doub
     return __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)) <= __dmul_rn(r, r);
 }
 
-// Wall fraction q (Sec. 2.3) of the link (i,j) -> (i,j) + e_k on the circle
-// (xc, yc, r): t = (|d|^2 - r^2) / (-(d.e) + sqrt((d.e)^2 - |e|^2 (|d|^2 - r^2))).
-__device__ __forceinline__ double link_q(int i, int j, int k, double xc, double yc, double r)
-{
-    double dx = __dsub_rn((double)i, xc);
-    double dy = __dsub_rn((double)j, yc);
-    double de = __dadd_rn(__dmul_rn((double)ex(k), dx), __dmul_rn((double)ey(k), dy));
-    double a = (double)(ex(k) * ex(k) + ey(k) * ey(k));
-    double c = __dsub_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(r, r));
-    double disc = __dsub_rn(__dmul_rn(de, de), __dmul_rn(a, c));
-    if (disc < 0.0) disc = 0.0;
-    double t = __ddiv_rn(c, __dadd_rn(-de, __dsqrt_rn(disc)));
-    return t > 1.0 ? 1.0 : t;
-}
-
 // ---------------------------------------------------------------------------
 // Elliptical particles (Sec. 2.6, Appendix A): semi-axes a = r along the body
 // axis at angle theta and b; 0 < b != r.  Every operation below is a
@@ -463,15 +448,6 @@ __device__ __forceinline__ void two_prod(float a, float b, float &p, float &e)
     p = a * b;
     e = fmaf(a, b, -p);
 }
-// (h, l) += (h2, l2)
-__device__ __forceinline__ void df_add(float &h, float &l, float h2, float l2)
-{
-    float s, e;
-    two_sum(h, h2, s, e);
-    h = s;
-    l = l + l2 + e;
-}
-
 // A disk with its centre split as x = xh + xl, y = yh + yl and r^2 = r2h + r2l
 // (built once per disk in FP64).
 struct DiskDF {
@@ -683,13 +659,6 @@ struct DirectSums {
     double f[3];  // Fx, Fy, Tz brackets
     int c[6];     // ax_x, ax_y, ax_t, dg_x, dg_y, dg_t
 };
-// Per-link momentum-exchange sums.  Each thread adds its links (add), then
-// finish() sums a warp's threads; the sums are exact, so every kernel that
-// sums links gets the same bits however it distributes them.  bx, by, tq:
-// the variable part of Eq. force / Eq. torque of a link; k its direction;
-// lvl its Bouzidi fallback level; half whether its thermal rule fell back to
-// half-way; tz the torque moment i e_k,y - j e_k,x of its constant part.
-
 // Sum over the warp, modulo 2^64, on every lane: three limbs of 22, 22 and 20
 // bits, each summed by one warp reduction (sums below 2^27), instead of five
 // rounds of two shuffles and a 64-bit addition.
@@ -702,6 +671,12 @@ __device__ __forceinline__ long long warp_sum64(long long v)
     return (long long)((unsigned long long)l0 + ((unsigned long long)l1 << 22) + ((unsigned long long)(long long)l2 << 44));
 }
 
+// Per-link momentum-exchange sums.  Each thread adds its links (add), then
+// finish() sums a warp's threads; the sums are exact, so every kernel that
+// sums links gets the same bits however it distributes them.  bx, by, tq:
+// the variable part of Eq. force / Eq. torque of a link; k its direction;
+// lvl its Bouzidi fallback level; half whether its thermal rule fell back to
+// half-way; tz the torque moment i e_k,y - j e_k,x of its constant part.
 struct LinkAcc {
     long long fx = 0, fy = 0, tq = 0;
     int axx = 0, axy = 0, axt = 0, dgx = 0, dgy = 0, dgt = 0, cl = 0, cs = 0, ct = 0;
@@ -839,27 +814,6 @@ __host__ __device__ inline bool zone_point(int k, int N, int line, int t, int &a
     return b >= 0 && b < N;
 }
 
-// Walk of line `line` of direction k in zone coordinates (a = column,
-// b = row): the valid points are (a0 + t da, b0 + t db), t = 0 .. cnt - 1 (the
-// same points as zone_point, in the same order, without per-point tests).
-__host__ __device__ inline void line_walk(int k, int N, int line, int &a0, int &b0, int &da, int &db,
-                                          int &cnt)
-{
-    if (k == 1 || k == 3) {
-        a0 = 0; b0 = line; da = 1; db = 0; cnt = N;
-    } else if (k == 2 || k == 4) {
-        a0 = line; b0 = 0; da = 0; db = 1; cnt = N;
-    } else if (k == 5 || k == 7) {
-        const int m = line - (N - 2); // b = a - m
-        const int t0 = m > 0 ? m : 0, t1 = (N - 1 + m) < (N - 1) ? (N - 1 + m) : (N - 1);
-        a0 = t0; b0 = t0 - m; da = 1; db = 1; cnt = t1 - t0 + 1;
-    } else {
-        const int sm = line + 1; // b = sm - a
-        const int t0 = (sm - N + 1) > 0 ? (sm - N + 1) : 0, t1 = sm < (N - 1) ? sm : (N - 1);
-        a0 = t0; b0 = sm - t0; da = 1; db = -1; cnt = t1 - t0 + 1;
-    }
-}
-
 // Slot s of a zone of size N -> direction k and line.
 __host__ __device__ inline void slot_dir_line(int s, int N, int &k, int &line)
 {
@@ -965,6 +919,7 @@ __device__ __forceinline__ void sc_tile(const ScInst *__restrict__ e, int g, int
 // ---------------------------------------------------------------------------
 // Kernel launchers (defined in k_fluid.cu and k_particles.cu).
 // ---------------------------------------------------------------------------
+// (kKRaster and kKFlags: kernels of earlier forms of the step, whose times stay zero)
 enum KernelKind { kKLinks = 0, kKParticles, kKRaster, kKFlags, kKStreamCollide,
                   kKBoundary, kKInit, kKFields, kKNearMask, kKStreamCollideNear, kNumKernelKinds };
 
