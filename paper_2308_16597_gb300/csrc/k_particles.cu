@@ -102,7 +102,8 @@ __device__ __forceinline__ void clear_zone_bits(const Dev &D, int parity, int p,
     for (int r = lane; r < N; r += 32) {
         const int j = Y0 + r;
         if (j < 0 || j >= D.ny) continue;
-        for (int w = w0; w <= w1; ++w) bits_put(D, bit_word(D, 32 * w, j, parity ^ 1), 0u);
+        const BitsRow row = bits_row(D, j, parity ^ 1);
+        for (int w = w0; w <= w1; ++w) bits_put(D, row, w, 0u);
     }
 }
 // (Whole block of nthreads threads.)
@@ -136,8 +137,9 @@ __device__ __forceinline__ int2 run_at(const Dev &D, int parity, int p, int r)
 __device__ __forceinline__ unsigned long long fluid_row(const Dev &D, int parity, int XA, int j, bool wide)
 {
     if (j < 0 || j >= D.ny) return 0ull;
+    const BitsRow row = bits_row(D, j, parity);
     const int w0 = XA >> 5, sh = XA & 31; // XA may be negative: words before the row are not fluid
-    auto word = [&](int w) -> unsigned { return w >= 0 && w < D.bpitch ? ~bits_get(D, bit_word(D, 32 * w, j, parity)) : 0u; };
+    auto word = [&](int w) -> unsigned { return w >= 0 && w < D.bpitch ? ~bits_get(D, row, w) : 0u; };
     const unsigned a = word(w0), b = word(w0 + 1), c = wide ? word(w0 + 2) : 0u;
     unsigned long long m = ((unsigned long long)__funnelshift_r(b, c, sh) << 32) | __funnelshift_r(a, b, sh);
     const int in = D.nx - XA; // columns inside the domain
@@ -704,9 +706,10 @@ __device__ __forceinline__ void raster_one(const Dev &D, int par, int *own, cons
             if (in_bounds(D, (long long)p * D.zone_max + b0 + lane, (long long)D.np * D.zone_max))
                 runs[b0 + lane] = make_int2(lo, hi);
             if (bits && lo <= hi) {
+                const BitsRow row = bits_row(D, j, par);
                 for (int w = lo >> 5; w <= hi >> 5; ++w) {
                     const int c0 = max(lo - 32 * w, 0), c1 = min(hi - 32 * w, 31);
-                    bits_or(D, bit_word(D, 32 * w, j, par), (~0u << c0) & (~0u >> (31 - c1)));
+                    bits_or(D, row, w, (~0u << c0) & (~0u >> (31 - c1)));
                 }
             }
             if (moved && j >= Y0_old && j < Y0_old + B.N && j >= 0 && j < D.ny) {
@@ -1175,8 +1178,8 @@ __global__ void k_flags_in(const Dev D, const uint8_t *flags, int parity)
         now |= (f == kSolid ? 1u : 0u) << b;
         before |= (f == kNewborn ? 1u : 0u) << b;
     }
-    bits_put(D, bit_word(D, 32 * w, j, parity), now);
-    bits_put(D, bit_word(D, 32 * w, j, parity ^ 1), before);
+    bits_put(D, bits_row(D, j, parity), w, now);
+    bits_put(D, bits_row(D, j, parity ^ 1), w, before);
 }
 
 // ---- batched kernels: one grid over all instances (InstArgs table, block
