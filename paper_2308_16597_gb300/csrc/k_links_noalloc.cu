@@ -10,6 +10,10 @@
 // passes the distributions, the owner map, the particles and the force
 // output; the only scratch (the index array) lives here.
 //
+// Zones of at most 60 nodes a side take the two kernels in the second half of
+// this file, which keep the links on chip and hold the particles' records in
+// that array; larger ones the three that follow.
+//
 // The array holds 2,097,152 slots (node + wall fraction, 8 bytes each) and
 // the slot offsets of up to 32,768 particles: 16 MiB + 128 KiB held on every
 // GPU that loads the library, for the life of the process.  All calls share
